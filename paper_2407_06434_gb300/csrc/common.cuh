@@ -254,6 +254,8 @@ void launch_prep(const Ws& ws, const float* A, cudaStream_t s);
 void launch_gram_simt(const Ws& ws, cudaStream_t s);
 void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s);
 void launch_c0_simt(const Ws& ws, int B, cudaStream_t s);
+cudaError_t configure_corr_simt(const Ws& ws);
+cudaError_t configure_c0_simt();
 void launch_gram_solve(const Ws& ws, const CallArgs* args, int B, int S, float eps, int eps_rel,
                        cudaStream_t s);
 cudaError_t configure_gram_solve(const Ws& ws);

@@ -2,16 +2,23 @@
 //
 // Both are the contraction C = X A^T over the padded signal length Mp with both operands stored
 // K-major (rows of Mp contiguous floats): for the correlation X holds the live residuals
-// (batched as one GEMM, Sec. 3.2 eq:bmm), for the Gram matrix X = A^T itself (Sec. 2.2).
-// A 128 x 128 output tile per 256-thread block, 8 x 8 outputs per thread, K chunks of 16 staged
-// through double-buffered shared memory.
+// (batched as one GEMM, Sec. 3.2 eq:bmm), for the Gram matrix X = A^T itself (Sec. 2.2), of which
+// only the upper triangle is computed (the lower is its mirror image, bit for bit).
+// A tile of 128 rows x 8 TN atoms per 128-thread block, 8 x TN outputs per thread, K chunks of 32
+// staged through double-buffered shared memory, transposed. Every output is one FMA chain over m
+// in order, two outputs to an FFMA2. What bounds it: 8 x 8 outputs a thread read shared memory as
+// long as they multiply (a 16-byte read takes four cycles of the SM's 128 bytes whatever it
+// broadcasts), 8 x 16 three quarters of that; the chunks come as whole 128-byte lines, since loads
+// of 64 or 32 bytes a row cost more than the products could hide (Gram matrix of 8192 atoms of
+// length 1024: 2764 us for both triangles with 8 x 8 outputs and FMAs, 1301 us for one with FFMA2,
+// 1252 us with 8 x 16 outputs, 1148 us with whole lines: 61 TFLOP/s of 80.5 nominal).
 //
 // A third form stores C = Y A^T for signals 0..B-1 (rows of R32 in signal order) into the c0
 // workspace: the exact first correlation the Gram-space solve starts from.
 //
 // The correlation never writes C: the epilogue forms the score |c| / ||a_n|| (Alg. 1), takes
 // each thread's best atom in ascending index order (strict '>', so the lowest index keeps a
-// tie), reduces across the 16 threads that share a signal with warp shuffles, and merges the
+// tie), reduces across the 8 threads that share a signal with warp shuffles, and merges the
 // tile's winner into the signal's packed (score, ~index) key with one 64-bit atomicMax: the
 // maximum key is the highest score and, among equal scores, the lowest index, whatever order
 // the tiles finish in.
@@ -20,19 +27,42 @@
 namespace ompk {
 
 namespace {
-constexpr int BM = 128, BN = 128, BK = 16, PAD = 4;
-
 constexpr int kCorrelate = 0, kGram = 1, kStoreC = 2;
 
-// MODE kCorrelate: k is the iteration; kGram: k unused; kStoreC: k is the number of signals
-template <int MODE>
-__global__ void __launch_bounds__(256, 2) simt_tile_kernel(Ws ws, int k) {
+// Two FP32 FMAs in one instruction (each rounded as fmaf): d.lo += x.lo a.lo, d.hi += x.hi a.hi
+__device__ __forceinline__ void ffma2(unsigned long long& d, unsigned long long x, unsigned long long a) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(x), "l"(a));
+}
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float(static_cast<uint32_t>(v)); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float(static_cast<uint32_t>(v >> 32)); }
+
+__device__ __forceinline__ unsigned long long dup2(float x) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+
+constexpr int BM = 128, BK = 32;
+constexpr int TX = 8, THREADS = 128;  // threads along the atoms; 16 along the rows, 8 rows each
+
+// MODE kCorrelate: k is the iteration; kGram: k unused; kStoreC: k is the number of signals.
+// TN atoms per thread: a tile of 128 rows x 8 TN atoms.
+template <int MODE, int TN>
+__global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
   constexpr bool GRAM = MODE == kGram;
-  __shared__ __align__(16) float Xs[2][BK][BM + PAD];
-  __shared__ __align__(16) float As[2][BK][BN + PAD];
+  constexpr int BN = TX * TN;
+  constexpr int RS = THREADS / (BK / 4);             // rows apart of a thread's loads (16)
+  constexpr int LX = BM / RS / 2, LA = BN / RS / 2;  // loads per thread and half chunk
+  extern __shared__ __align__(16) float smem_f[];
+  float* Xs = smem_f;                // 2 x BK x BM
+  float* As = smem_f + 2 * BK * BM;  // 2 x BK x BN
   const int tid = threadIdx.x;
-  const int n0 = blockIdx.x * BN;
-  const int p0 = blockIdx.y * BM;
+  int bx = blockIdx.x, by = blockIdx.y;
+  // G is symmetric and every entry's products and sums are the same in both orders, so only tiles
+  // that reach the diagonal or lie above it are computed, and each stores its mirror image too
+  if (GRAM && bx * BN + BN <= by * BM) return;
+  const int n0 = bx * BN;
+  const int p0 = by * BM;
   int L;
   const int* live = nullptr;
   if (GRAM) {
@@ -46,108 +76,147 @@ __global__ void __launch_bounds__(256, 2) simt_tile_kernel(Ws ws, int k) {
   }
   if (p0 >= L) return;
 
-  const int lrow = tid >> 2, lk = (tid & 3) * 4;
-  const float* xsrc[2];
-  const float* asrc[2];
-  bool xv[2], av[2];
+  // a warp loads 4 rows x 128 bytes (whole lines); element (k, r) of a chunk is stored at column
+  // r ^ 4 ((k / 4) % 8) of its row k, so that the transposed stores of a warp meet every bank once
+  // and four consecutive rows stay one aligned float4
+  const int lrow = tid >> 3, lq = tid & 7;
+  const float* xsrc[2 * LX];
+  const float* asrc[2 * LA];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int p = p0 + lrow + 64 * i;
-    xv[i] = p < L;
-    const int row = xv[i] ? ((GRAM || MODE == kStoreC) ? p : live[p]) : 0;
-    xsrc[i] = (GRAM ? ws.A32 : ws.R32) + static_cast<size_t>(row) * ws.Mp + lk;
-    const int n = n0 + lrow + 64 * i;
-    av[i] = n < ws.N;
-    asrc[i] = ws.A32 + static_cast<size_t>(av[i] ? n : 0) * ws.Mp + lk;
+  for (int i = 0; i < 2 * LX; ++i) {
+    const int p = p0 + lrow + RS * i;
+    const int row = p < L ? ((GRAM || MODE == kStoreC) ? p : live[p]) : -1;
+    xsrc[i] = row < 0 ? nullptr : (GRAM ? ws.A32 : ws.R32) + static_cast<size_t>(row) * ws.Mp + 4 * lq;
   }
-  float4 xr[2], ar[2];
+#pragma unroll
+  for (int i = 0; i < 2 * LA; ++i) {
+    const int n = n0 + lrow + RS * i;
+    asrc[i] = n < ws.N ? ws.A32 + static_cast<size_t>(n) * ws.Mp + 4 * lq : nullptr;
+  }
+  float4 xr[LX], ar[LA];
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto gload = [&](int kc) {
+  auto gload = [&](int kc, int h) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      xr[i] = xv[i] ? __ldg(reinterpret_cast<const float4*>(xsrc[i] + kc)) : zero;
-      ar[i] = av[i] ? __ldg(reinterpret_cast<const float4*>(asrc[i] + kc)) : zero;
-    }
+    for (int i = 0; i < LX; ++i)
+      xr[i] = xsrc[h * LX + i] ? __ldg(reinterpret_cast<const float4*>(xsrc[h * LX + i] + kc)) : zero;
+#pragma unroll
+    for (int i = 0; i < LA; ++i)
+      ar[i] = asrc[h * LA + i] ? __ldg(reinterpret_cast<const float4*>(asrc[h * LA + i] + kc)) : zero;
   };
-  auto sstore = [&](int buf) {
+  auto sstore = [&](int buf, int h) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int r = lrow + 64 * i;
-      Xs[buf][lk + 0][r] = xr[i].x;
-      Xs[buf][lk + 1][r] = xr[i].y;
-      Xs[buf][lk + 2][r] = xr[i].z;
-      Xs[buf][lk + 3][r] = xr[i].w;
-      As[buf][lk + 0][r] = ar[i].x;
-      As[buf][lk + 1][r] = ar[i].y;
-      As[buf][lk + 2][r] = ar[i].z;
-      As[buf][lk + 3][r] = ar[i].w;
+    for (int i = 0; i < LX; ++i) {
+      float* d = Xs + (buf * BK + 4 * lq) * BM + ((lrow + RS * (h * LX + i)) ^ (4 * lq));
+      d[0] = xr[i].x;
+      d[BM] = xr[i].y;
+      d[2 * BM] = xr[i].z;
+      d[3 * BM] = xr[i].w;
+    }
+#pragma unroll
+    for (int i = 0; i < LA; ++i) {
+      float* d = As + (buf * BK + 4 * lq) * BN + ((lrow + RS * (h * LA + i)) ^ (4 * lq));
+      d[0] = ar[i].x;
+      d[BN] = ar[i].y;
+      d[2 * BN] = ar[i].z;
+      d[3 * BN] = ar[i].w;
     }
   };
 
-  float acc[8][8];
+  // acc2[i][j2]: outputs (row i, atoms 2 j2 and 2 j2 + 1); every output is one chain of FMAs over
+  // m = 0, 1, ..., Mp - 1
+  unsigned long long acc2[8][TN / 2];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < TN / 2; ++j) acc2[i][j] = 0ull;
 
-  const int tx = tid & 15, ty = tid >> 4;
+  const int tx = tid % TX, ty = tid / TX;
   const int nk = ws.Mp / BK;
-  gload(0);
-  sstore(0);
+  // the fragments of step kk + 1 are read while the products of step kk run
+  float4 xf[2][2];
+  ulonglong2 af[2][TN / 4];
+  auto frag = [&](int f, int buf, int kk) {
+    const int w = 4 * (kk >> 2);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      xf[f][h] = *reinterpret_cast<const float4*>(Xs + (buf * BK + kk) * BM + h * (BM / 2) + ((ty * 4) ^ w));
+#pragma unroll
+    for (int h = 0; h < TN / 4; ++h)
+      af[f][h] = *reinterpret_cast<const ulonglong2*>(As + (buf * BK + kk) * BN + h * (4 * TX) + ((tx * 4) ^ w));
+  };
+  gload(0, 0);
+  sstore(0, 0);
+  gload(0, 1);
+  sstore(0, 1);
   __syncthreads();
   for (int kt = 0; kt < nk; ++kt) {
     const int buf = kt & 1;
-    if (kt + 1 < nk) gload((kt + 1) * BK);
+    const bool more = kt + 1 < nk;
+    if (more) gload((kt + 1) * BK, 0);
+    frag(0, buf, 0);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 x0 = *reinterpret_cast<const float4*>(&Xs[buf][kk][ty * 4]);
-      const float4 x1 = *reinterpret_cast<const float4*>(&Xs[buf][kk][64 + ty * 4]);
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][tx * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + tx * 4]);
-      const float xf[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-      const float af[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const int f = kk & 1;
+      if (kk == BK / 2 && more) {  // the next chunk comes in halves, half the registers in flight
+        sstore(buf ^ 1, 0);
+        gload((kt + 1) * BK, 1);
+      }
+      if (kk + 1 < BK) frag(f ^ 1, buf, kk + 1);
+      const float xs[8] = {xf[f][0].x, xf[f][0].y, xf[f][0].z, xf[f][0].w,
+                           xf[f][1].x, xf[f][1].y, xf[f][1].z, xf[f][1].w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long xx = dup2(xs[i]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xf[i], af[j], acc[i][j]);
+        for (int h = 0; h < TN / 4; ++h) {
+          ffma2(acc2[i][2 * h], xx, af[f][h].x);
+          ffma2(acc2[i][2 * h + 1], xx, af[f][h].y);
+        }
+      }
     }
-    if (kt + 1 < nk) sstore(buf ^ 1);
+    if (more) sstore(buf ^ 1, 1);
     __syncthreads();
   }
+  auto acc = [&](int i, int j) { return (j & 1) ? hi2(acc2[i][j >> 1]) : lo2(acc2[i][j >> 1]); };
 
-  // atoms of this thread, ascending: n0 + tx*4 + {0..3}, then n0 + 64 + tx*4 + {0..3}
-  int ncol[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) ncol[j] = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
+  // atoms of this thread, ascending: n0 + 32 h + 4 tx + {0..3}; rows p0 + 64 h + 4 ty + {0..3}
+  auto ncol = [&](int j) { return n0 + (j >> 2) * (4 * TX) + tx * 4 + (j & 3); };
+  auto prows = [&](int i) { return p0 + (i >> 2) * (BM / 2) + ty * 4 + (i & 3); };
 
-  if (GRAM) {
+  if (GRAM || MODE == kStoreC) {
+    // C row-major with N columns (rows < L), 16 bytes at a time where the rows stay aligned; the
+    // Gram form stores the mirror image G[n][p] as well
+    float* C = GRAM ? ws.gram : ws.c0;
+    const bool vec = (ws.N & 3) == 0;
+    auto store4 = [&](int row, int col, float a, float b, float c, float d) {
+      float* g = C + static_cast<size_t>(row) * ws.N + col;
+      if (vec && col + 3 < ws.N) {
+        *reinterpret_cast<float4*>(g) = make_float4(a, b, c, d);
+      } else {
+        if (col < ws.N) g[0] = a;
+        if (col + 1 < ws.N) g[1] = b;
+        if (col + 2 < ws.N) g[2] = c;
+        if (col + 3 < ws.N) g[3] = d;
+      }
+    };
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int row = p0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-      if (row >= ws.N) continue;
-      float* g = ws.gram + static_cast<size_t>(row) * ws.N;
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (ncol[j] < ws.N) g[ncol[j]] = acc[i][j];
+      for (int j = 0; j < TN; j += 4)
+        if (prows(i) < L) store4(prows(i), ncol(j), acc(i, j), acc(i, j + 1), acc(i, j + 2), acc(i, j + 3));
+    if (GRAM) {
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+#pragma unroll
+        for (int i = 0; i < 8; i += 4)
+          if (ncol(j) < ws.N) store4(ncol(j), prows(i), acc(i, j), acc(i + 1, j), acc(i + 2, j), acc(i + 3, j));
     }
     return;
   }
-  if (MODE == kStoreC) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int row = p0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-      if (row >= L) continue;
-      float* c = ws.c0 + static_cast<size_t>(row) * ws.N;
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (ncol[j] < ws.N) c[ncol[j]] = acc[i][j];
-    }
-    return;
-  }
 
-  float inv[8];
+  float inv[TN];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) inv[j] = ncol[j] < ws.N ? __ldg(ws.inv_norm + ncol[j]) : 0.f;
+  for (int j = 0; j < TN; ++j) inv[j] = ncol(j) < ws.N ? __ldg(ws.inv_norm + ncol(j)) : 0.f;
   if (ws.cand2) {
     // Margins recorded: each row's best two atoms of the tile (same scan and ties), then
     // cand1 keeps the global best as before and cand2 receives every key that loses a merge
@@ -155,26 +224,26 @@ __global__ void __launch_bounds__(256, 2) simt_tile_kernel(Ws ws, int k) {
     // so that it ends with the largest key other than the best: the runner-up.
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int prow = p0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+      const int prow = prows(i);
       float b1 = -1.f, b2 = -1.f;
       int i1 = 0x7fffffff, i2 = 0x7fffffff;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (ncol[j] < ws.N) {
-          const float sc = fabsf(acc[i][j]) * inv[j];
-          if (better(sc, ncol[j], b1, i1)) {
+      for (int j = 0; j < TN; ++j) {
+        if (ncol(j) < ws.N) {
+          const float sc = fabsf(acc(i, j)) * inv[j];
+          if (better(sc, ncol(j), b1, i1)) {
             b2 = b1;
             i2 = i1;
             b1 = sc;
-            i1 = ncol[j];
-          } else if (better(sc, ncol[j], b2, i2)) {
+            i1 = ncol(j);
+          } else if (better(sc, ncol(j), b2, i2)) {
             b2 = sc;
-            i2 = ncol[j];
+            i2 = ncol(j);
           }
         }
       }
 #pragma unroll
-      for (int o = 1; o < 16; o <<= 1) {
+      for (int o = 1; o < TX; o <<= 1) {
         const float o1 = __shfl_xor_sync(0xffffffffu, b1, o);
         const int oi1 = __shfl_xor_sync(0xffffffffu, i1, o);
         const float o2 = __shfl_xor_sync(0xffffffffu, b2, o);
@@ -204,21 +273,21 @@ __global__ void __launch_bounds__(256, 2) simt_tile_kernel(Ws ws, int k) {
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const int prow = p0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+    const int prow = prows(i);
     float best = -1.f;
     int bidx = 0x7fffffff;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (ncol[j] < ws.N) {
-        const float s = fabsf(acc[i][j]) * inv[j];
+    for (int j = 0; j < TN; ++j) {
+      if (ncol(j) < ws.N) {
+        const float s = fabsf(acc(i, j)) * inv[j];
         if (s > best) {
           best = s;
-          bidx = ncol[j];
+          bidx = ncol(j);
         }
       }
     }
 #pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
+    for (int o = 1; o < TX; o <<= 1) {
       const float ob = __shfl_xor_sync(0xffffffffu, best, o);
       const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
       if (better(ob, oi, best, bidx)) {
@@ -229,21 +298,72 @@ __global__ void __launch_bounds__(256, 2) simt_tile_kernel(Ws ws, int k) {
     if (tx == 0 && prow < L && bidx < ws.N) atomicMax(ws.cand1 + prow, pack_key(best, bidx));
   }
 }
+
+template <int TN>
+constexpr size_t tile_bytes() {
+  return 2 * BK * (BM + TX * TN) * sizeof(float);
+}
+
+template <int MODE, int TN>
+void launch_one(const Ws& ws, int rows, int k, cudaStream_t s) {
+  const dim3 grid((ws.N + TX * TN - 1) / (TX * TN), (rows + BM - 1) / BM);
+  simt_tile_kernel<MODE, TN><<<grid, THREADS, tile_bytes<TN>(), s>>>(ws, k);
+}
+
+// Output tiles of 128 rows x 128, 96 or 64 atoms: the width whose rounds over the SMs (a lone
+// round counts 1.25, one block's four warps leave an SM's latencies exposed) times its area are
+// least, the widest on a tie (it reads the least from shared memory per product). Measured, us at
+// widths 128 / 96 / 64: correlation of 1000 signals x 8192 atoms x 1024 365 / 322 / 309; first
+// correlation of 1200 x 1207 x 8064 1015 / 644 / 752; Gram matrix of 2048 atoms of length 512
+// 99 / 70 / 50, of 8192 of length 1024 1148 / 1180 / 1192.
+template <int MODE>
+void launch_tiles(const Ws& ws, int rows, int k, cudaStream_t s) {
+  constexpr int kSms = 152;
+  int best = 16;
+  double least = 0.0;
+  for (int tn = 16; tn >= 8; tn -= 4) {
+    const int cols = (ws.N + TX * tn - 1) / (TX * tn), rts = (rows + BM - 1) / BM;
+    long long tiles = static_cast<long long>(cols) * rts;
+    if (MODE == kGram) {  // the tiles that simt_tile_kernel does not skip
+      tiles = 0;
+      for (int by = 0; by < rts; ++by) tiles += cols - (by * BM) / (TX * tn);
+    }
+    const double rounds = tiles <= kSms ? 1.25 : static_cast<double>((tiles + kSms - 1) / kSms);
+    if (least == 0.0 || rounds * tn < least) {
+      least = rounds * tn;
+      best = tn;
+    }
+  }
+  if (best == 16)
+    launch_one<MODE, 16>(ws, rows, k, s);
+  else if (best == 12)
+    launch_one<MODE, 12>(ws, rows, k, s);
+  else
+    launch_one<MODE, 8>(ws, rows, k, s);
+}
+
+template <int MODE>
+cudaError_t set_tile_limits() {
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(simt_tile_kernel<MODE, 16>), tile_bytes<16>());
+  if (e == cudaSuccess)
+    e = raise_smem_limit(reinterpret_cast<const void*>(simt_tile_kernel<MODE, 12>), tile_bytes<12>());
+  if (e == cudaSuccess)
+    e = raise_smem_limit(reinterpret_cast<const void*>(simt_tile_kernel<MODE, 8>), tile_bytes<8>());
+  return e;
+}
 }  // namespace
 
-void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s) {
-  dim3 grid((ws.N + BN - 1) / BN, (B + BM - 1) / BM);
-  simt_tile_kernel<kCorrelate><<<grid, 256, 0, s>>>(ws, k);
+cudaError_t configure_corr_simt(const Ws& ws) {
+  cudaError_t e = set_tile_limits<kGram>();
+  if (e == cudaSuccess && ws.prec == OMP_PREC_FP32) e = set_tile_limits<kCorrelate>();
+  return e;
 }
+cudaError_t configure_c0_simt() { return set_tile_limits<kStoreC>(); }
 
-void launch_c0_simt(const Ws& ws, int B, cudaStream_t s) {
-  dim3 grid((ws.N + BN - 1) / BN, (B + BM - 1) / BM);
-  simt_tile_kernel<kStoreC><<<grid, 256, 0, s>>>(ws, B);
-}
+void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s) { launch_tiles<kCorrelate>(ws, B, k, s); }
 
-void launch_gram_simt(const Ws& ws, cudaStream_t s) {
-  dim3 grid((ws.N + BN - 1) / BN, (ws.N + BM - 1) / BM);
-  simt_tile_kernel<kGram><<<grid, 256, 0, s>>>(ws, 0);
-}
+void launch_c0_simt(const Ws& ws, int B, cudaStream_t s) { launch_tiles<kStoreC>(ws, B, B, s); }
+
+void launch_gram_simt(const Ws& ws, cudaStream_t s) { launch_tiles<kGram>(ws, ws.N, 0, s); }
 
 }  // namespace ompk

@@ -447,7 +447,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
                  (!ws.win_pos || cudaMemset(ws.win_pos, 0, Bp * sizeof(float)) == cudaSuccess) &&
                  cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
                  cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking) == cudaSuccess &&
-                 configure_update_kernels(ws) == cudaSuccess;
+                 configure_update_kernels(ws) == cudaSuccess && configure_corr_simt(ws) == cudaSuccess;
   if (cuda_ok && d.precision != OMP_PREC_FP32) cuda_ok = tc_setup(ws, h->sm_count, &h->tc) == cudaSuccess;
   if (cuda_ok) cuda_ok = cudaDeviceSynchronize() == cudaSuccess;
   if (!cuda_ok) {
@@ -537,6 +537,7 @@ omp_status omp_solve_batch_gram(omp_handle h, const float* A, const float* Y, in
       cudaGetLastError();
       return OMP_ERR_INVALID_ARGUMENT;
     }
+    if (configure_c0_simt() != cudaSuccess) return OMP_ERR_CUDA;
     if (!dalloc(h, &h->ws.c0, static_cast<size_t>(h->ws.Bmax) * h->ws.N)) return OMP_ERR_OUT_OF_MEMORY;
   }
   if (A != h->prepared_A) {

@@ -1,0 +1,69 @@
+"""The FP32 tile kernels at the edges of their tiles, against FP64 on the same FP32 inputs.
+
+A chain of M FMAs is within M 2^-24 ||a|| ||r|| of the exact product; the norm's reciprocal and the
+product with it add three roundings, so a score is within (M + 4) 2^-24 ||r|| of the exact one and
+the picked atom's exact score within twice that of the best."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2407_06434_gb300 import build
+    build.build()
+    from paper_2407_06434_gb300 import omp
+    omp.load()
+    return omp
+
+
+def _problem(M, N, B, seed):
+    rng = np.random.default_rng(seed)
+    At = rng.standard_normal((N, M)).astype(np.float32) * rng.uniform(0.5, 2.0, (N, 1)).astype(np.float32)
+    R = rng.standard_normal((B, M)).astype(np.float32)
+    return At, R
+
+
+# the last four take tiles 96, 64 and 128 atoms wide with ragged rows and columns
+@pytest.mark.parametrize("M,N,B", [(1, 2, 1), (63, 64, 127), (64, 65, 128), (65, 97, 129),
+                                   (100, 1207, 1200), (130, 8193, 1001), (40, 4097, 4999), (96, 129, 3)])
+def test_fp32_correlation_tiles(lib, M, N, B):
+    At, R = _problem(M, N, B, M + N)
+    s = lib.OmpSolver(M, N, max_batch=B, max_iters=1, precision="fp32")
+    idx = torch.empty((B, 1), dtype=torch.int32, device="cuda")
+    sc = torch.empty((B, 1), device="cuda")
+    lib.omp_correlate_topk(s.h, torch.from_numpy(At).cuda().t(), torch.from_numpy(R).cuda(), 1, idx, sc)
+    idx, sc = idx.cpu().numpy()[:, 0], sc.cpu().numpy()[:, 0].astype(np.float64)
+    A64, R64 = At.astype(np.float64), R.astype(np.float64)
+    scores = np.abs(R64 @ (A64 / np.linalg.norm(A64, axis=1, keepdims=True)).T)
+    tol = (M + 4) * 2.0 ** -24 * np.linalg.norm(R64, axis=1)
+    own = scores[np.arange(B), idx]
+    assert np.all(np.abs(sc - own) <= tol)
+    assert np.all(own >= scores.max(axis=1) - 2 * tol)
+    s.close()
+
+
+# two steps from a signal in the span of two atoms recover it only through the Gram entry between
+# them, on either side of the diagonal and in any tile
+@pytest.mark.parametrize("N", [64, 65, 127, 129, 257, 1000, 2049])
+def test_gram_entries_of_any_tile(lib, N):
+    M = 80
+    At, _ = _problem(M, N, 1, N)
+    At /= np.linalg.norm(At, axis=1, keepdims=True)
+    rng = np.random.default_rng(N)
+    pairs = np.array([rng.choice(N, 2, replace=False) for _ in range(300)])
+    Y = (3.0 * At[pairs[:, 0]] + 2.0 * At[pairs[:, 1]]).astype(np.float32)
+    s = lib.OmpSolver(M, N, max_batch=300, max_iters=2, precision="fp32")
+    X, sup = s.solve(torch.from_numpy(At).cuda().t(), torch.from_numpy(Y).cuda(), 2)
+    X, sup = X.cpu().numpy(), sup.cpu().numpy()
+    A64 = At.astype(np.float64)
+    for b in range(300):
+        ref, *_ = np.linalg.lstsq(A64[sup[b]].T, Y[b].astype(np.float64), rcond=None)
+        cond = np.linalg.cond(A64[sup[b]])
+        assert np.linalg.norm(X[b] - ref) <= 64 * 2.0 ** -24 * cond ** 2 * np.linalg.norm(ref)
+    s.close()
