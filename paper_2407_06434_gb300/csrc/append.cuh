@@ -52,6 +52,14 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
+// One float4 slot's part of a dot product. The order is spelled out so that every kernel that
+// forms such a sum rounds it alike: XF starts from the x product, else from the y product.
+template <bool XF>
+__device__ __forceinline__ float slot_dot(const float4& a, const float4& b) {
+  const float h = XF ? fmaf(a.y, b.y, __fmul_rn(a.x, b.x)) : fmaf(a.x, b.x, __fmul_rn(a.y, b.y));
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, h));
+}
+
 // 16-byte global -> shared copy (L2 only) that holds no register while in flight
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -455,8 +463,8 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
         if (s < M4) {
           const float4 x0 = n0 >= 0 ? __ldg(a0 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
           const float4 x1 = n1 >= 0 ? __ldg(a1 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-          acc0 += x0.x * r[t].x + x0.y * r[t].y + x0.z * r[t].z + x0.w * r[t].w;
-          acc1 += x1.x * r[t].x + x1.y * r[t].y + x1.z * r[t].z + x1.w * r[t].w;
+          acc0 += slot_dot<V == 1>(x0, r[t]);
+          acc1 += slot_dot<V == 1>(x1, r[t]);
         }
       }
       acc0 = warp_sum_f(acc0);
@@ -619,7 +627,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
   }
   float bp = 0.f;
 #pragma unroll
-  for (int t = 0; t < V; ++t) bp += q[t].x * r[t].x + q[t].y * r[t].y + q[t].z * r[t].z + q[t].w * r[t].w;
+  for (int t = 0; t < V; ++t) bp += slot_dot<V == 1>(q[t], r[t]);
   bp = warp_sum_f(bp);
   // per-warp partials of b and ||r||^2 (FP32 sums of FP32 products: no FP64 needed here)
   float* pf = gs.part;
@@ -637,7 +645,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     r[t].z = fmaf(-bf, q[t].z, r[t].z);
     r[t].w = fmaf(-bf, q[t].w, r[t].w);
     if (s < M4) rw[s] = r[t];
-    rr += r[t].x * r[t].x + r[t].y * r[t].y + r[t].z * r[t].z + r[t].w * r[t].w;
+    rr += slot_dot<false>(r[t], r[t]);
   }
   rr = warp_sum_f(rr);
   if (ws.tau) {
@@ -652,8 +660,8 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
       const int s = t * (W * 32) + wig * 32 + lane;
       if (s < M4) {
         const float4 u0 = x0[s], u1 = x1[s];
-        d0 += u0.x * r[t].x + u0.y * r[t].y + u0.z * r[t].z + u0.w * r[t].w;
-        d1 += u1.x * r[t].x + u1.y * r[t].y + u1.z * r[t].z + u1.w * r[t].w;
+        d0 += slot_dot<V == 1>(u0, r[t]);
+        d1 += slot_dot<V == 1>(u1, r[t]);
       }
     }
     d0 = warp_sum_f(d0);

@@ -81,6 +81,7 @@ struct Ws {
   float* escale;   // quantised paths: score scale per atom (1/||a|| or s_a/||a||), padded
   double* norm2;
   float* gram;
+  float* score;     // up to 8 signals x N: FP32 scores of a solve of few signals (small.cu)
   float* c0;        // Bmax x N FP32 first correlation of the Gram-space solve (allocated on use)
   // signal state
   float* R32;
@@ -281,6 +282,13 @@ void launch_update_w1(const Ws& ws, int V, int k, int B, int S, float eps, int e
 void launch_update_w2(const Ws& ws, int V, int k, int B, int S, float eps, int eps_rel, cudaStream_t s);
 void launch_update_w4(const Ws& ws, int V, int k, int B, int S, float eps, int eps_rel, cudaStream_t s);
 void launch_update_w8(const Ws& ws, int V, int k, int B, int S, float eps, int eps_rel, cudaStream_t s);
+
+// solves of few signals (small.cu): the form a solve takes (0: batched), and its launches
+int small_form(const Ws& ws, int B);
+int small_max_batch();
+cudaError_t configure_small(const Ws& ws);
+void launch_solo(const Ws& ws, int B, int S, float eps, int eps_rel, cudaStream_t s);
+void launch_wide(const Ws& ws, int sms, int B, int S, float eps, int eps_rel, cudaStream_t s);
 
 // learned proposal (restricted.cu, mlp.cu)
 size_t restricted_smem_per_signal(int S, int K, int Mp);

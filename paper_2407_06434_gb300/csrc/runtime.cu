@@ -140,6 +140,19 @@ void prof_mark(omp_handle_s* h, bool prof, int kind, int k, int end, cudaStream_
                            cudaEventRecordExternal);
 }
 
+// A solve of few signals (small.cu), where the sizes and options take one of those forms.
+bool enqueue_small(omp_handle_s* h, const Ws& ws, int B, int S, float eps, cudaStream_t s) {
+  const int form = small_form(ws, B);
+  if (form == 0) return false;
+  launch_init(ws, h->args_dev, B, s);
+  if (form == 1)
+    launch_solo(ws, B, S, eps, h->d.eps_relative, s);
+  else
+    for (int k = 0; k < S; ++k) launch_wide(ws, h->sm_count, B, S, eps, h->d.eps_relative, s);
+  launch_finalize(ws, h->args_dev, B, S, s);
+  return true;
+}
+
 void enqueue_solve(omp_handle_s* h, const Ws& ws, int B, int S, float eps, bool prof, cudaStream_t s) {
   launch_init(ws, h->args_dev, B, s);
   launch_compact(ws, 0, B, S, false, s);
@@ -230,7 +243,7 @@ omp_status run_solve(omp_handle_s* h, int B, int S, float eps, bool stats, cudaS
   h->prof_last_valid = prof;
   const Ws ws = solve_ws(h, stats);
   if (!h->d.use_graph) {
-    enqueue_solve(h, ws, B, S, eps, prof, stream);
+    if (prof || !enqueue_small(h, ws, B, S, eps, stream)) enqueue_solve(h, ws, B, S, eps, prof, stream);
     return check_launch();
   }
   for (auto& g : h->graphs)
@@ -257,7 +270,7 @@ omp_status run_solve(omp_handle_s* h, int B, int S, float eps, bool stats, cudaS
   } else {
     ok = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
-      enqueue_solve(h, ws, B, S, eps, false, h->cap_stream);
+      if (!enqueue_small(h, ws, B, S, eps, h->cap_stream)) enqueue_solve(h, ws, B, S, eps, false, h->cap_stream);
       ok = cudaStreamEndCapture(h->cap_stream, &graph) == cudaSuccess && graph != nullptr;
     }
   }
@@ -423,6 +436,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   ok = ok && dalloc(h, &ws.livek[0], Bm) && dalloc(h, &ws.livek[1], Bm);
   ok = ok && dalloc(h, &ws.cnt, Sm + 2) && dalloc(h, &ws.kdev, 1) && dalloc(h, &ws.flag, Bm) && dalloc(h, &ws.cand1, Bm);
   ok = ok && dalloc(h, &ws.upd_ctr, Sm + 1);
+  ok = ok && dalloc(h, &ws.score, N * (Bm < static_cast<size_t>(small_max_batch()) ? Bm : small_max_batch()));
   ok = ok && dalloc(h, &ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
        dalloc(h, &ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && dalloc(h, &ws.bv, Bm * Sm) &&
        dalloc(h, &ws.sup, Bm * Sm);
@@ -447,7 +461,8 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
                  (!ws.win_pos || cudaMemset(ws.win_pos, 0, Bp * sizeof(float)) == cudaSuccess) &&
                  cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
                  cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking) == cudaSuccess &&
-                 configure_update_kernels(ws) == cudaSuccess && configure_corr_simt(ws) == cudaSuccess;
+                 configure_update_kernels(ws) == cudaSuccess && configure_corr_simt(ws) == cudaSuccess &&
+                 configure_small(ws) == cudaSuccess;
   if (cuda_ok && d.precision != OMP_PREC_FP32) cuda_ok = tc_setup(ws, h->sm_count, &h->tc) == cudaSuccess;
   if (cuda_ok) cuda_ok = cudaDeviceSynchronize() == cudaSuccess;
   if (!cuda_ok) {

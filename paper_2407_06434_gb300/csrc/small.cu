@@ -1,0 +1,570 @@
+// Solves of few signals: the same iteration (Sec. 2.3, as in append.cuh) arranged for latency.
+//
+// A batch that does not fill the tensor-core tiles leaves the batched kernels waiting: one signal
+// over 8192 atoms of length 1024 took 39 us a step (the correlation 23 on 10 CTAs, one warp's
+// append and update 13, the compaction and three launches the rest), 16 signals over 64 x 256
+// 16 to 20 us. Here nothing is compacted and a signal has a block of eight warps:
+//   solo   a small dictionary: one block per signal runs every step in one launch, the residual,
+//          the scores and the factor in shared memory
+//   wide   a large dictionary and up to 8 signals: per step one launch scores every atom with the
+//          whole GPU (bound by reading the FP32 atom rows from L2), one does the rest with a block
+//          per signal
+// Scores here are FP32 dot products in an order of their own. An atom can only be the pick if its
+// score is within two error bounds of the best, so those atoms -- mostly one -- are scored again
+// as the batched path of the handle does it (FP32: one chain of FMAs over m; BF16: the rescoring's
+// order), and b and ||r|| are summed in the batched update's order: the same picks and bits.
+#include <type_traits>
+
+#include "append.cuh"
+
+namespace ompk {
+namespace {
+
+// One float4 slot's part of a dot product, rounded as the batched kernels (append.cuh) round it
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, int V0) {
+  return V0 == 1 ? slot_dot<true>(a, b) : slot_dot<false>(a, b);
+}
+constexpr int kT = 256, kWarps = kT / 32;
+constexpr int kSmallMaxB = 8;                      // wide: signals that share one pass over A
+constexpr int64_t kWideMaxElems = 24ll << 20;      // wide: FP32 rows of at most 96 MB stay in L2
+constexpr int64_t kWideMaxRows = 48 * 1024;         // wide: residuals in shared memory (192 KB)
+constexpr int64_t kSoloMaxElems = 1ll << 18;       // solo: at most 1 MB of atom rows a step and block
+constexpr int64_t kSoloMaxTotal = 24ll << 20;      // solo: at most 96 MB a step over all signals
+constexpr size_t kSmallMaxSmem = 100 * 1024;       // two blocks an SM at least
+
+struct SmallSmem {
+  float* r;      // Mp: the residual
+  float* P;      // Mp / 4 (rounded up to 32 lanes): per-slot partials of the ordered sums
+  float* part;   // 8: per-warp sums; [8]: the result
+  float* rs;     // 8 best scores and
+  int* ri;       // 8 their atoms
+  int* ctl;      // 4: candidates in the window, the pick
+  float* sc;     // N (solo): the scores
+  GroupSmem gs;  // the append's fields: tri, w, z, f, sup, scal
+};
+
+__host__ __device__ __forceinline__ int slots4(int Mp) { return (Mp / 4 + 31) / 32 * 32; }
+
+__host__ __device__ __forceinline__ size_t small_bytes(int Mp, int Smax, int nsc) {
+  const size_t words = static_cast<size_t>(Mp) + slots4(Mp) + (tri_floats(Smax) + 3) / 4 * 4 + 16 + 8 + 8 + 4 + 4 +
+                       4 * (static_cast<size_t>(Smax) + 4) + (nsc + 3) / 4 * 4;
+  return (words * 4 + 15) / 16 * 16;
+}
+
+__device__ __forceinline__ SmallSmem small_smem(unsigned char* base, int Mp, int Smax, int nsc) {
+  SmallSmem s;
+  s.r = reinterpret_cast<float*>(base);
+  s.P = s.r + Mp;
+  s.gs.tri = s.P + slots4(Mp);
+  s.sc = s.gs.tri + (tri_floats(Smax) + 3) / 4 * 4;
+  s.part = s.sc + (nsc + 3) / 4 * 4;
+  s.rs = s.part + 16;
+  s.ri = reinterpret_cast<int*>(s.rs + 8);
+  s.ctl = s.ri + 8;
+  s.gs.scal = s.ctl + 4;
+  s.gs.w = reinterpret_cast<float*>(s.gs.scal + 4);
+  s.gs.z = s.gs.w + Smax + 4;
+  s.gs.f = s.gs.z + Smax + 4;
+  s.gs.sup = reinterpret_cast<int*>(s.gs.f + Smax + 4);
+  return s;
+}
+
+// |<a, r>| / ||a|| as the batched BF16 rescoring forms it: the dot products of W0 warps' float4
+// slots, each lane's slots in order, a butterfly per warp, the warps' sums in order. One warp.
+__device__ __forceinline__ float rescore_dot(const float4* a, const float4* r, int M4, int W0, int V0, int lane) {
+  float v = 0.f;
+  for (int w = 0; w < W0; ++w) {
+    float acc = 0.f;
+#pragma unroll 8
+    for (int t = 0; t < V0; ++t) {
+      const int s = (t * W0 + w) * 32 + lane;
+      if (s < M4) {
+        const float4 x = __ldg(a + s);
+        const float4 y = r[s];
+        acc += dot4(x, y, V0);
+      }
+    }
+    v += warp_sum_f(acc);
+  }
+  return v;
+}
+
+// <a, r> as the batched FP32 correlation forms it: one chain of FMAs over m = 0, 1, ... One thread.
+__device__ __forceinline__ float chain_dot(const float4* a, const float4* r, int M4) {
+  float acc = 0.f;
+  for (int s0 = 0; s0 < M4; s0 += 16) {  // M4 is a multiple of 16
+    float4 x[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = __ldg(a + s0 + i);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float4 y = r[s0 + i];
+      acc = fmaf(y.x, x[i].x, acc);
+      acc = fmaf(y.y, x[i].y, acc);
+      acc = fmaf(y.z, x[i].z, acc);
+      acc = fmaf(y.w, x[i].w, acc);
+    }
+  }
+  return acc;
+}
+
+// The ordered sum of the block's per-slot partials sm.P (see rescore_dot); every thread gets it.
+// Begins and ends with a block barrier.
+__device__ __forceinline__ float ordered_sum(const SmallSmem& sm, int M4, int W0, int V0) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __syncthreads();
+  if (warp < W0) {
+    float acc = 0.f;
+    for (int t = 0; t < V0; ++t) {
+      const int s = (t * W0 + warp) * 32 + lane;
+      if (s < M4) acc += sm.P[s];
+    }
+    acc = warp_sum_f(acc);
+    if (lane == 0) sm.part[warp] = acc;
+  }
+  __syncthreads();
+  float v = 0.f;
+  for (int w = 0; w < W0; ++w) v += sm.part[w];
+  __syncthreads();
+  return v;
+}
+
+// An atom whose norm is so far from 1 that FP32 products with it may overflow or lose bits below
+// the normal range is always scored again: its score is a NaN, which passes the window's test.
+// (A zero atom scores 0 everywhere.)
+__device__ __forceinline__ float approx_score(float dot, float inv) {
+  return inv == 0.f || (inv > 1e-15f && inv < 1e15f) ? fabsf(dot) * inv : __int_as_float(0x7fffffff);
+}
+
+// The pick of the signal whose residual is sm.r, from the scores sc[0..N): the block agrees on it
+// (-1: no atom has a score).
+__device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, const float* sc, float rnorm, int W0,
+                                         int V0) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int N = ws.N, M4 = ws.Mp >> 2;
+  float bs = -1.f;
+  int bi = 0x7fffffff;
+  for (int n0 = tid; n0 < N; n0 += 8 * kT) {
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = n0 + i * kT < N ? sc[n0 + i * kT] : -2.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (v[i] > bs) {  // false for a NaN
+        bs = v[i];
+        bi = n0 + i * kT;
+      }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float os = __shfl_xor_sync(0xffffffffu, bs, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    if (better(os, oi, bs, bi)) {
+      bs = os;
+      bi = oi;
+    }
+  }
+  if (lane == 0) {
+    sm.rs[warp] = bs;
+    sm.ri[warp] = bi;
+  }
+  if (tid == 0) sm.ctl[0] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    if (better(sm.rs[w], sm.ri[w], bs, bi)) {
+      bs = sm.rs[w];
+      bi = sm.ri[w];
+    }
+  // both orders of summation are within gam_32 ||a|| ||r|| of the exact product; the products with
+  // 1/||a|| add two roundings each, 1% covers the rounding of the norms and of this bound
+  const float eps = 1.01f * (2.f * ws.gam_32 + 4.f * 0x1p-24f);
+  const bool ranged = rnorm > 1e-15f && rnorm < 1e15f;
+  const float thr = ranged ? bs - 2.f * eps * rnorm : -2.f;
+  int mine = 0;
+#pragma unroll 8
+  for (int n = tid; n < N; n += kT) mine += !(sc[n] < thr) ? 1 : 0;
+  mine = warp_sum_int(mine);
+  if (lane == 0 && mine) atomicAdd(sm.ctl, mine);
+  __syncthreads();
+  if (sm.ctl[0] == 1 && bi < N) return bi;  // the best is alone in the window
+  // score the window's atoms as the batched path does
+  const float4* r4 = reinterpret_cast<const float4*>(sm.r);
+  float cs = -1.f;
+  int ci = 0x7fffffff;
+  if (ws.prec == OMP_PREC_FP32) {
+    for (int n = tid; n < N; n += kT)
+      if (!(sc[n] < thr)) {
+        const float s =
+            fabsf(chain_dot(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp), r4, M4)) *
+            __ldg(ws.inv_norm + n);
+        if (s > cs) {
+          cs = s;
+          ci = n;
+        }
+      }
+  } else {
+    for (int n = warp; n < N; n += kWarps)
+      if (!(sc[n] < thr)) {
+        const float s = fabsf(rescore_dot(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp), r4,
+                                          M4, W0, V0, lane)) *
+                        __ldg(ws.inv_norm + n);
+        if (s > cs) {
+          cs = s;
+          ci = n;
+        }
+      }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float os = __shfl_xor_sync(0xffffffffu, cs, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, ci, o);
+    if (better(os, oi, cs, ci)) {
+      cs = os;
+      ci = oi;
+    }
+  }
+  __syncthreads();  // every warp has read rs and ri
+  if (lane == 0) {
+    sm.rs[warp] = cs;
+    sm.ri[warp] = ci;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    if (better(sm.rs[w], sm.ri[w], cs, ci)) {
+      cs = sm.rs[w];
+      ci = sm.ri[w];
+    }
+  return ci < N ? ci : -1;
+}
+
+// One step (append, residual update, stop test) of signal b with kk atoms, the residual in sm.r and
+// the support in sm.gs.sup. V: float4 slots per thread. Returns whether the signal goes on; *rn
+// becomes its ||r||. Fr: where the factor is read and its new column written in FP32.
+template <int V>
+__device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, const float* sc, int b, int kk, int S,
+                                           float eps, int eps_rel, float ynorm, int W0, int V0, float* Fr, float* rn) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int M4 = ws.Mp >> 2;
+  const GroupSmem& gs = sm.gs;
+  const float rprev = *rn;
+  const int ns = pick_atom(ws, sm, sc, rprev, W0, V0);
+  if (ns < 0) {
+    if (tid == 0) {
+      atomicOr(ws.err, OMP_DEVERR_BAD_STATE);
+      ws.flag[b] = 0;
+    }
+    return false;
+  }
+  if (warp == 0) {
+    const float* grow = ws.gram + static_cast<size_t>(ns) * ws.N;
+    for (int i = lane; i < kk; i += 32) gs.w[i] = __ldg(grow + gs.sup[i]);
+    __syncwarp();
+    double* Fg = ws.F + static_cast<size_t>(b) * ws.Fstride;
+    const int nb = (kk + 31) >> 5;
+    if (nb <= 1) append_column<1>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
+    else if (nb <= 2) append_column<2>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
+    else if (nb <= 4) append_column<4>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
+    else append_column<8>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
+  }
+  __syncthreads();
+  if (gs.scal[1]) {
+    if (tid == 0) {
+      ws.flag[b] = 0;
+      ws.stop[b] = kStopDependent;
+    }
+    return false;
+  }
+  // q = A_S f: thread's slots tid + 256 t, the rows in order, four rows in flight
+  float4 q[V];
+#pragma unroll
+  for (int t = 0; t < V; ++t) q[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  constexpr int R = V <= 2 ? 8 : V <= 4 ? 4 : 2;
+  for (int a0 = 0; a0 <= kk; a0 += R) {
+    float4 v[R][V];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int a = a0 + i;
+      const float4* row = reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(a <= kk ? gs.sup[a] : ns) * ws.Mp);
+#pragma unroll
+      for (int t = 0; t < V; ++t) {
+        const int s = t * kT + tid;
+        v[i][t] = a <= kk && s < M4 ? __ldg(row + s) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      if (a0 + i <= kk) {
+        const float f = gs.f[a0 + i];
+#pragma unroll
+        for (int t = 0; t < V; ++t) {
+          q[t].x = fmaf(f, v[i][t].x, q[t].x);
+          q[t].y = fmaf(f, v[i][t].y, q[t].y);
+          q[t].z = fmaf(f, v[i][t].z, q[t].z);
+          q[t].w = fmaf(f, v[i][t].w, q[t].w);
+        }
+      }
+    }
+  }
+  float4* r4 = reinterpret_cast<float4*>(sm.r);
+  float4 r[V];
+#pragma unroll
+  for (int t = 0; t < V; ++t) {
+    const int s = t * kT + tid;
+    r[t] = s < M4 ? r4[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (s < M4) sm.P[s] = dot4(q[t], r[t], V0);
+  }
+  const float bf = ordered_sum(sm, M4, W0, V0);
+#pragma unroll
+  for (int t = 0; t < V; ++t) {
+    const int s = t * kT + tid;
+    r[t].x = fmaf(-bf, q[t].x, r[t].x);
+    r[t].y = fmaf(-bf, q[t].y, r[t].y);
+    r[t].z = fmaf(-bf, q[t].z, r[t].z);
+    r[t].w = fmaf(-bf, q[t].w, r[t].w);
+    if (s < M4) {
+      r4[s] = r[t];
+      sm.P[s] = slot_dot<false>(r[t], r[t]);
+    }
+  }
+  const float rk = sqrtf(ordered_sum(sm, M4, W0, V0));
+  *rn = rk;
+  const float thr = eps_rel ? eps * ynorm : eps;
+  const bool hit = rk <= thr, last = kk + 1 >= S;
+  if (tid == 0) {
+    const size_t o = static_cast<size_t>(b) * ws.Smax + kk;
+    ws.bv[o] = static_cast<double>(bf);
+    ws.sup[o] = ns;
+    ws.drop[o] = rprev > 0.f ? (bf / rprev) * (bf / rprev) : 0.f;
+    ws.niter[b] = kk + 1;
+    ws.rnorm[b] = rk;
+    if (hit || last) {
+      ws.flag[b] = 0;
+      ws.stop[b] = hit ? kStopEps : kStopIters;
+    }
+  }
+  return !(hit || last);
+}
+
+// Scores of atoms [n_lo, n_hi) for one residual in shared memory, LPA lanes per atom (16 when a row
+// has 64 elements), the warp's atoms n_lo + warp index, ...; U atoms in flight per lane group.
+template <int LPA, int U>
+__device__ __forceinline__ void score_atoms(const Ws& ws, const float4* r4, int first, int stride, float* sc) {
+  const int lane = threadIdx.x & 31, sub = lane % LPA, grp = lane / LPA;
+  constexpr int GP = 32 / LPA;  // atoms a warp takes side by side
+  const int M4 = ws.Mp >> 2, N = ws.N;
+  for (int n0 = first * GP * U; n0 < N; n0 += stride * GP * U) {
+    float acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) acc[u] = 0.f;
+#pragma unroll 2
+    for (int s = sub; s < M4; s += LPA) {
+      const float4 y = r4[s];
+      float4 x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int n = n0 + u * GP + grp;
+        x[u] = n < N ? __ldg(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp) + s)
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        acc[u] = fmaf(x[u].w, y.w, fmaf(x[u].z, y.z, fmaf(x[u].y, y.y, fmaf(x[u].x, y.x, acc[u]))));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int o = LPA / 2; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+      const int n = n0 + u * GP + grp;
+      if (sub == 0 && n < N) sc[n] = approx_score(acc[u], __ldg(ws.inv_norm + n));
+    }
+  }
+}
+
+// Every step of one signal per block.
+template <int V>
+__global__ void __launch_bounds__(kT, 2) solo_kernel(Ws ws, int S, float eps, int eps_rel, int W0, int V0) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int b = blockIdx.x;
+  if (!ws.flag[b]) return;  // y == 0 or non-finite
+  SmallSmem sm = small_smem(smem, ws.Mp, ws.Smax, ws.N);
+  const float4* rg = reinterpret_cast<const float4*>(ws.R32 + static_cast<size_t>(b) * ws.Mp);
+  for (int s = tid; s < (ws.Mp >> 2); s += kT) reinterpret_cast<float4*>(sm.r)[s] = rg[s];
+  float* Fr = ws.Smax <= kTriMax ? sm.gs.tri : ws.F32 + static_cast<size_t>(b) * ws.Fstride;
+  const float ynorm = ws.ynorm[b];
+  float rn = ws.rnorm[b];
+  bool go = true;
+  for (int kk = 0; go; ++kk) {
+    __syncthreads();  // the residual is complete, and every read of the last step's scores is done
+    const float4* r4 = reinterpret_cast<const float4*>(sm.r);
+    if (ws.Mp == 64)
+      score_atoms<16, 8>(ws, r4, warp, kWarps, sm.sc);
+    else
+      score_atoms<32, 8>(ws, r4, warp, kWarps, sm.sc);
+    __syncthreads();
+    go = small_step<V>(ws, sm, sm.sc, b, kk, S, eps, eps_rel, ynorm, W0, V0, Fr, &rn);
+  }
+}
+
+// Scores of every atom for the (up to kSmallMaxB) signals still going, written to ws.score (B x N).
+// A warp takes atoms 8 apart over the grid; a row is read once for all signals.
+__global__ void __launch_bounds__(kT) wide_score_kernel(Ws ws, int B) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float4* rs = reinterpret_cast<float4*>(smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int M4 = ws.Mp >> 2, N = ws.N;
+  __shared__ int act[kSmallMaxB], na_s;  // the signals that go on
+  if (tid == 0) {
+    int n = 0;
+    for (int b = 0; b < B; ++b)
+      if (ws.flag[b]) act[n++] = b;
+    na_s = n;
+  }
+  __syncthreads();
+  const int na = na_s;
+  if (na == 0) return;
+  for (int i = 0; i < na; ++i)
+    for (int s = tid; s < M4; s += kT)
+      rs[static_cast<size_t>(i) * M4 + s] =
+          reinterpret_cast<const float4*>(ws.R32 + static_cast<size_t>(act[i]) * ws.Mp)[s];
+  __syncthreads();
+  if (na == 1) {
+    const int first = blockIdx.x * kWarps + warp, stride = gridDim.x * kWarps;
+    if (ws.Mp == 64)
+      score_atoms<16, 4>(ws, rs, first, stride, ws.score + static_cast<size_t>(act[0]) * N);
+    else
+      score_atoms<32, 4>(ws, rs, first, stride, ws.score + static_cast<size_t>(act[0]) * N);
+    return;
+  }
+  constexpr int U = 2;
+  for (int n0 = (blockIdx.x * kWarps + warp) * U; n0 < N; n0 += gridDim.x * kWarps * U) {
+    float acc[U][kSmallMaxB];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int i = 0; i < kSmallMaxB; ++i) acc[u][i] = 0.f;
+    for (int s = lane; s < M4; s += 32) {
+      float4 x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        x[u] = n0 + u < N ? __ldg(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n0 + u) * ws.Mp) + s)
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < kSmallMaxB; ++i) {
+        if (i < na) {
+          const float4 y = rs[static_cast<size_t>(i) * M4 + s];
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            acc[u][i] = fmaf(x[u].w, y.w, fmaf(x[u].z, y.z, fmaf(x[u].y, y.y, fmaf(x[u].x, y.x, acc[u][i]))));
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float inv = n0 + u < N ? __ldg(ws.inv_norm + n0 + u) : 0.f;
+#pragma unroll
+      for (int i = 0; i < kSmallMaxB; ++i) {
+        if (i < na) {
+          const float d = warp_sum_f(acc[u][i]);
+          if (lane == 0 && n0 + u < N) ws.score[static_cast<size_t>(act[i]) * N + n0 + u] = approx_score(d, inv);
+        }
+      }
+    }
+  }
+}
+
+// One step of each signal from the scores in ws.score
+template <int V>
+__global__ void __launch_bounds__(kT, 1) wide_step_kernel(Ws ws, int S, float eps, int eps_rel, int W0, int V0) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int tid = threadIdx.x;
+  const int b = blockIdx.x;
+  if (!ws.flag[b]) return;
+  SmallSmem sm = small_smem(smem, ws.Mp, ws.Smax, 0);
+  const int kk = ws.niter[b];
+  float4* rg = reinterpret_cast<float4*>(ws.R32 + static_cast<size_t>(b) * ws.Mp);
+  for (int s = tid; s < (ws.Mp >> 2); s += kT) reinterpret_cast<float4*>(sm.r)[s] = rg[s];
+  float* Ff = ws.F32 + static_cast<size_t>(b) * ws.Fstride;
+  const bool staged = ws.Smax <= kTriMax;
+  if (staged)
+    for (int i = tid; i < kk * (kk + 1) / 2; i += kT) sm.gs.tri[i] = Ff[i];
+  for (int i = tid; i < kk; i += kT) sm.gs.sup[i] = ws.sup[static_cast<size_t>(b) * ws.Smax + i];
+  float rn = ws.rnorm[b];
+  const float ynorm = ws.ynorm[b];
+  __syncthreads();
+  const bool go = small_step<V>(ws, sm, ws.score + static_cast<size_t>(b) * ws.N, b, kk, S, eps, eps_rel, ynorm, W0, V0,
+                                staged ? sm.gs.tri : Ff, &rn);
+  if (!go) return;
+  for (int s = tid; s < (ws.Mp >> 2); s += kT) rg[s] = reinterpret_cast<float4*>(sm.r)[s];
+  if (staged)  // the new factor column
+    for (int i = tid; i <= kk; i += kT) Ff[kk * (kk + 1) / 2 + i] = sm.gs.tri[kk * (kk + 1) / 2 + i];
+}
+
+int slots_per_thread(int Mp) {
+  const int need = (Mp / 4 + kT - 1) / kT;
+  int V = 1;
+  while (V < need) V <<= 1;
+  return V;
+}
+
+template <class F>
+void by_slots(int V, F f) {
+  if (V == 1) f(std::integral_constant<int, 1>{});
+  else if (V == 2) f(std::integral_constant<int, 2>{});
+  else if (V == 4) f(std::integral_constant<int, 4>{});
+  else f(std::integral_constant<int, 8>{});
+}
+
+}  // namespace
+
+// Which arrangement a solve takes: 0 batched, 1 solo, 2 wide. The quantised 8-bit path, fewer than
+// 8 rescored candidates, recorded margins, the 24-bit gather and the hook that turns the score
+// bound off stay batched: their picks depend on what the batched path keeps of its lists.
+int small_form(const Ws& ws, int B) {
+  if (ws.prec == OMP_PREC_FP8_E4M3 || ws.A24h || ws.margin) return 0;
+  if (ws.prec == OMP_PREC_BF16 && (ws.topk != kMaxTopk || !(ws.rescore_eps > 0.f))) return 0;
+  const int64_t elems = static_cast<int64_t>(ws.N) * ws.Mp;
+  if (elems <= kSoloMaxElems && elems * B <= kSoloMaxTotal && small_bytes(ws.Mp, ws.Smax, ws.N) <= kSmallMaxSmem)
+    return 1;
+  if (B <= kSmallMaxB && elems <= kWideMaxElems && static_cast<int64_t>(ws.Mp) * B <= kWideMaxRows) return 2;
+  return 0;
+}
+
+cudaError_t configure_small(const Ws& ws) {
+  cudaError_t e = cudaSuccess;
+  by_slots(slots_per_thread(ws.Mp), [&](auto v) {
+    constexpr int V = decltype(v)::value;
+    const size_t solo = small_bytes(ws.Mp, ws.Smax, ws.N);
+    if (solo <= kSmallMaxSmem) e = raise_smem_limit(reinterpret_cast<const void*>(solo_kernel<V>), solo);
+    if (e == cudaSuccess)
+      e = raise_smem_limit(reinterpret_cast<const void*>(wide_step_kernel<V>), small_bytes(ws.Mp, ws.Smax, 0));
+  });
+  if (e == cudaSuccess)
+    e = raise_smem_limit(reinterpret_cast<const void*>(wide_score_kernel), kWideMaxRows * 4);
+  return e;
+}
+
+int small_max_batch() { return kSmallMaxB; }
+
+void launch_solo(const Ws& ws, int B, int S, float eps, int eps_rel, cudaStream_t s) {
+  by_slots(slots_per_thread(ws.Mp), [&](auto v) {
+    constexpr int V = decltype(v)::value;
+    solo_kernel<V><<<B, kT, small_bytes(ws.Mp, ws.Smax, ws.N), s>>>(ws, S, eps, eps_rel, ws.upd_w,
+                                                                    update_slots(ws.Mp, ws.upd_w));
+  });
+}
+
+void launch_wide(const Ws& ws, int sms, int B, int S, float eps, int eps_rel, cudaStream_t s) {
+  const int per = kWarps * 4;
+  const int blocks = (ws.N + per - 1) / per, grid = blocks < 2 * sms ? blocks : 2 * sms;
+  wide_score_kernel<<<grid, kT, static_cast<size_t>(ws.Mp) * 4 * B, s>>>(ws, B);
+  by_slots(slots_per_thread(ws.Mp), [&](auto v) {
+    constexpr int V = decltype(v)::value;
+    wide_step_kernel<V><<<B, kT, small_bytes(ws.Mp, ws.Smax, 0), s>>>(ws, S, eps, eps_rel, ws.upd_w,
+                                                                     update_slots(ws.Mp, ws.upd_w));
+  });
+}
+
+}  // namespace ompk

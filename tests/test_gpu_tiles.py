@@ -67,3 +67,61 @@ def test_gram_entries_of_any_tile(lib, N):
         cond = np.linalg.cond(A64[sup[b]])
         assert np.linalg.norm(X[b] - ref) <= 64 * 2.0 ** -24 * cond ** 2 * np.linalg.norm(ref)
     s.close()
+
+
+def _planted(M, N, B, S, seed):
+    rng = np.random.default_rng(seed)
+    At = rng.standard_normal((N, M)).astype(np.float32)
+    At *= (rng.uniform(0.5, 2.0, (N, 1)) / np.linalg.norm(At, axis=1, keepdims=True)).astype(np.float32)
+    Y = 1e-3 * rng.standard_normal((B, M))
+    for b in range(B):
+        sup = rng.choice(N, S, replace=False)
+        Y[b] += At[sup].T.astype(np.float64) @ rng.standard_normal(S)
+    return torch.from_numpy(At).cuda().t(), torch.from_numpy(Y.astype(np.float32)).cuda()
+
+
+# Few signals take kernels of their own, which pick the same atoms and round every sum alike: the
+# device-side loop (use_graph 2) always runs the batched kernels, and the results are bit for bit
+# the same. Sizes: one slot per lane and ragged ones, one block per signal at and above the small
+# dictionary's limit, 1 to 8 signals over a large one, a factor too long to stage, an eps stop.
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("M,N,B,S,eps", [
+    (64, 256, 16, 8, 0.0), (33, 40, 3, 5, 0.0), (128, 512, 100, 16, 0.0), (203, 700, 30, 20, 1e-2),
+    (1024, 256, 40, 24, 0.0), (1024, 257, 8, 24, 0.0), (1024, 8192, 1, 32, 0.0), (700, 5000, 7, 24, 1e-2),
+    (1500, 4001, 8, 30, 0.0), (4096, 3000, 2, 40, 0.0), (5000, 1201, 2, 100, 0.0), (8192, 600, 6, 16, 0.0)])
+def test_few_signals_match_the_batched_kernels(lib, prec, M, N, B, S, eps):
+    A, Y = _planted(M, N, B, S, M + 7 * N + B)
+    if B > 2:
+        Y[1] = 0.0                      # an empty signal
+        Y[2] = Y[0]                     # and a repeated one
+    out = []
+    for graph in (1, 0, 2):
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=prec, use_graph=graph)
+        out.append([t.cpu().numpy() for t in s.solve(A, Y, S, eps, diagnostics=True)])
+        s.close()
+    for got in out[:2]:
+        for g, want in zip(got, out[2]):
+            assert np.array_equal(g.view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_few_signals_ties_and_extreme_scales(lib, prec):
+    """Duplicate atoms (the lowest index wins), a zero atom, atoms and signals far from unit norm."""
+    A, Y = _planted(96, 300, 4, 6, 5)
+    At = A.t().contiguous()
+    At[200] = At[17]
+    At[18] = At[17]
+    At[5] = 0.0
+    At[40] *= 1e18
+    At[41] *= 1e-18
+    Y[0] = 2.0 * At[17] + 0.5 * At[60]
+    Y[1] *= 1e-17
+    Y[3] = At[41] * 1e18 + At[40] * 1e-18
+    out = []
+    for graph in (1, 2):
+        s = lib.OmpSolver(96, 300, max_batch=4, max_iters=6, precision=prec, use_graph=graph)
+        out.append([t.cpu().numpy() for t in s.solve(At.t(), Y, 6, 0.0, diagnostics=True)])
+        s.close()
+    assert out[0][1][0, 0] == 17
+    for g, want in zip(*out):
+        assert np.array_equal(g.view(np.uint32), want.view(np.uint32))
