@@ -138,20 +138,38 @@ __device__ __forceinline__ GroupSmem group_smem(unsigned char* base, int grp, co
 // for t < NB covers the kk <= 32 NB rows/columns of F (NB is the smallest power of two that fits,
 // so early iterations issue no predicated-off work). Fr is where the current factor is read (a
 // shared-memory copy or F itself); the new column goes to Ff (FP32) and Fg (FP64).
-template <int NB>
+// nrm2 is ||a_ns||^2, loaded by the caller ahead of time. The two triangular loops read UR steps ahead
+// of their chains of FMAs (a step at a time each waits for a shared-memory round trip), where the
+// kernel has the registers.
+template <int NB, int UR = 1>
 __device__ __forceinline__ void append_column(const Ws& ws, const GroupSmem& gs, const float* Fr,
-                                              float* Ff, double* Fg, int kk, int ns, int lane) {
+                                              float* Ff, double* Fg, int kk, int ns, double nrm2, int lane) {
   // z_j = sum_{i<=j} F[i,j] w_i
   float zl[NB];
 #pragma unroll
   for (int t = 0; t < NB; ++t) zl[t] = 0.f;
-  for (int i = 0; i < kk; ++i) {
-    const float wi = gs.w[i];
+  const float* col[NB];  // lane slot j's own column (a lane past the support reads the last one)
+  int top[NB];
 #pragma unroll
-    for (int t = 0; t < NB; ++t) {
-      const int j = lane + 32 * t;
-      if (j < kk && i <= j) zl[t] = fmaf(Fr[static_cast<size_t>(j) * (j + 1) / 2 + i], wi, zl[t]);
+  for (int t = 0; t < NB; ++t) {
+    top[t] = min(lane + 32 * t, kk - 1);
+    col[t] = Fr + top[t] * (top[t] + 1) / 2;
+  }
+  for (int i0 = 0; i0 < kk; i0 += UR) {
+    float wv[UR], fv[NB][UR];
+#pragma unroll
+    for (int e = 0; e < UR; ++e) {
+      wv[e] = gs.w[UR > 1 ? min(i0 + e, kk - 1) : i0];
+#pragma unroll
+      for (int t = 0; t < NB; ++t) fv[t][e] = col[t][min(i0 + e, top[t])];
     }
+#pragma unroll
+    for (int e = 0; e < UR; ++e)
+#pragma unroll
+      for (int t = 0; t < NB; ++t) {
+        const int j = lane + 32 * t;
+        if (j < kk && i0 + e <= j) zl[t] = fmaf(fv[t][e], wv[e], zl[t]);
+      }
   }
   // ||z||^2 as an unevaluated sum hi + lo of FP32 numbers: each square is split exactly by an
   // FMA and the sums are error-free (Knuth's two-sum), so the FP64 Schur complement below gets
@@ -175,7 +193,6 @@ __device__ __forceinline__ void append_column(const Ws& ws, const GroupSmem& gs,
     two_sum(zh, zlo, oh);
   }
   const double zz = static_cast<double>(zh) + static_cast<double>(zlo);
-  const double nrm2 = ws.norm2[ns];
   const double delta = nrm2 - zz;
   const bool dep = !(delta > kDepRtol * nrm2);
   if (lane == 0) gs.scal[1] = dep ? 1 : 0;
@@ -194,14 +211,22 @@ __device__ __forceinline__ void append_column(const Ws& ws, const GroupSmem& gs,
   float ul[NB];
 #pragma unroll
   for (int t = 0; t < NB; ++t) ul[t] = 0.f;
-  for (int j = 0; j < kk; ++j) {
-    const float zj = gs.z[j];
-    const float* col = Fr + static_cast<size_t>(j) * (j + 1) / 2;
+  for (int j0 = 0, cj = 0; j0 < kk; j0 += UR) {  // cj: the offset of column j0
+    float zv[UR], fv[NB][UR];
 #pragma unroll
-    for (int t = 0; t < NB; ++t) {
-      const int i = lane + 32 * t;
-      if (i <= j) ul[t] = fmaf(col[i], zj, ul[t]);
+    for (int e = 0; e < UR; ++e) {
+      const int j = j0 + e;
+      const bool in = UR == 1 || j < kk;
+      zv[e] = gs.z[in ? j : 0];
+#pragma unroll
+      for (int t = 0; t < NB; ++t) fv[t][e] = Fr[in ? cj + min(lane + 32 * t, j) : 0];
+      cj += j + 1;
     }
+#pragma unroll
+    for (int e = 0; e < UR; ++e)
+#pragma unroll
+      for (int t = 0; t < NB; ++t)
+        if (j0 + e < kk && lane + 32 * t <= j0 + e) ul[t] = fmaf(fv[t][e], zv[e], ul[t]);
   }
   const size_t off = static_cast<size_t>(kk) * (kk + 1) / 2;
 #pragma unroll
@@ -541,14 +566,21 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
       cp_async_wait_all();
     __syncwarp();
     const float* grow = ws.gram + static_cast<size_t>(ns) * ws.N;
+    const double nrm2 = __ldg(ws.norm2 + ns);
     for (int i = lane; i < kk; i += 32) gs.w[i] = __ldg(grow + gs.sup[i]);
     __syncwarp();
-    const float* Fr = staged ? gs.tri : Ff;
+    // (two calls, so that the staged factor is read as shared memory and not through a generic
+    // address; it is staged for at most 64 atoms)
     const int nb = (kk + 31) >> 5;
-    if (nb <= 1) append_column<1>(ws, gs, Fr, Ff, Fg, kk, ns, lane);
-    else if (nb <= 2) append_column<2>(ws, gs, Fr, Ff, Fg, kk, ns, lane);
-    else if (nb <= 4) append_column<4>(ws, gs, Fr, Ff, Fg, kk, ns, lane);
-    else append_column<8>(ws, gs, Fr, Ff, Fg, kk, ns, lane);
+    if (staged) {
+      if (nb <= 1) append_column<1>(ws, gs, gs.tri, Ff, Fg, kk, ns, nrm2, lane);
+      else append_column<2>(ws, gs, gs.tri, Ff, Fg, kk, ns, nrm2, lane);
+    } else {
+      if (nb <= 1) append_column<1>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+      else if (nb <= 2) append_column<2>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+      else if (nb <= 4) append_column<4>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+      else append_column<8>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+    }
   }
   group_sync(W, grp);
   if (gs.scal[1]) {

@@ -81,7 +81,7 @@ struct Ws {
   float* escale;   // quantised paths: score scale per atom (1/||a|| or s_a/||a||), padded
   double* norm2;
   float* gram;
-  float* score;     // up to 8 signals x N: FP32 scores of a solve of few signals (small.cu)
+  float* score;     // FP32 scores of a solve of up to 8 signals (small.cu)
   float* c0;        // Bmax x N FP32 first correlation of the Gram-space solve (allocated on use)
   // signal state
   float* R32;
@@ -285,7 +285,7 @@ void launch_update_w8(const Ws& ws, int V, int k, int B, int S, float eps, int e
 
 // solves of few signals (small.cu): the form a solve takes (0: batched), and its launches
 int small_form(const Ws& ws, int B);
-int small_max_batch();
+size_t small_score_floats(int N, int Bmax);
 cudaError_t configure_small(const Ws& ws);
 void launch_solo(const Ws& ws, int B, int S, float eps, int eps_rel, cudaStream_t s);
 void launch_wide(const Ws& ws, int sms, int B, int S, float eps, int eps_rel, cudaStream_t s);

@@ -436,7 +436,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   ok = ok && dalloc(h, &ws.livek[0], Bm) && dalloc(h, &ws.livek[1], Bm);
   ok = ok && dalloc(h, &ws.cnt, Sm + 2) && dalloc(h, &ws.kdev, 1) && dalloc(h, &ws.flag, Bm) && dalloc(h, &ws.cand1, Bm);
   ok = ok && dalloc(h, &ws.upd_ctr, Sm + 1);
-  ok = ok && dalloc(h, &ws.score, N * (Bm < static_cast<size_t>(small_max_batch()) ? Bm : small_max_batch()));
+  ok = ok && dalloc(h, &ws.score, small_score_floats(ws.N, ws.Bmax));
   ok = ok && dalloc(h, &ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
        dalloc(h, &ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && dalloc(h, &ws.bv, Bm * Sm) &&
        dalloc(h, &ws.sup, Bm * Sm);

@@ -25,12 +25,18 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, int V0) 
   return V0 == 1 ? slot_dot<true>(a, b) : slot_dot<false>(a, b);
 }
 constexpr int kT = 256, kWarps = kT / 32;
+constexpr int kGS = 4;                             // wide: scores per recorded maximum
 constexpr int kSmallMaxB = 8;                      // wide: signals that share one pass over A
 constexpr int64_t kWideMaxElems = 24ll << 20;      // wide: FP32 rows of at most 96 MB stay in L2
 constexpr int64_t kWideMaxRows = 48 * 1024;         // wide: residuals in shared memory (192 KB)
 constexpr int64_t kSoloMaxElems = 1ll << 18;       // solo: at most 1 MB of atom rows a step and block
 constexpr int64_t kSoloMaxTotal = 24ll << 20;      // solo: at most 96 MB a step over all signals
-constexpr size_t kSmallMaxSmem = 100 * 1024;       // two blocks an SM at least
+constexpr size_t kSmallMaxSmem = 100 * 1024;       // solo: two blocks an SM at least
+constexpr size_t kWideMaxSmem = 216 * 1024;
+
+// floats per signal of ws.score: N scores, then the largest of each kGS of them
+__host__ __device__ __forceinline__ size_t score_pitch(int N) { return static_cast<size_t>(N) + (N + kGS - 1) / kGS; }
+
 
 struct SmallSmem {
   float* r;      // Mp: the residual
@@ -40,21 +46,23 @@ struct SmallSmem {
   int* ri;       // 8 their atoms
   int* ctl;      // 4: candidates in the window, the pick
   float* sc;     // N (solo): the scores
+  float* rows;   // RC x Mp: the support's first RC atom rows, or (solo) the whole dictionary
   GroupSmem gs;  // the append's fields: tri, w, z, f, sup, scal
 };
 
 __host__ __device__ __forceinline__ int slots4(int Mp) { return (Mp / 4 + 31) / 32 * 32; }
 
-__host__ __device__ __forceinline__ size_t small_bytes(int Mp, int Smax, int nsc) {
-  const size_t words = static_cast<size_t>(Mp) + slots4(Mp) + (tri_floats(Smax) + 3) / 4 * 4 + 16 + 8 + 8 + 4 + 4 +
-                       4 * (static_cast<size_t>(Smax) + 4) + (nsc + 3) / 4 * 4;
+__host__ __device__ __forceinline__ size_t small_bytes(int Mp, int Smax, int nsc, int RC) {
+  const size_t words = static_cast<size_t>(Mp) * (1 + RC) + slots4(Mp) + (tri_floats(Smax) + 3) / 4 * 4 +
+                       (nsc + 3) / 4 * 4 + 16 + 8 + 8 + 4 + 4 + 4 * (static_cast<size_t>(Smax) + 4);
   return (words * 4 + 15) / 16 * 16;
 }
 
-__device__ __forceinline__ SmallSmem small_smem(unsigned char* base, int Mp, int Smax, int nsc) {
+__device__ __forceinline__ SmallSmem small_smem(unsigned char* base, int Mp, int Smax, int nsc, int RC) {
   SmallSmem s;
   s.r = reinterpret_cast<float*>(base);
-  s.P = s.r + Mp;
+  s.rows = s.r + Mp;
+  s.P = s.rows + static_cast<size_t>(Mp) * RC;
   s.gs.tri = s.P + slots4(Mp);
   s.sc = s.gs.tri + (tri_floats(Smax) + 3) / 4 * 4;
   s.part = s.sc + (nsc + 3) / 4 * 4;
@@ -67,6 +75,13 @@ __device__ __forceinline__ SmallSmem small_smem(unsigned char* base, int Mp, int
   s.gs.f = s.gs.z + Smax + 4;
   s.gs.sup = reinterpret_cast<int*>(s.gs.f + Smax + 4);
   return s;
+}
+
+// rows of the support kept in shared memory: as many as `budget` bytes leave room for
+int row_cache(int Mp, int Smax, int nsc, size_t budget) {
+  const size_t base = small_bytes(Mp, Smax, nsc, 0);
+  const size_t room = base < budget ? (budget - base) / (static_cast<size_t>(Mp) * 4) : 0;
+  return room < static_cast<size_t>(Smax) ? static_cast<int>(room) : Smax;
 }
 
 // |<a, r>| / ||a|| as the batched BF16 rescoring forms it: the dot products of W0 warps' float4
@@ -109,23 +124,28 @@ __device__ __forceinline__ float chain_dot(const float4* a, const float4* r, int
 }
 
 // The ordered sum of the block's per-slot partials sm.P (see rescore_dot); every thread gets it.
-// Begins and ends with a block barrier.
-__device__ __forceinline__ float ordered_sum(const SmallSmem& sm, int M4, int W0, int V0) {
+// `part`: one of the two halves of sm.part (alternate them: no barrier follows the last read).
+__device__ __forceinline__ float ordered_sum(const SmallSmem& sm, float* part, int M4, int W0, int V0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __syncthreads();
   if (warp < W0) {
-    float acc = 0.f;
-    for (int t = 0; t < V0; ++t) {
+    float acc = 0.f, p[8];  // V0 <= 8
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
       const int s = (t * W0 + warp) * 32 + lane;
-      if (s < M4) acc += sm.P[s];
+      p[t] = t < V0 && s < M4 ? sm.P[s] : 0.f;
     }
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (t < V0) acc += p[t];
     acc = warp_sum_f(acc);
-    if (lane == 0) sm.part[warp] = acc;
+    if (lane == 0) part[warp] = acc;
   }
   __syncthreads();
   float v = 0.f;
-  for (int w = 0; w < W0; ++w) v += sm.part[w];
-  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w)
+    if (w < W0) v += part[w];
   return v;
 }
 
@@ -136,58 +156,63 @@ __device__ __forceinline__ float approx_score(float dot, float inv) {
   return inv == 0.f || (inv > 1e-15f && inv < 1e15f) ? fabsf(dot) * inv : __int_as_float(0x7fffffff);
 }
 
-// The pick of the signal whose residual is sm.r, from the scores sc[0..N): the block agrees on it
+__device__ __forceinline__ void load_head(float (&head)[8], const float* gm, int NG) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int g = threadIdx.x + i * kT;
+    head[i] = g < NG ? gm[g] : -2.f;
+  }
+}
+
+// The pick of the signal whose residual is sm.r, from the scores sc[0..N) and, per GS of them, their
+// largest gm[0..N/GS) (gm = sc for GS 1; a NaN where a group holds one): the block agrees on it
 // (-1: no atom has a score).
-__device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, const float* sc, float rnorm, int W0,
-                                         int V0) {
+// head: this thread's first 8 maxima (gm[tid + 256 i], -2 past the end), loaded ahead.
+template <int GS>
+__device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, const float* sc, const float* gm,
+                                         const float (&head)[8], float rnorm, int W0, int V0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int N = ws.N, M4 = ws.Mp >> 2;
+  const int N = ws.N, M4 = ws.Mp >> 2, NG = (N + GS - 1) / GS;
   float bs = -1.f;
-  int bi = 0x7fffffff;
-  for (int n0 = tid; n0 < N; n0 += 8 * kT) {
+  for (int g0 = tid; g0 < NG; g0 += 8 * kT) {
     float v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = n0 + i * kT < N ? sc[n0 + i * kT] : -2.f;
+    for (int i = 0; i < 8; ++i) v[i] = g0 == tid ? head[i] : g0 + i * kT < NG ? gm[g0 + i * kT] : -2.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (v[i] > bs) {  // false for a NaN
-        bs = v[i];
-        bi = n0 + i * kT;
-      }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float os = __shfl_xor_sync(0xffffffffu, bs, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (better(os, oi, bs, bi)) {
-      bs = os;
-      bi = oi;
+    for (int i = 0; i < 8; ++i) {
+      bs = fmaxf(bs, v[i]);  // a NaN is passed over
+      if (GS > 1 && v[i] != v[i])
+        for (int n = (g0 + i * kT) * GS; n < min(N, (g0 + i * kT) * GS + GS); ++n) bs = fmaxf(bs, sc[n]);
     }
   }
-  if (lane == 0) {
-    sm.rs[warp] = bs;
-    sm.ri[warp] = bi;
-  }
+  bs = warp_max(bs);
+  if (lane == 0) sm.rs[warp] = bs;
   if (tid == 0) sm.ctl[0] = 0;
   __syncthreads();
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w)
-    if (better(sm.rs[w], sm.ri[w], bs, bi)) {
-      bs = sm.rs[w];
-      bi = sm.ri[w];
-    }
+  for (int w = 0; w < kWarps; ++w) bs = fmaxf(bs, sm.rs[w]);
   // both orders of summation are within gam_32 ||a|| ||r|| of the exact product; the products with
   // 1/||a|| add two roundings each, 1% covers the rounding of the norms and of this bound
   const float eps = 1.01f * (2.f * ws.gam_32 + 4.f * 0x1p-24f);
   const bool ranged = rnorm > 1e-15f && rnorm < 1e15f;
   const float thr = ranged ? bs - 2.f * eps * rnorm : -2.f;
-  int mine = 0;
-#pragma unroll 8
-  for (int n = tid; n < N; n += kT) mine += !(sc[n] < thr) ? 1 : 0;
-  mine = warp_sum_int(mine);
-  if (lane == 0 && mine) atomicAdd(sm.ctl, mine);
+  auto window = [&](int g, float m) {
+    if (!(m < thr))
+      for (int n = g * GS; n < min(N, g * GS + GS); ++n)
+        if (GS == 1 || !(sc[n] < thr)) {
+          atomicAdd(sm.ctl, 1);
+          sm.ctl[1] = n;
+        }
+  };
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (tid + i * kT < NG) window(tid + i * kT, head[i]);
+  for (int g = tid + 8 * kT; g < NG; g += kT) window(g, gm[g]);
   __syncthreads();
-  if (sm.ctl[0] == 1 && bi < N) return bi;  // the best is alone in the window
+  if (sm.ctl[0] == 1) {  // alone in the window: the best, or an atom that has no score
+    const int n = sm.ctl[1];
+    return sc[n] >= 0.f ? n : -1;
+  }
   // score the window's atoms as the batched path does
   const float4* r4 = reinterpret_cast<const float4*>(sm.r);
   float cs = -1.f;
@@ -224,7 +249,6 @@ __device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, cons
       ci = oi;
     }
   }
-  __syncthreads();  // every warp has read rs and ri
   if (lane == 0) {
     sm.rs[warp] = cs;
     sm.ri[warp] = ci;
@@ -241,15 +265,17 @@ __device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, cons
 
 // One step (append, residual update, stop test) of signal b with kk atoms, the residual in sm.r and
 // the support in sm.gs.sup. V: float4 slots per thread. Returns whether the signal goes on; *rn
-// becomes its ||r||. Fr: where the factor is read and its new column written in FP32.
-template <int V>
-__device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, const float* sc, int b, int kk, int S,
-                                           float eps, int eps_rel, float ynorm, int W0, int V0, float* Fr, float* rn) {
+// becomes its ||r||. The FP32 factor is in sm.gs.tri (Smax <= kTriMax) or in ws.F32. The first
+// nrow rows of the support are in sm.rows (copies in flight included); a row past them goes there
+// too if keep allows, for the next step. DICT: sm.rows is the whole dictionary.
+template <int V, int GS, bool DICT>
+__device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, const float* sc, const float* gm, const float (&head)[8], int nrow, int b, int kk, int S,
+                                           float eps, int eps_rel, float ynorm, int W0, int V0, int keep, float* rn) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int M4 = ws.Mp >> 2;
   const GroupSmem& gs = sm.gs;
   const float rprev = *rn;
-  const int ns = pick_atom(ws, sm, sc, rprev, W0, V0);
+  const int ns = pick_atom<GS>(ws, sm, sc, gm, head, rprev, W0, V0);
   if (ns < 0) {
     if (tid == 0) {
       atomicOr(ws.err, OMP_DEVERR_BAD_STATE);
@@ -257,17 +283,34 @@ __device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, co
     }
     return false;
   }
+  // the new atom's row arrives while the first warp appends
+  float4 vn[V];
+#pragma unroll
+  for (int t = 0; t < V; ++t) {
+    const int s = t * kT + tid;
+    vn[t] = s < M4 ? __ldg(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(ns) * ws.Mp) + s)
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   if (warp == 0) {
     const float* grow = ws.gram + static_cast<size_t>(ns) * ws.N;
+    const double nrm2 = __ldg(ws.norm2 + ns);
     for (int i = lane; i < kk; i += 32) gs.w[i] = __ldg(grow + gs.sup[i]);
     __syncwarp();
     double* Fg = ws.F + static_cast<size_t>(b) * ws.Fstride;
+    float* Ff = ws.F32 + static_cast<size_t>(b) * ws.Fstride;
     const int nb = (kk + 31) >> 5;
-    if (nb <= 1) append_column<1>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
-    else if (nb <= 2) append_column<2>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
-    else if (nb <= 4) append_column<4>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
-    else append_column<8>(ws, gs, Fr, Fr, Fg, kk, ns, lane);
+    float* tri = gs.tri;
+    if (ws.Smax <= kTriMax) {
+      if (nb <= 1) append_column<1, 4>(ws, gs, tri, tri, Fg, kk, ns, nrm2, lane);
+      else append_column<2, 4>(ws, gs, tri, tri, Fg, kk, ns, nrm2, lane);
+    } else {
+      if (nb <= 1) append_column<1, 4>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+      else if (nb <= 2) append_column<2, 4>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+      else if (nb <= 4) append_column<4, 2>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+      else append_column<8>(ws, gs, Ff, Ff, Fg, kk, ns, nrm2, lane);
+    }
   }
+  cp_async_wait_all();  // the rows this thread copied
   __syncthreads();
   if (gs.scal[1]) {
     if (tid == 0) {
@@ -276,35 +319,56 @@ __device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, co
     }
     return false;
   }
-  // q = A_S f: thread's slots tid + 256 t, the rows in order, four rows in flight
+  // q = A_S f: thread's slots tid + 256 t, the rows in order -- from shared memory, the rest (a
+  // support longer than sm.rows) R rows in flight, the new one last
   float4 q[V];
 #pragma unroll
   for (int t = 0; t < V; ++t) q[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add_row = [&](float f, int t, const float4& v) {
+    q[t].x = fmaf(f, v.x, q[t].x);
+    q[t].y = fmaf(f, v.y, q[t].y);
+    q[t].z = fmaf(f, v.z, q[t].z);
+    q[t].w = fmaf(f, v.w, q[t].w);
+  };
+#pragma unroll(V == 1 ? 4 : 1)
+  for (int a = 0; a < (DICT ? kk : nrow); ++a) {
+    const float f = gs.f[a];
+    const float4* row = reinterpret_cast<const float4*>(sm.rows) + (DICT ? gs.sup[a] : a) * M4;
+#pragma unroll
+    for (int t = 0; t < V; ++t) {
+      const int s = t * kT + tid;
+      add_row(f, t, s < M4 ? row[s] : make_float4(0.f, 0.f, 0.f, 0.f));
+    }
+  }
   constexpr int R = V <= 2 ? 8 : V <= 4 ? 4 : 2;
-  for (int a0 = 0; a0 <= kk; a0 += R) {
+  for (int a0 = DICT ? kk : nrow; a0 < kk; a0 += R) {
     float4 v[R][V];
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       const int a = a0 + i;
-      const float4* row = reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(a <= kk ? gs.sup[a] : ns) * ws.Mp);
+      const float4* row = reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(gs.sup[min(a, kk - 1)]) * ws.Mp);
 #pragma unroll
       for (int t = 0; t < V; ++t) {
         const int s = t * kT + tid;
-        v[i][t] = a <= kk && s < M4 ? __ldg(row + s) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[i][t] = a < kk && s < M4 ? __ldg(row + s) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-      if (a0 + i <= kk) {
+      if (a0 + i < kk) {
         const float f = gs.f[a0 + i];
 #pragma unroll
-        for (int t = 0; t < V; ++t) {
-          q[t].x = fmaf(f, v[i][t].x, q[t].x);
-          q[t].y = fmaf(f, v[i][t].y, q[t].y);
-          q[t].z = fmaf(f, v[i][t].z, q[t].z);
-          q[t].w = fmaf(f, v[i][t].w, q[t].w);
-        }
+        for (int t = 0; t < V; ++t) add_row(f, t, v[i][t]);
       }
+    }
+  }
+  {
+    const float f = gs.f[kk];
+#pragma unroll
+    for (int t = 0; t < V; ++t) {
+      const int s = t * kT + tid;
+      add_row(f, t, vn[t]);
+      if (!DICT && kk < keep && s < M4) reinterpret_cast<float4*>(sm.rows + static_cast<size_t>(kk) * ws.Mp)[s] = vn[t];
     }
   }
   float4* r4 = reinterpret_cast<float4*>(sm.r);
@@ -315,7 +379,7 @@ __device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, co
     r[t] = s < M4 ? r4[s] : make_float4(0.f, 0.f, 0.f, 0.f);
     if (s < M4) sm.P[s] = dot4(q[t], r[t], V0);
   }
-  const float bf = ordered_sum(sm, M4, W0, V0);
+  const float bf = ordered_sum(sm, sm.part, M4, W0, V0);
 #pragma unroll
   for (int t = 0; t < V; ++t) {
     const int s = t * kT + tid;
@@ -328,7 +392,7 @@ __device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, co
       sm.P[s] = slot_dot<false>(r[t], r[t]);
     }
   }
-  const float rk = sqrtf(ordered_sum(sm, M4, W0, V0));
+  const float rk = sqrtf(ordered_sum(sm, sm.part + 8, M4, W0, V0));
   *rn = rk;
   const float thr = eps_rel ? eps * ynorm : eps;
   const bool hit = rk <= thr, last = kk + 1 >= S;
@@ -347,64 +411,81 @@ __device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, co
   return !(hit || last);
 }
 
-// Scores of atoms [n_lo, n_hi) for one residual in shared memory, LPA lanes per atom (16 when a row
-// has 64 elements), the warp's atoms n_lo + warp index, ...; U atoms in flight per lane group.
-template <int LPA, int U>
-__device__ __forceinline__ void score_atoms(const Ws& ws, const float4* r4, int first, int stride, float* sc) {
+// Scores of every atom for one residual in shared memory, LPA lanes per atom (16 when a row has 64
+// elements), U atoms in flight per lane group; warp `first` of `stride` takes every stride-th group.
+// With gm, the largest score of each U consecutive atoms too (LPA 32; a NaN if one is).
+template <int LPA, int U, bool SH>
+__device__ __forceinline__ void score_atoms(const Ws& ws, const float4* rows, const float4* r4, int first, int stride,
+                                            float* sc, float* gm = nullptr) {
   const int lane = threadIdx.x & 31, sub = lane % LPA, grp = lane / LPA;
   constexpr int GP = 32 / LPA;  // atoms a warp takes side by side
   const int M4 = ws.Mp >> 2, N = ws.N;
   for (int n0 = first * GP * U; n0 < N; n0 += stride * GP * U) {
-    float acc[U];
+    float acc[U], inv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) acc[u] = 0.f;
-#pragma unroll 2
+    for (int u = 0; u < U; ++u) {
+      acc[u] = 0.f;
+      const int n = n0 + u * GP + grp;
+      inv[u] = n < N ? __ldg(ws.inv_norm + n) : 0.f;
+    }
+#pragma unroll 4
     for (int s = sub; s < M4; s += LPA) {
       const float4 y = r4[s];
       float4 x[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int n = n0 + u * GP + grp;
-        x[u] = n < N ? __ldg(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp) + s)
-                     : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int n = min(n0 + u * GP + grp, N - 1);
+        x[u] = SH ? rows[n * M4 + s] : __ldg(rows + static_cast<size_t>(n) * M4 + s);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
         acc[u] = fmaf(x[u].w, y.w, fmaf(x[u].z, y.z, fmaf(x[u].y, y.y, fmaf(x[u].x, y.x, acc[u]))));
     }
+    float best = -1.f;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
 #pragma unroll
       for (int o = LPA / 2; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
       const int n = n0 + u * GP + grp;
-      if (sub == 0 && n < N) sc[n] = approx_score(acc[u], __ldg(ws.inv_norm + n));
+      const float v = approx_score(acc[u], inv[u]);
+      if (n < N) best = v >= best ? v : best > v ? best : v;  // a NaN stays
+      if (sub == 0 && n < N) sc[n] = v;
     }
+    if (gm && lane == 0) gm[n0 / U] = best;
   }
 }
 
 // Every step of one signal per block.
-template <int V>
-__global__ void __launch_bounds__(kT, 2) solo_kernel(Ws ws, int S, float eps, int eps_rel, int W0, int V0) {
+// DICT: the dictionary fits in shared memory beside the rest; every step then reads it there.
+template <int V, bool DICT>
+__global__ void __launch_bounds__(kT, 2) solo_kernel(Ws ws, int S, float eps, int eps_rel, int W0, int V0, int RC) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int b = blockIdx.x;
+  const int b = blockIdx.x, M4 = ws.Mp >> 2;
   if (!ws.flag[b]) return;  // y == 0 or non-finite
-  SmallSmem sm = small_smem(smem, ws.Mp, ws.Smax, ws.N);
+  SmallSmem sm = small_smem(smem, ws.Mp, ws.Smax, ws.N, RC);
+  const float4* A4 = reinterpret_cast<const float4*>(ws.A32);
+  float4* rows4 = reinterpret_cast<float4*>(sm.rows);
+  const float4* r4 = reinterpret_cast<const float4*>(sm.r);
+  if (DICT)
+    for (int i = tid; i < ws.N * M4; i += kT) cp_async16(rows4 + i, A4 + i);
   const float4* rg = reinterpret_cast<const float4*>(ws.R32 + static_cast<size_t>(b) * ws.Mp);
-  for (int s = tid; s < (ws.Mp >> 2); s += kT) reinterpret_cast<float4*>(sm.r)[s] = rg[s];
-  float* Fr = ws.Smax <= kTriMax ? sm.gs.tri : ws.F32 + static_cast<size_t>(b) * ws.Fstride;
+  for (int s = tid; s < M4; s += kT) reinterpret_cast<float4*>(sm.r)[s] = rg[s];
   const float ynorm = ws.ynorm[b];
   float rn = ws.rnorm[b];
   bool go = true;
+  cp_async_wait_all();
   for (int kk = 0; go; ++kk) {
     __syncthreads();  // the residual is complete, and every read of the last step's scores is done
-    const float4* r4 = reinterpret_cast<const float4*>(sm.r);
     if (ws.Mp == 64)
-      score_atoms<16, 8>(ws, r4, warp, kWarps, sm.sc);
+      score_atoms<16, DICT ? 4 : 8, DICT>(ws, DICT ? rows4 : A4, r4, warp, kWarps, sm.sc);
     else
-      score_atoms<32, 8>(ws, r4, warp, kWarps, sm.sc);
+      score_atoms<32, 4, DICT>(ws, DICT ? rows4 : A4, r4, warp, kWarps, sm.sc);
     __syncthreads();
-    go = small_step<V>(ws, sm, sm.sc, b, kk, S, eps, eps_rel, ynorm, W0, V0, Fr, &rn);
+    float head[8];
+    load_head(head, sm.sc, ws.N);
+    go = small_step<V, 1, DICT>(ws, sm, sm.sc, sm.sc, head, min(kk, RC), b, kk, S, eps, eps_rel, ynorm, W0, V0, RC,
+                                &rn);
   }
 }
 
@@ -415,6 +496,7 @@ __global__ void __launch_bounds__(kT) wide_score_kernel(Ws ws, int B) {
   float4* rs = reinterpret_cast<float4*>(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int M4 = ws.Mp >> 2, N = ws.N;
+  const size_t NP = score_pitch(N);
   __shared__ int act[kSmallMaxB], na_s;  // the signals that go on
   if (tid == 0) {
     int n = 0;
@@ -432,13 +514,10 @@ __global__ void __launch_bounds__(kT) wide_score_kernel(Ws ws, int B) {
   __syncthreads();
   if (na == 1) {
     const int first = blockIdx.x * kWarps + warp, stride = gridDim.x * kWarps;
-    if (ws.Mp == 64)
-      score_atoms<16, 4>(ws, rs, first, stride, ws.score + static_cast<size_t>(act[0]) * N);
-    else
-      score_atoms<32, 4>(ws, rs, first, stride, ws.score + static_cast<size_t>(act[0]) * N);
+    score_atoms<32, kGS, false>(ws, reinterpret_cast<const float4*>(ws.A32), rs, first, stride, ws.score + static_cast<size_t>(act[0]) * NP, ws.score + static_cast<size_t>(act[0]) * NP + N);
     return;
   }
-  constexpr int U = 2;
+  constexpr int U = kGS;
   for (int n0 = (blockIdx.x * kWarps + warp) * U; n0 < N; n0 += gridDim.x * kWarps * U) {
     float acc[U][kSmallMaxB];
 #pragma unroll
@@ -461,15 +540,21 @@ __global__ void __launch_bounds__(kT) wide_score_kernel(Ws ws, int B) {
         }
       }
     }
+    float inv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const float inv = n0 + u < N ? __ldg(ws.inv_norm + n0 + u) : 0.f;
+    for (int u = 0; u < U; ++u) inv[u] = n0 + u < N ? __ldg(ws.inv_norm + n0 + u) : 0.f;
 #pragma unroll
-      for (int i = 0; i < kSmallMaxB; ++i) {
-        if (i < na) {
-          const float d = warp_sum_f(acc[u][i]);
-          if (lane == 0 && n0 + u < N) ws.score[static_cast<size_t>(act[i]) * N + n0 + u] = approx_score(d, inv);
+    for (int i = 0; i < kSmallMaxB; ++i) {
+      if (i < na) {
+        float* sc = ws.score + static_cast<size_t>(act[i]) * NP;
+        float best = -1.f;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float v = approx_score(warp_sum_f(acc[u][i]), inv[u]);
+          if (n0 + u < N) best = v >= best ? v : best > v ? best : v;  // a NaN stays
+          if (lane == 0 && n0 + u < N) sc[n0 + u] = v;
         }
+        if (lane == 0) sc[N + n0 / U] = best;
       }
     }
   }
@@ -477,27 +562,48 @@ __global__ void __launch_bounds__(kT) wide_score_kernel(Ws ws, int B) {
 
 // One step of each signal from the scores in ws.score
 template <int V>
-__global__ void __launch_bounds__(kT, 1) wide_step_kernel(Ws ws, int S, float eps, int eps_rel, int W0, int V0) {
+__global__ void __launch_bounds__(kT, 1) wide_step_kernel(Ws ws, int S, float eps, int eps_rel, int W0, int V0,
+                                                          int RC) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x;
   const int b = blockIdx.x;
-  if (!ws.flag[b]) return;
-  SmallSmem sm = small_smem(smem, ws.Mp, ws.Smax, 0);
-  const int kk = ws.niter[b];
+  const int flag = ws.flag[b], kk = ws.niter[b];
+  float rn = ws.rnorm[b];
+  const float ynorm = ws.ynorm[b];
+  if (!flag) return;
+  // the scores' maxima first: what follows queues behind them
+  const float* sc = ws.score + static_cast<size_t>(b) * score_pitch(ws.N);
+  float head[8];
+  load_head(head, sc + ws.N, (ws.N + kGS - 1) / kGS);
+  SmallSmem sm = small_smem(smem, ws.Mp, ws.Smax, 0, RC);
+  const int M4 = ws.Mp >> 2;
   float4* rg = reinterpret_cast<float4*>(ws.R32 + static_cast<size_t>(b) * ws.Mp);
-  for (int s = tid; s < (ws.Mp >> 2); s += kT) reinterpret_cast<float4*>(sm.r)[s] = rg[s];
+  for (int s = tid; s < M4; s += kT) cp_async16(reinterpret_cast<float4*>(sm.r) + s, rg + s);
   float* Ff = ws.F32 + static_cast<size_t>(b) * ws.Fstride;
   const bool staged = ws.Smax <= kTriMax;
   if (staged)
-    for (int i = tid; i < kk * (kk + 1) / 2; i += kT) sm.gs.tri[i] = Ff[i];
-  for (int i = tid; i < kk; i += kT) sm.gs.sup[i] = ws.sup[static_cast<size_t>(b) * ws.Smax + i];
-  float rn = ws.rnorm[b];
-  const float ynorm = ws.ynorm[b];
-  __syncthreads();
-  const bool go = small_step<V>(ws, sm, ws.score + static_cast<size_t>(b) * ws.N, b, kk, S, eps, eps_rel, ynorm, W0, V0,
-                                staged ? sm.gs.tri : Ff, &rn);
+    for (int i = tid; i < (kk * (kk + 1) / 2 + 3) / 4; i += kT) cp_async16(sm.gs.tri + 4 * i, Ff + 4 * i);
+  const int* sup = ws.sup + static_cast<size_t>(b) * ws.Smax;
+  for (int i = tid; i < kk; i += kT) cp_async4(sm.gs.sup + i, sup + i);
+  cp_async_commit();
+  // the support's rows land while the block picks and appends
+  const int nrow = min(kk, RC);
+#pragma unroll 8
+  for (int a = 0; a < nrow; ++a) {
+    const float4* row = reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(sup[a]) * ws.Mp);
+#pragma unroll
+    for (int t = 0; t < V; ++t) {
+      const int s = t * kT + tid;
+      if (s < M4) cp_async16(reinterpret_cast<float4*>(sm.rows + static_cast<size_t>(a) * ws.Mp) + s, row + s);
+    }
+  }
+  cp_async_commit();
+  cp_async_wait_one();  // all but the rows; pick_atom's barriers publish them
+  const bool go = small_step<V, kGS, false>(ws, sm, sc, sc + ws.N, head, nrow, b, kk, S, eps, eps_rel, ynorm, W0, V0, 0,
+                                     &rn);
+  cp_async_wait_all();
   if (!go) return;
-  for (int s = tid; s < (ws.Mp >> 2); s += kT) rg[s] = reinterpret_cast<float4*>(sm.r)[s];
+  for (int s = tid; s < M4; s += kT) rg[s] = reinterpret_cast<float4*>(sm.r)[s];
   if (staged)  // the new factor column
     for (int i = tid; i <= kk; i += kT) Ff[kk * (kk + 1) / 2 + i] = sm.gs.tri[kk * (kk + 1) / 2 + i];
 }
@@ -526,7 +632,7 @@ int small_form(const Ws& ws, int B) {
   if (ws.prec == OMP_PREC_FP8_E4M3 || ws.A24h || ws.margin) return 0;
   if (ws.prec == OMP_PREC_BF16 && (ws.topk != kMaxTopk || !(ws.rescore_eps > 0.f))) return 0;
   const int64_t elems = static_cast<int64_t>(ws.N) * ws.Mp;
-  if (elems <= kSoloMaxElems && elems * B <= kSoloMaxTotal && small_bytes(ws.Mp, ws.Smax, ws.N) <= kSmallMaxSmem)
+  if (elems <= kSoloMaxElems && elems * B <= kSoloMaxTotal && small_bytes(ws.Mp, ws.Smax, ws.N, 0) <= kSmallMaxSmem)
     return 1;
   if (B <= kSmallMaxB && elems <= kWideMaxElems && static_cast<int64_t>(ws.Mp) * B <= kWideMaxRows) return 2;
   return 0;
@@ -536,34 +642,36 @@ cudaError_t configure_small(const Ws& ws) {
   cudaError_t e = cudaSuccess;
   by_slots(slots_per_thread(ws.Mp), [&](auto v) {
     constexpr int V = decltype(v)::value;
-    const size_t solo = small_bytes(ws.Mp, ws.Smax, ws.N);
-    if (solo <= kSmallMaxSmem) e = raise_smem_limit(reinterpret_cast<const void*>(solo_kernel<V>), solo);
-    if (e == cudaSuccess)
-      e = raise_smem_limit(reinterpret_cast<const void*>(wide_step_kernel<V>), small_bytes(ws.Mp, ws.Smax, 0));
+    e = raise_smem_limit(reinterpret_cast<const void*>(solo_kernel<V, false>), kSmallMaxSmem);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void*>(solo_kernel<V, true>), kSmallMaxSmem);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void*>(wide_step_kernel<V>), kWideMaxSmem);
   });
-  if (e == cudaSuccess)
-    e = raise_smem_limit(reinterpret_cast<const void*>(wide_score_kernel), kWideMaxRows * 4);
+  if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void*>(wide_score_kernel), kWideMaxRows * 4);
   return e;
 }
 
-int small_max_batch() { return kSmallMaxB; }
+size_t small_score_floats(int N, int Bmax) { return score_pitch(N) * (Bmax < kSmallMaxB ? Bmax : kSmallMaxB); }
 
 void launch_solo(const Ws& ws, int B, int S, float eps, int eps_rel, cudaStream_t s) {
+  const bool dict = small_bytes(ws.Mp, ws.Smax, ws.N, ws.N) <= kSmallMaxSmem;
+  const int rc = dict ? ws.N : row_cache(ws.Mp, ws.Smax, ws.N, kSmallMaxSmem);
+  const size_t bytes = small_bytes(ws.Mp, ws.Smax, ws.N, rc);
   by_slots(slots_per_thread(ws.Mp), [&](auto v) {
     constexpr int V = decltype(v)::value;
-    solo_kernel<V><<<B, kT, small_bytes(ws.Mp, ws.Smax, ws.N), s>>>(ws, S, eps, eps_rel, ws.upd_w,
-                                                                    update_slots(ws.Mp, ws.upd_w));
+    (dict ? solo_kernel<V, true> : solo_kernel<V, false>)<<<B, kT, bytes, s>>>(ws, S, eps, eps_rel, ws.upd_w,
+                                                                             update_slots(ws.Mp, ws.upd_w), rc);
   });
 }
 
 void launch_wide(const Ws& ws, int sms, int B, int S, float eps, int eps_rel, cudaStream_t s) {
-  const int per = kWarps * 4;
+  const int per = kWarps * kGS;
   const int blocks = (ws.N + per - 1) / per, grid = blocks < 2 * sms ? blocks : 2 * sms;
   wide_score_kernel<<<grid, kT, static_cast<size_t>(ws.Mp) * 4 * B, s>>>(ws, B);
+  const int rc = row_cache(ws.Mp, ws.Smax, 0, kWideMaxSmem);
   by_slots(slots_per_thread(ws.Mp), [&](auto v) {
     constexpr int V = decltype(v)::value;
-    wide_step_kernel<V><<<B, kT, small_bytes(ws.Mp, ws.Smax, 0), s>>>(ws, S, eps, eps_rel, ws.upd_w,
-                                                                     update_slots(ws.Mp, ws.upd_w));
+    wide_step_kernel<V><<<B, kT, small_bytes(ws.Mp, ws.Smax, 0, rc), s>>>(ws, S, eps, eps_rel, ws.upd_w,
+                                                                         update_slots(ws.Mp, ws.upd_w), rc);
   });
 }
 
