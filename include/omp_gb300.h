@@ -47,7 +47,9 @@ typedef enum {
 } omp_status;
 
 typedef enum {
-  OMP_PREC_FP32 = 0,     /* correlation A^T R in FP32 on the CUDA cores, fused top-1 */
+  OMP_PREC_FP32 = 0,     /* every pick decided by FP32 scores on the CUDA cores, top-1 (large batches
+                            score in FP32 only the atoms that a rigorous bound on BF16 tensor-core
+                            scores leaves, which picks the same atoms) */
   OMP_PREC_BF16 = 1,     /* BF16 tensor-core correlation, FP32 accumulate, top-8 rescored in FP32 */
   OMP_PREC_FP8_E4M3 = 2  /* E4M3 tensor-core correlation with per-atom and per-signal scales,
                             FP32 accumulate, top-8 rescored in FP32 */

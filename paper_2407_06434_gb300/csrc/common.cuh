@@ -27,7 +27,7 @@
 //     cand1[Bmax]    FP32 path: packed (score, ~index) key, merged with atomicMax
 //     cand2[Bmax]    FP32 path, margins recorded: the runner-up's key (every key that loses a
 //                    merge, and each tile's own second best, is merged into it)
-//     cand_s/cand_i  quantised paths: per position, candidate pieces x 8 (score, index)
+//     cand_s/cand_i  quantised paths and the FP32 path's filter: per position, candidate pieces x 8 (score, index)
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -59,6 +59,9 @@ struct alignas(16) TauRec {
 struct Ws {
   int M, Mp, N, Smax, Bmax, Bpad;
   int prec;        // omp_precision
+  int filt;        // FP32 path: BF16 tensor-core scores and a bound leave the few atoms that FP32
+                   // scores decide between (filter.cu); 0: every atom scored in FP32
+  int tcprec;      // what the tensor-core correlation multiplies (BF16 or E4M3)
   int topk;        // candidates rescored per signal (1 for FP32)
   int pieces;      // candidate slots per position (quantised paths)
   int tc_grid;     // tensor-core correlation: persistent grid size
@@ -98,6 +101,8 @@ struct Ws {
   float* tau_pos;  // the same per live position of the current step (0: no pruning); or null
   float* win_pos;  // per live position: three score error bounds at the row's residual (the
                    // window below the row's running best outside which columns are pruned)
+  int* ovf;        // FP32 path: positions that need every atom scored in FP32, and their
+  int* ovf_cnt;    // number per iteration (Smax + 1)
   uint8_t* flag;
   unsigned long long* cand1;
   float* cand_s;
@@ -254,6 +259,8 @@ cudaError_t raise_smem_limit(const void* kernel, size_t bytes);
 void launch_prep(const Ws& ws, const float* A, cudaStream_t s);
 void launch_gram_simt(const Ws& ws, cudaStream_t s);
 void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s);
+void launch_corr_overflow(const Ws& ws, int k, cudaStream_t s);
+void launch_filter_select(const Ws& ws, int k, int B, cudaStream_t s);
 void launch_c0_simt(const Ws& ws, int B, cudaStream_t s);
 cudaError_t configure_corr_simt(const Ws& ws);
 cudaError_t configure_c0_simt();

@@ -27,7 +27,7 @@
 namespace ompk {
 
 namespace {
-constexpr int kCorrelate = 0, kGram = 1, kStoreC = 2;
+constexpr int kCorrelate = 0, kGram = 1, kStoreC = 2, kOverflow = 3;
 
 // Two FP32 FMAs in one instruction (each rounded as fmaf): d.lo += x.lo a.lo, d.hi += x.hi a.hi
 __device__ __forceinline__ void ffma2(unsigned long long& d, unsigned long long x, unsigned long long a) {
@@ -45,10 +45,9 @@ __device__ __forceinline__ unsigned long long dup2(float x) {
 constexpr int BM = 128, BK = 32;
 constexpr int TX = 8, THREADS = 128;  // threads along the atoms; 16 along the rows, 8 rows each
 
-// MODE kCorrelate: k is the iteration; kGram: k unused; kStoreC: k is the number of signals.
-// TN atoms per thread: a tile of 128 rows x 8 TN atoms.
+// One tile: rows by * 128 .., atoms bx * 8 TN ..; L rows in all
 template <int MODE, int TN>
-__global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
+__device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, const int* live, const int* ovf) {
   constexpr bool GRAM = MODE == kGram;
   constexpr int BN = TX * TN;
   constexpr int RS = THREADS / (BK / 4);             // rows apart of a thread's loads (16)
@@ -57,25 +56,8 @@ __global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
   float* Xs = smem_f;                // 2 x BK x BM
   float* As = smem_f + 2 * BK * BM;  // 2 x BK x BN
   const int tid = threadIdx.x;
-  int bx = blockIdx.x, by = blockIdx.y;
-  // G is symmetric and every entry's products and sums are the same in both orders, so only tiles
-  // that reach the diagonal or lie above it are computed, and each stores its mirror image too
-  if (GRAM && bx * BN + BN <= by * BM) return;
   const int n0 = bx * BN;
   const int p0 = by * BM;
-  int L;
-  const int* live = nullptr;
-  if (GRAM) {
-    L = ws.N;
-  } else if (MODE == kStoreC) {
-    L = k;
-  } else {
-    k = iter_of(ws, k);
-    L = ws.cnt[k + 1];
-    live = ws.live[k & 1];
-  }
-  if (p0 >= L) return;
-
   // a warp loads 4 rows x 128 bytes (whole lines); element (k, r) of a chunk is stored at column
   // r ^ 4 ((k / 4) % 8) of its row k, so that the transposed stores of a warp meet every bank once
   // and four consecutive rows stay one aligned float4
@@ -85,7 +67,7 @@ __global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
 #pragma unroll
   for (int i = 0; i < 2 * LX; ++i) {
     const int p = p0 + lrow + RS * i;
-    const int row = p < L ? ((GRAM || MODE == kStoreC) ? p : live[p]) : -1;
+    const int row = p >= L ? -1 : (GRAM || MODE == kStoreC) ? p : live[MODE == kOverflow ? ovf[p] : p];
     xsrc[i] = row < 0 ? nullptr : (GRAM ? ws.A32 : ws.R32) + static_cast<size_t>(row) * ws.Mp + 4 * lq;
   }
 #pragma unroll
@@ -217,7 +199,7 @@ __global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
   float inv[TN];
 #pragma unroll
   for (int j = 0; j < TN; ++j) inv[j] = ncol(j) < ws.N ? __ldg(ws.inv_norm + ncol(j)) : 0.f;
-  if (ws.cand2) {
+  if (MODE == kCorrelate && ws.cand2) {
     // Margins recorded: each row's best two atoms of the tile (same scan and ties), then
     // cand1 keeps the global best as before and cand2 receives every key that loses a merge
     // (the smaller of the old and the new key of each atomicMax) and each tile's second best,
@@ -295,8 +277,45 @@ __global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
         bidx = oi;
       }
     }
-    if (tx == 0 && prow < L && bidx < ws.N) atomicMax(ws.cand1 + prow, pack_key(best, bidx));
+    if (tx == 0 && prow < L && bidx < ws.N)
+      atomicMax(ws.cand1 + (MODE == kOverflow ? ovf[prow] : prow), pack_key(best, bidx));
   }
+}
+
+// MODE kCorrelate: k is the iteration; kGram: k unused; kStoreC: k is the number of signals;
+// kOverflow: as kCorrelate for the positions that the filter could not decide (a launch of one row of
+// tiles, walked down).
+// TN atoms per thread: a tile of 128 rows x 8 TN atoms.
+template <int MODE, int TN>
+__global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
+  constexpr bool GRAM = MODE == kGram;
+  constexpr int BN = TX * TN;
+  const int bx = blockIdx.x, by = blockIdx.y;
+  // G is symmetric and every entry's products and sums are the same in both orders, so only tiles
+  // that reach the diagonal or lie above it are computed, and each stores its mirror image too
+  if (GRAM && bx * BN + BN <= by * BM) return;
+  int L;
+  const int* live = nullptr;
+  const int* ovf = nullptr;
+  if (GRAM) {
+    L = ws.N;
+  } else if (MODE == kStoreC) {
+    L = k;
+  } else {
+    k = iter_of(ws, k);
+    L = MODE == kOverflow ? ws.ovf_cnt[k] : ws.cnt[k + 1];
+    live = ws.live[k & 1];
+    ovf = ws.ovf;
+  }
+  if (MODE == kOverflow) {
+    for (int r = 0; r * BM < L; ++r) {
+      simt_tile<MODE, TN>(ws, bx, r, L, live, ovf);
+      __syncthreads();  // the next tile overwrites the chunks
+    }
+    return;
+  }
+  if (by * BM >= L) return;
+  simt_tile<MODE, TN>(ws, bx, by, L, live, ovf);
 }
 
 template <int TN>
@@ -356,11 +375,18 @@ cudaError_t set_tile_limits() {
 cudaError_t configure_corr_simt(const Ws& ws) {
   cudaError_t e = set_tile_limits<kGram>();
   if (e == cudaSuccess && ws.prec == OMP_PREC_FP32) e = set_tile_limits<kCorrelate>();
+  if (e == cudaSuccess && ws.filt)
+    e = raise_smem_limit(reinterpret_cast<const void*>(simt_tile_kernel<kOverflow, 8>), tile_bytes<8>());
   return e;
 }
 cudaError_t configure_c0_simt() { return set_tile_limits<kStoreC>(); }
 
 void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s) { launch_tiles<kCorrelate>(ws, B, k, s); }
+
+// Mostly no position is left over: one narrow row of tiles that returns at once
+void launch_corr_overflow(const Ws& ws, int k, cudaStream_t s) {
+  simt_tile_kernel<kOverflow, 8><<<(ws.N + 8 * TX - 1) / (8 * TX), THREADS, tile_bytes<8>(), s>>>(ws, k);
+}
 
 void launch_c0_simt(const Ws& ws, int B, cudaStream_t s) { launch_tiles<kStoreC>(ws, B, B, s); }
 

@@ -355,11 +355,11 @@ cudaError_t tc_setup(const Ws& ws, int sm_count, TcPlan** plan) {
   *plan = nullptr;
   TcPlan* p = new TcPlan();
   p->grid = sm_count;
-  const void* a = ws.prec == OMP_PREC_BF16 ? static_cast<const void*>(ws.A16) : static_cast<const void*>(ws.A8);
-  const bool ok = make_kmajor_map(&p->r0, ws.Rq[0], ws.prec, ws.Bpad, ws.Mp, BM) &&
-                  make_kmajor_map(&p->r1, ws.Rq[1], ws.prec, ws.Bpad, ws.Mp, BM) &&
-                  make_kmajor_map(&p->a[0], a, ws.prec, ws.N, ws.Mp, BN) &&
-                  make_kmajor_map(&p->a[1], a, ws.prec, ws.N, ws.Mp, BN / 2);
+  const void* a = ws.tcprec == OMP_PREC_BF16 ? static_cast<const void*>(ws.A16) : static_cast<const void*>(ws.A8);
+  const bool ok = make_kmajor_map(&p->r0, ws.Rq[0], ws.tcprec, ws.Bpad, ws.Mp, BM) &&
+                  make_kmajor_map(&p->r1, ws.Rq[1], ws.tcprec, ws.Bpad, ws.Mp, BM) &&
+                  make_kmajor_map(&p->a[0], a, ws.tcprec, ws.N, ws.Mp, BN) &&
+                  make_kmajor_map(&p->a[1], a, ws.tcprec, ws.N, ws.Mp, BN / 2);
   if (!ok) {
     delete p;
     return cudaErrorNotSupported;
@@ -427,7 +427,7 @@ void launch_corr_tc(const Ws& ws, const TcPlan* plan, int k, int B, cudaStream_t
   const CUtensorMap* am = &plan->a[cl_index(cl)];
   void* args[] = {const_cast<CUtensorMap*>(r0), const_cast<CUtensorMap*>(r1), const_cast<CUtensorMap*>(am),
                   const_cast<Ws*>(&ws), &k};
-  const void* kernel = kern_of(ws.prec, ws.tc_stages, cl);
+  const void* kernel = kern_of(ws.tcprec, ws.tc_stages, cl);
   if (kernel && ws.tc_grid % cl == 0) cudaLaunchKernelExC(&cfg, kernel, args);  // else: no shape
 }
 

@@ -48,7 +48,15 @@ __global__ void __launch_bounds__(256) prep_kernel(Ws ws, const float* __restric
     // e2: squared norm of the quantisation error of the atom as the correlation sees it (the E4M3
     // code times the atom's scale), for the data-driven score bound of the E4M3 path
     double e2 = 0.0;
-    if (ws.prec == OMP_PREC_BF16) {
+    if (ws.filt) {
+      __nv_bfloat16* a16 = ws.A16 + static_cast<size_t>(n) * ws.Mp;
+      for (int m = lane; m < ws.Mp; m += 32) {
+        const __nv_bfloat16 c = __float2bfloat16_rn(a32[m]);
+        a16[m] = c;
+        const float d = __bfloat162float(c) - a32[m];  // exact
+        e2 += static_cast<double>(d) * d;
+      }
+    } else if (ws.prec == OMP_PREC_BF16) {
       __nv_bfloat16* a16 = ws.A16 + static_cast<size_t>(n) * ws.Mp;
       for (int m = lane; m < ws.Mp; m += 32) a16[m] = __float2bfloat16_rn(a32[m]);
     } else if (ws.prec == OMP_PREC_FP8_E4M3) {
@@ -65,7 +73,11 @@ __global__ void __launch_bounds__(256) prep_kernel(Ws ws, const float* __restric
     }
     if (ws.ea) {
       e2 = warp_sum(e2);
-      if (lane == 0 && s > 0.0) {
+      if (ws.filt && lane == 0 && s != 0.0 && !(s > 1e-24 && s < 1e24)) {
+        // products with such an atom (or one that is not finite) may leave FP32's normal range, so no
+        // bound holds: every atom is scored in FP32
+        atomicMax(reinterpret_cast<unsigned int*>(ws.ea), 0x7f800000u);
+      } else if (lane == 0 && s > 0.0) {
         const float rel = static_cast<float>(sqrt(e2 / s)) * (1.f + 0x1p-20f);
         atomicMax(reinterpret_cast<unsigned int*>(ws.ea), __float_as_uint(rel));
       }

@@ -110,18 +110,34 @@ omp_status check_launch() {
 }
 
 void enqueue_correlate(omp_handle_s* h, const Ws& ws, int k, int B, cudaStream_t s) {
-  if (ws.prec == OMP_PREC_FP32)
+  if (ws.prec == OMP_PREC_FP32 && !ws.filt) {
     launch_corr_simt(ws, k, B, s);
-  else
-    launch_corr_tc(ws, h->tc, k, B, s);
+    return;
+  }
+  launch_corr_tc(ws, h->tc, k, B, s);
+  if (ws.filt) {
+    launch_filter_select(ws, k, B, s);
+    launch_corr_overflow(ws, k, s);
+  }
+}
+
+// FP32 path: every atom scored in FP32
+void no_filter(Ws& w) {
+  w.filt = 0;
+  w.tcprec = w.prec;
 }
 
 // The workspace view a solve runs with: the handle's own, or -- when the caller asks for each
 // step's top-two margin -- one whose kernels record it: the FP32 correlation also merges the
 // runner-up's key, and the quantised paths run without the score bound (every candidate
 // rescored in FP32, no pruning), which picks the same atoms (the exactness tests compare the two).
-Ws solve_ws(const omp_handle_s* h, bool stats) {
+Ws solve_ws(const omp_handle_s* h, int B, bool stats) {
   Ws w = h->ws;
+  // The FP32 path's filter pays from about 3e8 products a step on, and for rows of 256 elements and
+  // more always: the tile kernel then takes a chain of that many products at least. Measured, us a
+  // step with and without: 64 x 256, 2000 signals 29 / 22; 128 x 512, 2000 29 / 25; 100 x 8000, 500
+  // 35 / 42; 256 x 1024, 1000 29 / 30; 512 x 2048, 16 28 / 41; 256 x 1024, 5000 43 / 79.
+  if (w.filt && (stats || (w.Mp < 256 && static_cast<double>(w.N) * w.Mp * B < 3e8))) no_filter(w);
   if (stats) {
     w.margin = h->margin_buf;
     w.cand2 = w.prec == OMP_PREC_FP32 ? h->cand2_buf : nullptr;
@@ -222,10 +238,12 @@ bool capture_while_solve(omp_handle_s* h, const Ws& ws, int B, int S, float eps,
 }
 
 void enqueue_topk(omp_handle_s* h, const float* R, int B, int topk, cudaStream_t s) {
-  launch_load_rows(h->ws, R, B, s);
-  launch_compact(h->ws, 0, B, 1, false, s);
-  enqueue_correlate(h, h->ws, 0, B, s);
-  launch_topk_out(h->ws, h->args_dev, B, topk, s);
+  Ws ws = h->ws;
+  if (ws.filt) no_filter(ws);  // the score is an output
+  launch_load_rows(ws, R, B, s);
+  launch_compact(ws, 0, B, 1, false, s);
+  enqueue_correlate(h, ws, 0, B, s);
+  launch_topk_out(ws, h->args_dev, B, topk, s);
 }
 
 omp_status prepare(omp_handle_s* h, const float* A, cudaStream_t s) {
@@ -241,7 +259,7 @@ omp_status run_solve(omp_handle_s* h, int B, int S, float eps, bool stats, cudaS
   const bool prof = h->prof_on;
   h->prof_last_S = S;
   h->prof_last_valid = prof;
-  const Ws ws = solve_ws(h, stats);
+  const Ws ws = solve_ws(h, B, stats);
   if (!h->d.use_graph) {
     if (prof || !enqueue_small(h, ws, B, S, eps, stream)) enqueue_solve(h, ws, B, S, eps, prof, stream);
     return check_launch();
@@ -400,21 +418,27 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   // padded to 4 entries so each signal's FP32 factor starts on a 16-byte boundary
   ws.Fstride = (static_cast<int64_t>(ws.Smax) * (ws.Smax + 1) / 2 + 3) / 4 * 4;
   ws.upd_w = update_default_warps(ws.Mp);
-  ws.pieces = d.precision == OMP_PREC_FP32 ? 0 : tc_pieces();
+  // The FP32 path filters its atoms with a BF16 correlation. (The test hook that turns the score
+  // bound off turns this off too.)
+  const bool hook = always && std::atoi(always) == 1;
+  ws.filt = d.precision == OMP_PREC_FP32 && !hook ? 1 : 0;
+  ws.tcprec = ws.filt ? OMP_PREC_BF16 : ws.prec;
+  const bool tc = ws.tcprec != OMP_PREC_FP32;
+  ws.pieces = tc ? tc_pieces() : 0;
   ws.tc_cl = 1;
-  if (d.precision != OMP_PREC_FP32) tc_fill_sched(ws, h->sm_count);
+  if (tc) tc_fill_sched(ws, h->sm_count);
   const size_t N = ws.N, Mp = ws.Mp, Bm = ws.Bmax, Bp = ws.Bpad, Sm = ws.Smax;
-  const size_t qbytes = d.precision == OMP_PREC_BF16 ? 2 : 1;
+  const size_t qbytes = ws.tcprec == OMP_PREC_BF16 ? 2 : 1;
   bool ok = true;
   ok = ok && dalloc(h, &ws.A32, N * Mp);
   if (d.gather24) ok = ok && dalloc(h, &ws.A24h, N * Mp) && dalloc(h, &ws.A24l, N * Mp);
-  if (d.precision == OMP_PREC_BF16) ok = ok && dalloc(h, &ws.A16, N * Mp);
+  if (ws.tcprec == OMP_PREC_BF16) ok = ok && dalloc(h, &ws.A16, N * Mp);
   if (d.precision == OMP_PREC_FP8_E4M3) ok = ok && dalloc(h, &ws.A8, N * Mp) && dalloc(h, &ws.sa, N);
   const size_t Npad = (N + 255) / 256 * 256;
-  if (d.precision != OMP_PREC_FP32) ok = ok && dalloc(h, &ws.escale, Npad);
+  if (tc) ok = ok && dalloc(h, &ws.escale, Npad);
   ok = ok && dalloc(h, &ws.inv_norm, N) && dalloc(h, &ws.norm2, N) && dalloc(h, &ws.gram, N * N);
   ok = ok && dalloc(h, &ws.R32, Bm * Mp);
-  if (d.precision != OMP_PREC_FP32) {
+  if (tc) {
     uint8_t* q0 = nullptr;
     uint8_t* q1 = nullptr;
     ok = ok && dalloc(h, &q0, Bp * Mp * qbytes) && dalloc(h, &q1, Bp * Mp * qbytes);
@@ -432,6 +456,9 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   if (want_tau && ws.rescore_eps > 0.f && ws.Smax <= kTauSmax)
     ok = ok && dalloc(h, &ws.tau, Bm) && dalloc(h, &ws.tau_pos, Bp) && dalloc(h, &ws.win_pos, Bp) &&
          (ws.prec != OMP_PREC_FP8_E4M3 || dalloc(h, &ws.ea, 1));
+  if (ws.filt)
+    ok = ok && dalloc(h, &ws.win_pos, Bp) && dalloc(h, &ws.ea, 1) && dalloc(h, &ws.ovf, Bm) &&
+         dalloc(h, &ws.ovf_cnt, Sm + 1);
   ok = ok && dalloc(h, &ws.live[0], Bm) && dalloc(h, &ws.live[1], Bm);
   ok = ok && dalloc(h, &ws.livek[0], Bm) && dalloc(h, &ws.livek[1], Bm);
   ok = ok && dalloc(h, &ws.cnt, Sm + 2) && dalloc(h, &ws.kdev, 1) && dalloc(h, &ws.flag, Bm) && dalloc(h, &ws.cand1, Bm);
@@ -463,7 +490,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
                  cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking) == cudaSuccess &&
                  configure_update_kernels(ws) == cudaSuccess && configure_corr_simt(ws) == cudaSuccess &&
                  configure_small(ws) == cudaSuccess;
-  if (cuda_ok && d.precision != OMP_PREC_FP32) cuda_ok = tc_setup(ws, h->sm_count, &h->tc) == cudaSuccess;
+  if (cuda_ok && tc) cuda_ok = tc_setup(ws, h->sm_count, &h->tc) == cudaSuccess;
   if (cuda_ok) cuda_ok = cudaDeviceSynchronize() == cudaSuccess;
   if (!cuda_ok) {
     cudaGetLastError();
@@ -629,8 +656,8 @@ omp_status solve_candidates(omp_handle h, const float* A, const float* Y, int64_
   a.resid = resid_norm_out;
   a.fallback = fallback_out;
   launch_set_args(h->args_dev, a, s);
-  const Ws& ws = h->ws;
   const int b = static_cast<int>(B);
+  const Ws ws = solve_ws(h, b, false);
   launch_init(ws, h->args_dev, b, s);
   if (p && !proposal_run_inference(p, A, Y, b, s)) return OMP_ERR_CUDA;
   if (!launch_restricted(ws, h->args_dev, cand, K, tau, b, S, eps, h->d.eps_relative, ws.fb, s))
@@ -729,7 +756,7 @@ omp_status omp_autotune(omp_handle h, const float* A, const float* Y, int64_t B,
       cudaGraph_t g = nullptr;
       bool ok = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
       if (ok) {
-        enqueue_solve(h, solve_ws(h, false), b, S, eps, false, h->cap_stream);
+        enqueue_solve(h, solve_ws(h, b, false), b, S, eps, false, h->cap_stream);
         ok = cudaStreamEndCapture(h->cap_stream, &g) == cudaSuccess && g != nullptr;
       }
       if (ok) ok = cudaGraphInstantiate(&r->exec, g, 0) == cudaSuccess;
@@ -742,7 +769,7 @@ omp_status omp_autotune(omp_handle h, const float* A, const float* Y, int64_t B,
         if (cudaGraphLaunch(r.exec, s) != cudaSuccess) failed = true;
       } else {
         apply(r.c);
-        enqueue_solve(h, solve_ws(h, false), b, S, eps, false, s);
+        enqueue_solve(h, solve_ws(h, b, false), b, S, eps, false, s);
       }
     };
     auto time_run = [&](const Run& r) {

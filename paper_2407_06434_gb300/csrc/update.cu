@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(256) init_kernel(Ws ws, const CallArgs* args, 
   if (blockIdx.x == 0 && threadIdx.x == 0) *ws.kdev = 0;
   if (blockIdx.x == 0 && ws.upd_ctr)
     for (int i = threadIdx.x; i <= ws.Smax; i += blockDim.x) ws.upd_ctr[i] = 0;
+  if (blockIdx.x == 0 && ws.filt)
+    for (int i = threadIdx.x; i <= ws.Smax; i += blockDim.x) ws.ovf_cnt[i] = 0;
   if (b >= B) return;
   const float* y = args->Y + static_cast<size_t>(b) * ws.M;
   float* r = ws.R32 + static_cast<size_t>(b) * ws.Mp;
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(256) compact_kernel(Ws ws, int j, int S, int r
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
     pnk[m] = ws.niter[pid[m]];
-    prn[m] = ws.tau_pos ? ws.rnorm[pid[m]] : 0.f;
+    prn[m] = ws.tau_pos || ws.filt ? ws.rnorm[pid[m]] : 0.f;
     ptr[m] = ws.tau_pos && j > 0 ? ws.tau[pid[m]] : TauRec{0.f, 0.f, -1, 0};
   }
   // kept flags before p0 (a multiple of 16; flags are 0 or 1 bytes, so a word's bit count is
@@ -207,7 +209,8 @@ __global__ void __launch_bounds__(256) compact_kernel(Ws ws, int j, int S, int r
       continue;
     }
     const float4* src = reinterpret_cast<const float4*>(ws.R32 + static_cast<size_t>(id) * ws.Mp);
-    if (ws.prec == OMP_PREC_BF16) {
+    if (ws.tcprec == OMP_PREC_BF16) {
+      float e2 = 0.f;  // FP32 path: squared norm of the row's rounding error
       __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(
           static_cast<__nv_bfloat16*>(ws.Rq[j & 1]) + static_cast<size_t>(dest) * ws.Mp);
       for (int m0 = 0; m0 < M4; m0 += 256) {
@@ -221,12 +224,28 @@ __global__ void __launch_bounds__(256) compact_kernel(Ws ws, int j, int S, int r
         for (int t = 0; t < 8; ++t) {
           const int m = m0 + t * 32 + lane;
           if (m < M4) {
-            dst[2 * m] = __floats2bfloat162_rn(v[t].x, v[t].y);
-            dst[2 * m + 1] = __floats2bfloat162_rn(v[t].z, v[t].w);
+            const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[t].x, v[t].y);
+            const __nv_bfloat162 h1 = __floats2bfloat162_rn(v[t].z, v[t].w);
+            dst[2 * m] = h0;
+            dst[2 * m + 1] = h1;
+            if (ws.filt) {
+              const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+              const float d0 = f0.x - v[t].x, d1 = f0.y - v[t].y, d2 = f1.x - v[t].z, d3 = f1.y - v[t].w;
+              e2 += d0 * d0 + d1 * d1 + d2 * d2 + d3 * d3;
+            }
           }
         }
       }
-    } else if (ws.prec == OMP_PREC_FP8_E4M3) {
+      if (ws.filt) {
+        // three score error bounds at this residual, from the actual rounding errors (rounded up)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+        if (lane == 0) {
+          const float rn = prn[m], er = sqrtf(e2) / rn * (1.f + 0x1p-16f);
+          ws.win_pos[dest] = 3.f * data_bound(ws, *ws.ea, er) * rn * (1.f + 0x1p-20f);
+        }
+      }
+    } else if (ws.tcprec == OMP_PREC_FP8_E4M3) {
       float amax = 0.f;
       for (int m0 = 0; m0 < M4; m0 += 256) {
         float4 v[8];

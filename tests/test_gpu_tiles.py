@@ -125,3 +125,51 @@ def test_few_signals_ties_and_extreme_scales(lib, prec):
     assert out[0][1][0, 0] == 17
     for g, want in zip(*out):
         assert np.array_equal(g.view(np.uint32), want.view(np.uint32))
+
+
+def _solve_both(lib, monkeypatch, A, Y, S, eps, graph=1, **kw):
+    """The FP32 solve with its filter and (OMP_RESCORE_ALWAYS=1 when the handle is created) without."""
+    out = []
+    for hook in ("0", "1"):
+        monkeypatch.setenv("OMP_RESCORE_ALWAYS", hook)
+        s = lib.OmpSolver(A.shape[0], A.shape[1], max_batch=Y.shape[0], max_iters=S, precision="fp32",
+                          use_graph=graph, **kw)
+        out.append([t.cpu().numpy() for t in s.solve(A, Y, S, eps, diagnostics=True)])
+        s.close()
+    return out
+
+
+# The FP32 path scores in FP32 only the atoms that a bound on the BF16 scores leaves: the same bits
+# as scoring every atom. Few and many column tiles, ragged rows, more steps than planted atoms (the
+# noise floor, where many scores are close), an eps stop that retires signals at different steps.
+@pytest.mark.parametrize("M,N,B,S,planted,eps,graph", [
+    (64, 300, 700, 12, 12, 0.0, 1), (256, 1000, 300, 40, 20, 0.0, 1), (203, 1500, 129, 24, 24, 1e-2, 1),
+    (1024, 4100, 257, 24, 16, 0.0, 1), (1024, 4100, 200, 20, 20, 1e-2, 2), (2100, 2500, 70, 16, 16, 0.0, 0),
+    (640, 8000, 1100, 8, 4, 0.0, 1)])
+def test_fp32_filter_is_exact(lib, monkeypatch, M, N, B, S, planted, eps, graph):
+    A, Y = _planted(M, N, B, planted, M + N + B)
+    Y[3] = 0.0
+    got, want = _solve_both(lib, monkeypatch, A, Y, S, eps, graph)
+    for g, w in zip(got, want):
+        assert np.array_equal(g.view(np.uint32), w.view(np.uint32))
+
+
+def test_fp32_filter_close_atoms_and_extreme_scales(lib, monkeypatch):
+    """Clusters of more nearly equal atoms than a list holds, exact duplicates, signals and atoms far
+    from unit norm, an atom of norm 0: the positions that the bound cannot decide."""
+    rng = np.random.default_rng(11)
+    A, Y = _planted(300, 2000, 400, 10, 12)
+    At = A.t().contiguous()
+    base = At[:20].repeat_interleave(40, 0)
+    noise = torch.from_numpy(rng.standard_normal(base.shape).astype(np.float32)).cuda()
+    At[1000:1800] = base + 1e-6 * noise          # 40 near copies of each of 20 atoms
+    At[1900:1950] = At[7]                        # exact duplicates
+    At[1960] = 0.0
+    Y[:100] = At[torch.from_numpy(rng.integers(0, 20, 100)).cuda()] + 1e-3 * Y[:100]
+    Y[100] *= 1e-20
+    Y[101] *= 1e18
+    for scale in (1.0, 1e17):
+        At[1970] = At[1970] / At[1970].norm() * scale
+        got, want = _solve_both(lib, monkeypatch, At.t(), Y, 10, 0.0)
+        for g, w in zip(got, want):
+            assert np.array_equal(g.view(np.uint32), w.view(np.uint32))
