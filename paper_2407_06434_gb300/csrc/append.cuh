@@ -16,7 +16,7 @@
 //                                  with the handle's 24-bit option the rows rounded to a 15-bit
 //                                  mantissa, read as 3 bytes per element)
 //   b_k   = q^T r,  r <- r - b_k q (y_hat = A_k F_k (A_k F_k)^T y built one term at a time)
-// and, with one warp per signal, the next step's quantised operand row at this position, and
+// and the next step's quantised operand row at this position, and
 // (BF16) the next correlation's pruning threshold from the exact FP32 correlation of the new
 // residual with the best candidate that was not picked.
 //
@@ -315,19 +315,11 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
 
   // The candidate lists head the critical path (merge, rescoring, append), so their loads are
   // issued first; they are only read at the merge below.
-  float vs[8];
-  int vi[8];
+  Lists l;
+  int total = 0;
   if (!top1 && wig == 0) {
-    const int total = tc_piece_count(ws, L, p) * kMaxTopk;
-    const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
-    const int* ci = ws.cand_i + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const int e = lane + 32 * t;
-      const bool ok = e < total;
-      vs[t] = ok ? cs[e] : -1.f;
-      vi[t] = ok ? ci[e] : 0x7fffffff;
-    }
+    total = tc_piece_count(ws, L, p) * kMaxTopk;
+    load_lists(ws, total, p, lane, l);
   }
 
   // Loads that do not depend on the selection go out next. The packed FP32 factor (so that the
@@ -373,12 +365,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     ns = key_index(ws.cand1[p]);
   } else {
     if (wig == 0) {
-#pragma unroll
-      for (int t = 0; t < 8; ++t)
-        if (vi[t] < 0) {  // an unfilled list entry
-          vs[t] = -1.f;
-          vi[t] = 0x7fffffff;
-        }
+      settle_lists(ws, total, p, lane, l);
       // Candidates come out best first; one more than 2 rescore_eps ||r|| below the best has an
       // FP32 score strictly below the best one's, so the rescoring stops before it. FP8 scores
       // leave out the residual's scale qs, so the window is taken in their units.
@@ -388,35 +375,9 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
       float s_first = 0.f;
       int nres = ws.topk;
       for (int sel = 0; sel < ws.topk; ++sel) {
-        float bs = -2.f;
-        int bi = 0x7fffffff, bt = -1;
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-          if (better(vs[t], vi[t], bs, bi)) {
-            bs = vs[t];
-            bi = vi[t];
-            bt = t;
-          }
-        float g_s = bs;
-        int g_i = bi;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float os = __shfl_xor_sync(0xffffffffu, g_s, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, g_i, o);
-          if (better(os, oi, g_s, g_i)) {
-            g_s = os;
-            g_i = oi;
-          }
-        }
-        if (bt >= 0 && bi == g_i && bs == g_s) {
-#pragma unroll
-          for (int t = 0; t < 8; ++t)
-            if (t == bt) {
-              vs[t] = -2.f;
-              vi[t] = 0x7fffffff;
-            }
-        }
-        if (lane == 0) gs.cidx[sel] = (g_i >= 0 && g_i < ws.N) ? g_i : -1;
+        int g_i;
+        const float g_s = take_best(l, g_i);
+        if (lane == 0) gs.cidx[sel] = g_i < ws.N ? g_i : -1;
         if (lane == 0) gs.cq[sel] = g_s;
         if (lane == 0 && sel < 2) gs.top2[sel] = g_s;
         if (sel == 0)
@@ -703,8 +664,8 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
       gs.cpart[2 * wig + 1] = d1;
     }
   }
-  float qe2 = -1.f;  // squared norm of the next row's quantisation error (W == 1; -1: not known)
-  if (W == 1 && !top1) {
+  float qe2 = -1.f;  // squared norm of the next row's quantisation error (W == 1, E4M3; -1: not known)
+  if (!top1) {
     // The next step's quantised operand row, at this position: the compaction keeps it where
     // no signal before this one retired, and re-quantises from R32 otherwise. Same rounding as
     // the compaction's (BF16 round-to-nearest-even; E4M3 satfinite with the row's amax / 448).
@@ -717,7 +678,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
           static_cast<__nv_bfloat16*>(ws.Rq[j]) + static_cast<size_t>(p) * ws.Mp);
 #pragma unroll
       for (int t = 0; t < V; ++t) {
-        const int s = t * 32 + lane;
+        const int s = t * (W * 32) + wig * 32 + lane;
         if (s < M4) {
           const __nv_bfloat162 h0 = __floats2bfloat162_rn(r[t].x, r[t].y);
           const __nv_bfloat162 h1 = __floats2bfloat162_rn(r[t].z, r[t].w);
@@ -729,18 +690,23 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
       float amax = 0.f;
 #pragma unroll
       for (int t = 0; t < V; ++t) {
-        const int s = t * 32 + lane;
+        const int s = t * (W * 32) + wig * 32 + lane;
         if (s < M4)
           amax = fmaxf(amax, fmaxf(fmaxf(fabsf(r[t].x), fabsf(r[t].y)), fmaxf(fabsf(r[t].z), fabsf(r[t].w))));
       }
       amax = warp_max(amax);
+      if (W > 1) {  // over the block's warps (gs.cpart's first 16 entries hold the threshold's parts)
+        if (lane == 0) gs.cpart[32 + wig] = amax;
+        group_sync(W, grp);
+        for (int w = 0; w < W; ++w) amax = fmaxf(amax, gs.cpart[32 + w]);
+      }
       const float inv = amax > 0.f ? 448.f / amax : 0.f;
-      if (lane == 0) ws.sr[j][p] = amax > 0.f ? amax / 448.f : 0.f;
+      if (wig == 0 && lane == 0) ws.sr[j][p] = amax > 0.f ? amax / 448.f : 0.f;
       const float sr = amax > 0.f ? amax / 448.f : 0.f;
       uint32_t* dq = reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(ws.Rq[j]) + static_cast<size_t>(p) * ws.Mp);
 #pragma unroll
       for (int t = 0; t < V; ++t) {
-        const int s = t * 32 + lane;
+        const int s = t * (W * 32) + wig * 32 + lane;
         if (s < M4) {
           const __nv_fp8_storage_t b0 = __nv_cvt_float_to_fp8(r[t].x * inv, __NV_SATFINITE, __NV_E4M3);
           const __nv_fp8_storage_t b1 = __nv_cvt_float_to_fp8(r[t].y * inv, __NV_SATFINITE, __NV_E4M3);
@@ -758,7 +724,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
         }
       }
     }
-    if (ws.prec == OMP_PREC_FP8_E4M3) qe2 = warp_sum_f(e2);
+    if (W == 1 && ws.prec == OMP_PREC_FP8_E4M3) qe2 = warp_sum_f(e2);
   }
   if (lane == 0) pf[8 + wig] = rr;
   group_sync(W, grp);

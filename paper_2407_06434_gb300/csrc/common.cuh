@@ -42,7 +42,7 @@ constexpr int kMpAlign = 64;          // M padding (x2 for E4M3): one 128-byte K
 constexpr int kSigTile = 128;         // signals per correlation tile (TMEM lanes)
 constexpr int kMaxTopk = 8;
 constexpr int kTauSmax = 64;          // the BF16 pruning threshold is kept for max_iters <= 64
-constexpr int kPieces = 32;           // candidate slots per position (quantised paths)
+constexpr int kPieces = 68;           // candidate lists per position at most (tensor-core paths)
 constexpr int kTcParts = 2;           // candidate lists per signal and correlation CTA
 constexpr double kDepRtol = 1e-10;    // dependent-atom test: delta <= 1e-10 ||a||^2
 constexpr int kStopIters = 0, kStopEps = 1, kStopDependent = 2, kStopZero = 3;
@@ -236,9 +236,12 @@ __host__ __device__ __forceinline__ void tc_sched(int L, int G, int Tn, int cmin
 __host__ __device__ __forceinline__ int tc_start(int g, int T, int Geff) {
   return static_cast<int>(static_cast<long long>(g) * T / Geff);
 }
-// the cluster whose range contains unit u
+// the cluster whose range contains unit u (32-bit division where the numbers allow: a 64-bit one costs
+// a few hundred cycles of a signal's chain)
 __host__ __device__ __forceinline__ int tc_owner(int u, int T, int Geff) {
-  return static_cast<int>((static_cast<long long>(u + 1) * Geff - 1) / T);
+  const unsigned long long n = static_cast<unsigned long long>(u + 1) * Geff - 1;
+  if (n <= 0xffffffffull) return static_cast<int>(static_cast<unsigned>(n) / static_cast<unsigned>(T));
+  return static_cast<int>(n / T);
 }
 // candidate slots [0, count) of live position p hold its signal tile's lists: kTcParts per
 // piece (one per part of the atom columns of each unit)
@@ -247,6 +250,74 @@ __device__ __forceinline__ int tc_piece_count(const Ws& ws, int L, int p) {
   tc_sched(L, ws.tc_grid, ws.tc_tn, ws.tc_cmin, ws.tc_cl, T, Geff);
   const int sg = p / kSigTile / ws.tc_cl;
   return kTcParts * (tc_owner(sg * ws.tc_tn + ws.tc_tn - 1, T, Geff) - tc_owner(sg * ws.tc_tn, T, Geff) + 1);
+}
+
+// The candidate lists of live position p, spread over a warp: 8 entries per lane, scores as ordered
+// integers (their bits plus one; 0: no entry). load_lists issues the loads of the first 256 entries,
+// settle_lists waits for them. Entries beyond 256 (a small batch's tiles are split over many CTAs)
+// replace a lane's worst: no lane can hold more than 8 of the position's best 8.
+struct Lists {
+  float s[8];
+  int i[8];
+  uint32_t k[8];
+};
+__device__ __forceinline__ void load_lists(const Ws& ws, int total, int p, int lane, Lists& l) {
+  const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
+  const int* ci = ws.cand_i + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const bool in = lane + 32 * t < total;
+    l.s[t] = in ? cs[lane + 32 * t] : 0.f;
+    l.i[t] = in ? ci[lane + 32 * t] : -1;
+  }
+}
+__device__ __forceinline__ void settle_lists(const Ws& ws, int total, int p, int lane, Lists& l) {
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const bool ok = l.i[t] >= 0;  // an unfilled list entry is -1
+    l.k[t] = ok ? __float_as_uint(l.s[t]) + 1u : 0u;  // scores are >= 0
+    if (!ok) l.i[t] = 0x7fffffff;
+  }
+  const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
+  const int* ci = ws.cand_i + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
+#pragma unroll 1
+  for (int e = 256 + lane; e < total; e += 32) {
+    int n = ci[e];
+    if (n < 0) continue;
+    uint32_t v = __float_as_uint(cs[e]) + 1u;
+    // sink the new entry through the lane's eight: each slot keeps the better of the two
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (v > l.k[t] || (v == l.k[t] && n < l.i[t])) {
+        const uint32_t ov = l.k[t];
+        const int on = l.i[t];
+        l.k[t] = v;
+        l.i[t] = n;
+        v = ov;
+        n = on;
+      }
+  }
+}
+// The best remaining entry (highest score, lowest index among equal ones), taken off the lists: its
+// score (-1: none left) and index, the same in every lane.
+__device__ __forceinline__ float take_best(Lists& l, int& idx) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) m = max(m, l.k[t]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  unsigned i = 0x7fffffffu;
+#pragma unroll
+  for (int t = 0; t < 8; ++t)
+    if (l.k[t] == m) i = min(i, static_cast<unsigned>(l.i[t]));
+  i = __reduce_min_sync(0xffffffffu, i);
+#pragma unroll
+  for (int t = 0; t < 8; ++t)
+    if (l.k[t] == m && l.i[t] == static_cast<int>(i)) {
+      l.k[t] = 0;
+      l.i[t] = 0x7fffffff;
+    }
+  idx = m ? static_cast<int>(i) : -1;
+  return m ? __uint_as_float(m - 1u) : -1.f;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -27,40 +27,27 @@ __global__ void __launch_bounds__(32 * kWarpsF) filter_select_kernel(Ws ws, int 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int p = blockIdx.x * kWarpsF + warp;
   if (p >= L) return;  // the whole warp
+  Lists l;
   const int total = tc_piece_count(ws, L, p) * kMaxTopk;
-  const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
-  const int* ci = ws.cand_i + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
-  float vs[8];
-  int vi[8];
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int e = lane + 32 * t;
-    vs[t] = e < total ? cs[e] : -1.f;
-    vi[t] = e < total ? ci[e] : -1;
-  }
+  load_lists(ws, total, p, lane, l);
   const int id = ws.live[k & 1][p];
   const float win = ws.win_pos[p];
   const float rn = ws.rnorm[id];
-  float best = -1.f;
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    if (vi[t] < 0 || vi[t] >= ws.N) vs[t] = -1.f;
-    best = fmaxf(best, vs[t]);
-  }
-  best = warp_max(best);
-  // win is three bounds; two of them, rounded up
-  const float thr = best - 0.66667f * win;
-  int n = 0, mine = -1;  // candidates in the window; lane c < n keeps candidate c
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    unsigned m = __ballot_sync(0xffffffffu, vs[t] >= 0.f && !(vs[t] < thr));
-    while (m) {
-      const int src = __ffs(m) - 1;
-      m &= m - 1;
-      const int idx = __shfl_sync(0xffffffffu, vi[t], src);
-      if (lane == n) mine = idx;
-      ++n;
+  settle_lists(ws, total, p, lane, l);
+  // The window's candidates, best first; lane c < n keeps candidate c. win is three bounds: two of
+  // them, rounded up, below the best.
+  int n = 0, mine = -1;
+  float best = -1.f, thr = 0.f;
+  while (n <= kMaxC) {
+    int idx;
+    const float v = take_best(l, idx);
+    if (n == 0) {
+      best = v;
+      thr = best - 0.66667f * win;
     }
+    if (!(v >= 0.f) || v < thr) break;
+    if (lane == n) mine = idx;
+    ++n;
   }
   const bool ranged = rn > 1e-12f && rn < 1e12f && win < 1e30f;  // false for a NaN
   if (!ranged || n == 0 || n > kMaxC) {

@@ -160,12 +160,11 @@ __global__ void __launch_bounds__(256) compact_kernel(Ws ws, int j, int S, int r
   }
   const int M4 = ws.Mp / 4;
   // Positions that do not move (nothing before them retired) keep the quantised rows the
-  // one-warp update kernel wrote for them; other blocks quantise from the FP32 residuals.
+  // update kernel wrote for them; other blocks quantise from the FP32 residuals.
   int keep_all = 1;
   for (int i = 0; i < kCompactChunk; ++i)
     if (p0 + i < Lin && dest_s[i] != i) keep_all = 0;
-  const bool rows_in_place = reuse && ws.upd_w == 1 && ws.prec != OMP_PREC_FP32 && before == p0 &&
-                             keep_all;
+  const bool rows_in_place = reuse && ws.prec != OMP_PREC_FP32 && before == p0 && keep_all;
 #pragma unroll
   for (int m = 0; m < 2; ++m) {
     const int i = warp + 8 * m;
@@ -375,41 +374,15 @@ __global__ void __launch_bounds__(32) topk_out_kernel(Ws ws, const CallArgs* arg
     return;
   }
   const int total = tc_piece_count(ws, ws.cnt[1], p) * kMaxTopk;
-  const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
-  const int* ci = ws.cand_i + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
-  float vs[8];
-  int vi[8];
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int e = lane + 32 * t;
-    const bool ok = e < total;
-    vs[t] = ok ? cs[e] : -1.f;
-    vi[t] = ok ? ci[e] : 0x7fffffff;
-    if (vi[t] < 0) { vs[t] = -1.f; vi[t] = 0x7fffffff; }
-  }
+  Lists l;
+  load_lists(ws, total, p, lane, l);
+  settle_lists(ws, total, p, lane, l);
   for (int sel = 0; sel < topk; ++sel) {
-    float bs = -2.f;
-    int bi = 0x7fffffff, bt = -1;
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-      if (better(vs[t], vi[t], bs, bi)) { bs = vs[t]; bi = vi[t]; bt = t; }
-    float gs = bs;
-    int gi = bi;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float os = __shfl_xor_sync(0xffffffffu, gs, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, gi, o);
-      if (better(os, oi, gs, gi)) { gs = os; gi = oi; }
-    }
-    if (bt >= 0 && bi == gi && bs == gs) {
-#pragma unroll
-      for (int t = 0; t < 8; ++t)
-        if (t == bt) { vs[t] = -2.f; vi[t] = 0x7fffffff; }
-    }
+    int gi;
+    const float gs = take_best(l, gi);
     if (lane == 0) {
-      const bool ok = gi >= 0 && gi < ws.N && gs >= 0.f;
-      io[sel] = ok ? gi : -1;
-      so[sel] = ok ? gs : -1.f;
+      io[sel] = gi < ws.N ? gi : -1;
+      so[sel] = gi >= 0 && gi < ws.N ? gs : -1.f;
     }
   }
 }
