@@ -526,7 +526,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     else
       cp_async_wait_all();
     __syncwarp();
-    const float* grow = ws.gram + static_cast<size_t>(ns) * ws.N;
+    const float* grow = ws.gram + static_cast<size_t>(ns) * ws.ldg;
     const double nrm2 = __ldg(ws.norm2 + ns);
     for (int i = lane; i < kk; i += 32) gs.w[i] = __ldg(grow + gs.sup[i]);
     __syncwarp();

@@ -8,7 +8,7 @@
 //     A16   N x Mp  bf16    RN-even copy                                     -- BF16 correlation
 //     A8    N x Mp  e4m3    per-atom scaled copy, sa[n] = amax_n / 448        -- FP8 correlation
 //     inv_norm[N] float = 1/||a_n|| (from FP64), norm2[N] double = ||a_n||^2
-//     gram  N x N   float   G = A^T A (Sec. 2.2 precompute)
+//     gram  N x ldg float   G = A^T A (Sec. 2.2 precompute); rows padded with zeros to a multiple of 4
 //   per signal, indexed by the signal id b (its row in Y):
 //     R32   Bmax x Mp float  residual r (the master copy)
 //     F     Bmax x Smax(Smax+1)/2 double  packed upper-triangular inverse Cholesky factor,
@@ -83,9 +83,10 @@ struct Ws {
   float* inv_norm;
   float* escale;   // quantised paths: score scale per atom (1/||a|| or s_a/||a||), padded
   double* norm2;
+  int ldg;         // row pitch of gram and c0: N rounded up to a multiple of 4
   float* gram;
   float* score;     // FP32 scores of a solve of up to 8 signals (small.cu)
-  float* c0;        // Bmax x N FP32 first correlation of the Gram-space solve (allocated on use)
+  float* c0;        // Bmax x ldg FP32 first correlation of the Gram-space solve (allocated on use)
   // signal state
   float* R32;
   void* Rq[2];
@@ -212,6 +213,17 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float x) {
   s = t;
   e = __fadd_rn(e, err);
 }
+
+// Sum of squares of a row spread over a warp, each lane adding its elements by square_in: FP32 sums
+// with their rounding errors carried (two_sum, the squares split by an FMA) hold it to about 2^-46,
+// without FP64 arithmetic per element, which GB300 issues at a small fraction of its FP32 rate. Squares
+// that leave FP32's comfortable range show in the total; the caller then sums in FP64.
+__device__ __forceinline__ void square_in(float& hi, float& lo, float v) {
+  const float p = __fmul_rn(v, v);
+  lo = __fadd_rn(lo, fmaf(v, v, -p));
+  two_sum(hi, lo, p);
+}
+__device__ __forceinline__ bool squares_ok(double s) { return s > 1e-20 && s < 1e30; }
 
 // Iteration index of a per-iteration kernel: the launch's own k, or, when the launch passes -1
 // (the body of the graph's device-side while loop, identical for every iteration), the counter

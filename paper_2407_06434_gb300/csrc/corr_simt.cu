@@ -166,20 +166,12 @@ __device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, c
   auto prows = [&](int i) { return p0 + (i >> 2) * (BM / 2) + ty * 4 + (i & 3); };
 
   if (GRAM || MODE == kStoreC) {
-    // C row-major with N columns (rows < L), 16 bytes at a time where the rows stay aligned; the
-    // Gram form stores the mirror image G[n][p] as well
+    // C row-major in rows of ldg, 16 bytes at a time (the products past N are zeros); the Gram form
+    // stores the mirror image G[n][p] as well
     float* C = GRAM ? ws.gram : ws.c0;
-    const bool vec = (ws.N & 3) == 0;
     auto store4 = [&](int row, int col, float a, float b, float c, float d) {
-      float* g = C + static_cast<size_t>(row) * ws.N + col;
-      if (vec && col + 3 < ws.N) {
-        *reinterpret_cast<float4*>(g) = make_float4(a, b, c, d);
-      } else {
-        if (col < ws.N) g[0] = a;
-        if (col + 1 < ws.N) g[1] = b;
-        if (col + 2 < ws.N) g[2] = c;
-        if (col + 3 < ws.N) g[3] = d;
-      }
+      if (col < ws.ldg)
+        *reinterpret_cast<float4*>(C + static_cast<size_t>(row) * ws.ldg + col) = make_float4(a, b, c, d);
     };
 #pragma unroll
     for (int i = 0; i < 8; ++i)

@@ -159,8 +159,8 @@ template <int W>
 __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S, float eps, int eps_rel) {
   constexpr int T = 32 * W;
   // c update shape: a lone warp keeps 4 float4 accumulators and 2 Gram rows in flight; wider
-  // blocks spread the atoms thinner (one float4 per thread) and keep 8 rows in flight
-  constexpr int VP = W == 1 ? 4 : 1;
+  // blocks two accumulators (2048 atoms a pass) and 4 rows
+  constexpr int VP = W == 1 ? 4 : 2;
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
@@ -174,10 +174,9 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
   double* bvg = ws.bv + static_cast<size_t>(b) * ws.Smax;
   double* Fg = ws.F + static_cast<size_t>(b) * ws.Fstride;
   float* Ff = ws.F32 + static_cast<size_t>(b) * ws.Fstride;
-  const float* c0 = ws.c0 + static_cast<size_t>(b) * N;
+  const float* c0 = ws.c0 + static_cast<size_t>(b) * ws.ldg;
   for (int n = tid; n < np4(N); n += T) g.c[n] = n < N ? c0[n] : 0.f;
   bsync<W>();
-  const bool vec = (N & 3) == 0;  // Gram rows start 16-byte aligned
 
   double r2 = static_cast<double>(yn) * static_cast<double>(yn);
   const double thr = eps_rel ? static_cast<double>(eps) * static_cast<double>(yn) : static_cast<double>(eps);
@@ -232,7 +231,7 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
       break;
     }
     // ---- w_i = G[n*, s_i]
-    const float* grow = ws.gram + static_cast<size_t>(ns) * N;
+    const float* grow = ws.gram + static_cast<size_t>(ns) * ws.ldg;
     for (int i = tid; i < k; i += T) g.w[i] = __ldg(grow + g.sup[i]);
     const double nrm2 = ws.norm2[ns];
     const float cn = g.c[ns];
@@ -244,6 +243,7 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
     for (int j = tid; j < k; j += T) {
       const float* col = g.Fs + static_cast<size_t>(j) * (j + 1) / 2;
       float zj = 0.f;
+#pragma unroll 4
       for (int i = 0; i <= j; ++i) zj = fmaf(col[i], g.w[i], zj);
       g.z[j] = zj;
       const float p = __fmul_rn(zj, zj);
@@ -285,7 +285,12 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
     const size_t off = static_cast<size_t>(k) * (k + 1) / 2;
     for (int i = tid; i < k; i += T) {
       float u = 0.f;
-      for (int j = i; j < k; ++j) u = fmaf(g.Fs[static_cast<size_t>(j) * (j + 1) / 2 + i], g.z[j], u);
+      int cj = i * (i + 1) / 2 + i;  // entry i of column j
+#pragma unroll 4
+      for (int j = i; j < k; ++j) {
+        u = fmaf(g.Fs[cj], g.z[j], u);
+        cj += j + 1;
+      }
       const double fv = -gamma * static_cast<double>(u);
       const float f32 = static_cast<float>(fv);
       g.f[i] = f32;
@@ -304,29 +309,21 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
     }
     bsync<W>();
     // ---- c <- c - b_k sum_j f_j G[s_j, :], in panels: thread t takes 4 atoms per 4T, 16-byte
-    // Gram loads (scalar ones when N is not a multiple of 4)
+    // Gram loads
     const float bf = static_cast<float>(g.rd[9]);
     for (int p0 = 0; p0 < N; p0 += 4 * T * VP) {
       float4 acc[VP];
 #pragma unroll
       for (int t = 0; t < VP; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll (W == 1 ? 2 : 8)
+#pragma unroll (W == 1 ? 2 : 4)
       for (int a = 0; a <= k; ++a) {
         const float fa = g.f[a];
-        const float* gr = ws.gram + static_cast<size_t>(g.sup[a]) * N;
+        const float* gr = ws.gram + static_cast<size_t>(g.sup[a]) * ws.ldg;
 #pragma unroll
         for (int t = 0; t < VP; ++t) {
           const int n0 = p0 + 4 * T * t + 4 * tid;
           if (n0 < N) {
-            float4 gv;
-            if (vec) {
-              gv = __ldg(reinterpret_cast<const float4*>(gr + n0));
-            } else {
-              gv.x = __ldg(gr + n0);
-              gv.y = n0 + 1 < N ? __ldg(gr + n0 + 1) : 0.f;
-              gv.z = n0 + 2 < N ? __ldg(gr + n0 + 2) : 0.f;
-              gv.w = n0 + 3 < N ? __ldg(gr + n0 + 3) : 0.f;
-            }
+            const float4 gv = __ldg(reinterpret_cast<const float4*>(gr + n0));
             acc[t].x = fmaf(fa, gv.x, acc[t].x);
             acc[t].y = fmaf(fa, gv.y, acc[t].y);
             acc[t].z = fmaf(fa, gv.z, acc[t].z);

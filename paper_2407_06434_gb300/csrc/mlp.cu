@@ -305,9 +305,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 // ------------------------------------------------------------------------ small kernels
 // Feature input: y in BF16 (zero padded to Mp) and 1/||y|| (0 for y == 0 or non-finite y). One warp
-// per signal, the row read once: up to 16 values a lane stay in registers for the second step (a
-// longer row is read again). Bound by the row's round trip to HBM and by the FP64 sum of squares,
-// which GB300 issues at a small fraction of its FP32 rate.
+// per signal, the row read once: up to 16 values a lane stay in registers for the second step 
 __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict__ Y, int M, int Mp, int B,
                                                         __nv_bfloat16* Yq, float* inv_ynorm) {
   constexpr int R = 16;
@@ -315,7 +313,7 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;
   const float* y = Y + static_cast<size_t>(b) * M;
-  double s = 0.0;
+  float hi = 0.f, lo = 0.f;
   bool finite = true;
   for (int m0 = 0; m0 < Mp; m0 += 32 * R) {
     float v[R];
@@ -327,7 +325,7 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       finite = finite && isfinite(v[i]);
-      s += static_cast<double>(v[i]) * v[i];
+      square_in(hi, lo, v[i]);
     }
     // written as if finite; a signal with a NaN or Inf is cleared below
     __nv_bfloat16* q = Yq + static_cast<size_t>(b) * Mp;
@@ -337,7 +335,12 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
       if (m < Mp) q[m] = __float2bfloat16_rn(v[i]);
     }
   }
-  s = warp_sum(s);
+  double s = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
+  if (!squares_ok(s)) {  // zero, tiny or huge signals (or a NaN)
+    s = 0.0;
+    for (int m = lane; m < M; m += 32) s += static_cast<double>(y[m]) * y[m];
+    s = warp_sum(s);
+  }
   finite = __all_sync(0xffffffffu, finite);
   if (!finite)
     for (int m = lane; m < Mp; m += 32) Yq[static_cast<size_t>(b) * Mp + m] = __float2bfloat16_rn(0.f);

@@ -15,13 +15,19 @@ __global__ void __launch_bounds__(256) prep_kernel(Ws ws, const float* __restric
   for (int n = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; n < ws.N; n += warps) {
     const float* a = A + static_cast<size_t>(n) * ws.M;
     float* a32 = ws.A32 + static_cast<size_t>(n) * ws.Mp;
+    constexpr int R = 16;  // loads in flight per lane
     double s = 0.0;
     float amax = 0.f;
-    for (int m = lane; m < ws.Mp; m += 32) {
-      const float v = m < ws.M ? a[m] : 0.f;
-      a32[m] = v;
-      s += static_cast<double>(v) * static_cast<double>(v);
-      amax = fmaxf(amax, fabsf(v));
+    for (int m0 = lane; m0 < ws.Mp; m0 += 32 * R) {
+      float v[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) v[i] = m0 + 32 * i < ws.M ? __ldg(a + m0 + 32 * i) : 0.f;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        if (m0 + 32 * i < ws.Mp) a32[m0 + 32 * i] = v[i];
+        s += static_cast<double>(v[i]) * static_cast<double>(v[i]);
+        amax = fmaxf(amax, fabsf(v[i]));
+      }
     }
     s = warp_sum(s);
     amax = warp_max(amax);

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kRThreads)
     // ---- new D row and the correlations: thread i, D[k][i] = gamma (G[n*, a_i] - sum_j z_j D[j][i])
     float* Dk = sm.D + static_cast<size_t>(k) * K;
     if (has) {
-      float acc = valid ? __ldg(ws.gram + static_cast<size_t>(ns) * ws.N + atom) : 0.f;
+      float acc = valid ? __ldg(ws.gram + static_cast<size_t>(ns) * ws.ldg + atom) : 0.f;
       for (int j = 0; j < k; ++j) acc = fmaf(-sm.z[j], sm.D[static_cast<size_t>(j) * K + tid], acc);
       const float d = gf * acc;
       Dk[tid] = d;

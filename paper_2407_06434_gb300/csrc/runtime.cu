@@ -402,6 +402,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   const int64_t malign = d.precision == OMP_PREC_FP8_E4M3 ? 2 * kMpAlign : kMpAlign;
   ws.Mp = static_cast<int>((d.M + malign - 1) / malign * malign);
   ws.N = static_cast<int>(d.N);
+  ws.ldg = (ws.N + 3) / 4 * 4;
   ws.Smax = d.max_iters;
   ws.Bmax = static_cast<int>(d.max_batch);
   ws.Bpad = (ws.Bmax + kSigTile - 1) / kSigTile * kSigTile;
@@ -436,7 +437,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   if (d.precision == OMP_PREC_FP8_E4M3) ok = ok && dalloc(h, &ws.A8, N * Mp) && dalloc(h, &ws.sa, N);
   const size_t Npad = (N + 255) / 256 * 256;
   if (tc) ok = ok && dalloc(h, &ws.escale, Npad);
-  ok = ok && dalloc(h, &ws.inv_norm, N) && dalloc(h, &ws.norm2, N) && dalloc(h, &ws.gram, N * N);
+  ok = ok && dalloc(h, &ws.inv_norm, N) && dalloc(h, &ws.norm2, N) && dalloc(h, &ws.gram, N * ws.ldg);
   ok = ok && dalloc(h, &ws.R32, Bm * Mp);
   if (tc) {
     uint8_t* q0 = nullptr;
@@ -580,7 +581,7 @@ omp_status omp_solve_batch_gram(omp_handle h, const float* A, const float* Y, in
       return OMP_ERR_INVALID_ARGUMENT;
     }
     if (configure_c0_simt() != cudaSuccess) return OMP_ERR_CUDA;
-    if (!dalloc(h, &h->ws.c0, static_cast<size_t>(h->ws.Bmax) * h->ws.N)) return OMP_ERR_OUT_OF_MEMORY;
+    if (!dalloc(h, &h->ws.c0, static_cast<size_t>(h->ws.Bmax) * h->ws.ldg)) return OMP_ERR_OUT_OF_MEMORY;
   }
   if (A != h->prepared_A) {
     st = prepare(h, A, s);

@@ -292,7 +292,7 @@ __device__ __forceinline__ bool small_step(const Ws& ws, const SmallSmem& sm, co
                    : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   if (warp == 0) {
-    const float* grow = ws.gram + static_cast<size_t>(ns) * ws.N;
+    const float* grow = ws.gram + static_cast<size_t>(ns) * ws.ldg;
     const double nrm2 = __ldg(ws.norm2 + ns);
     for (int i = lane; i < kk; i += 32) gs.w[i] = __ldg(grow + gs.sup[i]);
     __syncwarp();

@@ -39,15 +39,26 @@ __global__ void __launch_bounds__(256) init_kernel(Ws ws, const CallArgs* args, 
   if (b >= B) return;
   const float* y = args->Y + static_cast<size_t>(b) * ws.M;
   float* r = ws.R32 + static_cast<size_t>(b) * ws.Mp;
-  double s = 0.0;
+  constexpr int R = 16;  // loads in flight per lane
+  float hi = 0.f, lo = 0.f;
   bool finite = true;
-  for (int m = lane; m < ws.Mp; m += 32) {
-    const float v = m < ws.M ? y[m] : 0.f;
-    finite = finite && isfinite(v);
-    r[m] = v;
-    s += static_cast<double>(v) * static_cast<double>(v);
+  for (int m0 = lane; m0 < ws.Mp; m0 += 32 * R) {
+    float v[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) v[i] = m0 + 32 * i < ws.M ? __ldg(y + m0 + 32 * i) : 0.f;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      finite = finite && isfinite(v[i]);
+      if (m0 + 32 * i < ws.Mp) r[m0 + 32 * i] = v[i];
+      square_in(hi, lo, v[i]);
+    }
   }
-  s = warp_sum(s);
+  double s = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
+  if (!squares_ok(s)) {  // zero, tiny or huge signals (or a NaN)
+    s = 0.0;
+    for (int m = lane; m < ws.M; m += 32) s += static_cast<double>(y[m]) * static_cast<double>(y[m]);
+    s = warp_sum(s);
+  }
   finite = __all_sync(0xffffffffu, finite);
   if (!finite)
     for (int m = lane; m < ws.Mp; m += 32) r[m] = 0.f;
