@@ -2,9 +2,8 @@
 // updated through the Gram matrix instead of a correlation GEMM per step), for dictionaries
 // whose Gram matrix is small (N up to a few thousand atoms, so G = A^T A stays in L2).
 //
-// One block of W warps (W = 1 for up to 1536 atoms and a batch of at least 32 signals per SM,
-// 8 otherwise) runs all iterations of one
-// signal:
+// One block of W warps (1, 4 or 8 by the number of atoms and signals, see gram_warps) runs all
+// iterations of one signal:
 //   c      = A^T y                           FP32, from one batched SIMT GEMM before the loop
 //   per step k (0-based; the paper's k+1):
 //     n*   = argmax_n |c_n| / ||a_n||        lowest atom index on ties (Alg. 1)
@@ -158,9 +157,9 @@ __device__ double residual_norm2(const Ws& ws, const GSmem& g, const double* Fg,
 template <int W>
 __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S, float eps, int eps_rel) {
   constexpr int T = 32 * W;
-  // c update shape: a lone warp keeps 4 float4 accumulators and 2 Gram rows in flight; wider
+  // c update shape: 1 or 4 warps keep 4 float4 accumulators a thread and 2 Gram rows in flight; wider
   // blocks two accumulators (2048 atoms a pass) and 4 rows
-  constexpr int VP = W == 1 ? 4 : 2;
+  constexpr int VP = W <= 4 ? 4 : 2;
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
@@ -315,7 +314,7 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
       float4 acc[VP];
 #pragma unroll
       for (int t = 0; t < VP; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll (W == 1 ? 2 : 4)
+#pragma unroll (W <= 4 ? 2 : 4)
       for (int a = 0; a <= k; ++a) {
         const float fa = g.f[a];
         const float* gr = ws.gram + static_cast<size_t>(g.sup[a]) * ws.ldg;
@@ -369,10 +368,17 @@ __global__ void __launch_bounds__(32 * W) gram_solve_kernel(Ws ws, int B, int S,
   }
 }
 
-// warps per signal: one for small dictionaries when the batch fills the GPU with one-warp
-// signals (16 per SM), eight otherwise (a larger N shortens each signal's argmax and c update;
-// a small batch needs the parallelism within each signal)
-int gram_warps(int N, int B, int sms) { return (N <= 1536 && B >= 2 * 16 * sms) ? 1 : 8; }
+// Warps per signal: eight (a larger N shortens each signal's argmax and c update; a small batch needs
+// the parallelism within each signal), or four for dictionaries of one pass (2048 atoms) once the
+// batch is more than the eight-warp blocks that fit at once. Measured, us a solve with 8 and 4 warps:
+// 1207 atoms, 24 steps: 300 signals 200 / 202, 700 239 / 231, 1000 380 / 257, 3000 826 / 671; 4000 atoms:
+// 700 signals 391 / 422; 8064 x 1207, 1200 signals, 30 steps: iteration 519 / 348. One warp for up to
+// 1024 atoms and at least 32 signals per SM (4 and 1 warps: 1024 atoms, 32 steps, 5000 signals
+// 1189 / 1172, 8000 1814 / 1331; 1500 atoms, 24 steps, 5000 signals 1062 / 1205).
+int gram_warps(int N, int B, int sms) {
+  if (N <= 1024 && B >= 2 * 16 * sms) return 1;
+  return N <= 2048 && B >= 4 * sms ? 4 : 8;
+}
 
 template <int W>
 cudaError_t set_attr(size_t bytes) {
@@ -384,15 +390,19 @@ cudaError_t set_attr(size_t bytes) {
 cudaError_t configure_gram_solve(const Ws& ws) {
   const size_t bytes = gs_bytes(ws.N, ws.Smax);
   if (bytes > 227 * 1024) return cudaErrorInvalidValue;
-  const cudaError_t e = set_attr<1>(bytes);
+  cudaError_t e = set_attr<1>(bytes);
+  if (e == cudaSuccess) e = set_attr<4>(bytes);
   return e == cudaSuccess ? set_attr<8>(bytes) : e;
 }
 
 void launch_gram_solve(const Ws& ws, const CallArgs*, int B, int S, float eps, int eps_rel,
                        cudaStream_t s) {
   const size_t smem = gs_bytes(ws.N, S);
-  if (gram_warps(ws.N, B, ws.tc_grid > 0 ? ws.tc_grid : 152) == 1)
+  const int W = gram_warps(ws.N, B, ws.tc_grid > 0 ? ws.tc_grid : 152);
+  if (W == 1)
     gram_solve_kernel<1><<<B, 32, smem, s>>>(ws, B, S, eps, eps_rel);
+  else if (W == 4)
+    gram_solve_kernel<4><<<B, 128, smem, s>>>(ws, B, S, eps, eps_rel);
   else
     gram_solve_kernel<8><<<B, 256, smem, s>>>(ws, B, S, eps, eps_rel);
 }

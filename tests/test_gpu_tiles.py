@@ -173,3 +173,22 @@ def test_fp32_filter_close_atoms_and_extreme_scales(lib, monkeypatch):
         got, want = _solve_both(lib, monkeypatch, At.t(), Y, 10, 0.0)
         for g, w in zip(got, want):
             assert np.array_equal(g.view(np.uint32), w.view(np.uint32))
+
+
+# The Gram-space solve with 1, 4 and 8 warps a signal (by atoms and batch), atom counts that leave
+# the padded Gram rows 1 to 3 columns short, and more atoms than one pass of c holds, against the dense
+# FP32 solve: the same picks wherever they agree so far, coefficients within the FP32 error of both.
+@pytest.mark.parametrize("M,N,B,S", [(96, 1021, 4900, 8), (96, 1022, 700, 8), (96, 2047, 620, 8), (128, 2051, 640, 8),
+                                     (128, 4099, 50, 8), (96, 63, 650, 6)])
+def test_gram_solve_warps(lib, M, N, B, S):
+    A, Y = _planted(M, N, B, S, M + N + B)
+    s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision="fp32")
+    X1, s1 = (t.cpu().numpy() for t in s.solve_gram(A, Y, S))
+    X2, s2 = (t.cpu().numpy() for t in s.solve(A, Y, S))
+    s.close()
+    same = np.all(s1 == s2, axis=1)
+    assert np.mean(same) > 0.98  # the rest are near-ties
+    A64 = A.double().cpu().numpy()
+    for b in np.flatnonzero(same)[::17]:
+        cond = np.linalg.cond(A64[:, s1[b]])
+        assert np.linalg.norm(X1[b] - X2[b]) <= 256 * 2.0 ** -24 * cond ** 2 * np.linalg.norm(X2[b])
