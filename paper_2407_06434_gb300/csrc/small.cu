@@ -25,6 +25,7 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, int V0) 
   return V0 == 1 ? slot_dot<true>(a, b) : slot_dot<false>(a, b);
 }
 constexpr int kT = 256, kWarps = kT / 32;
+constexpr int kList = 32;                          // atoms of a pick's window that are listed
 constexpr int kGS = 4;                             // wide: scores per recorded maximum
 constexpr int kSmallMaxB = 8;                      // wide: signals that share one pass over A
 constexpr int64_t kWideMaxElems = 24ll << 20;      // wide: FP32 rows of at most 96 MB stay in L2
@@ -196,12 +197,13 @@ __device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, cons
   const float eps = 1.01f * (2.f * ws.gam_32 + 4.f * 0x1p-24f);
   const bool ranged = rnorm > 1e-15f && rnorm < 1e15f;
   const float thr = ranged ? bs - 2.f * eps * rnorm : -2.f;
+  int* list = reinterpret_cast<int*>(sm.P);  // the first kList atoms of the window
   auto window = [&](int g, float m) {
     if (!(m < thr))
       for (int n = g * GS; n < min(N, g * GS + GS); ++n)
         if (GS == 1 || !(sc[n] < thr)) {
-          atomicAdd(sm.ctl, 1);
-          sm.ctl[1] = n;
+          const int c = atomicAdd(sm.ctl, 1);
+          if (c < kList) list[c] = n;
         }
   };
 #pragma unroll
@@ -209,36 +211,35 @@ __device__ __forceinline__ int pick_atom(const Ws& ws, const SmallSmem& sm, cons
     if (tid + i * kT < NG) window(tid + i * kT, head[i]);
   for (int g = tid + 8 * kT; g < NG; g += kT) window(g, gm[g]);
   __syncthreads();
-  if (sm.ctl[0] == 1) {  // alone in the window: the best, or an atom that has no score
-    const int n = sm.ctl[1];
+  const int cnt = sm.ctl[0];
+  if (cnt == 1) {  // alone in the window: the best, or an atom that has no score
+    const int n = list[0];
     return sc[n] >= 0.f ? n : -1;
   }
   // score the window's atoms as the batched path does
   const float4* r4 = reinterpret_cast<const float4*>(sm.r);
   float cs = -1.f;
   int ci = 0x7fffffff;
+  const float4* A4 = reinterpret_cast<const float4*>(ws.A32);
+  auto take = [&](int n, float dot) {
+    const float s = fabsf(dot) * __ldg(ws.inv_norm + n);
+    if (better(s, n, cs, ci) && s >= 0.f) {  // false for a NaN
+      cs = s;
+      ci = n;
+    }
+  };
+  const bool listed = cnt <= kList;  // else the whole row of scores is walked again
+  const int end = listed ? cnt : N;
   if (ws.prec == OMP_PREC_FP32) {
-    for (int n = tid; n < N; n += kT)
-      if (!(sc[n] < thr)) {
-        const float s =
-            fabsf(chain_dot(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp), r4, M4)) *
-            __ldg(ws.inv_norm + n);
-        if (s > cs) {
-          cs = s;
-          ci = n;
-        }
-      }
+    for (int i = tid; i < end; i += kT) {
+      const int n = listed ? list[i] : i;
+      if (listed || !(sc[n] < thr)) take(n, chain_dot(A4 + static_cast<size_t>(n) * M4, r4, M4));
+    }
   } else {
-    for (int n = warp; n < N; n += kWarps)
-      if (!(sc[n] < thr)) {
-        const float s = fabsf(rescore_dot(reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp), r4,
-                                          M4, W0, V0, lane)) *
-                        __ldg(ws.inv_norm + n);
-        if (s > cs) {
-          cs = s;
-          ci = n;
-        }
-      }
+    for (int i = warp; i < end; i += kWarps) {
+      const int n = listed ? list[i] : i;
+      if (listed || !(sc[n] < thr)) take(n, rescore_dot(A4 + static_cast<size_t>(n) * M4, r4, M4, W0, V0, lane));
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
