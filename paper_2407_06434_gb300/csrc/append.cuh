@@ -875,26 +875,26 @@ void launch_w(const Ws& ws, int V, int k, int B, int S, float eps, int eps_rel, 
   else launch_t<W, 8>(ws, k, B, S, eps, eps_rel, s);
 }
 
-template <int W, int V>
-cudaError_t set_attr_t(int bytes) {
-  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(append_update_kernel<W, V, false, false>), bytes);
+template <int W, int V, bool G24>
+cudaError_t set_attr_g(int bytes) {
+  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(append_update_kernel<W, V, G24, false>), bytes);
   if (e == cudaSuccess)
-    e = raise_smem_limit(reinterpret_cast<const void*>(append_update_kernel<W, V, true, false>), bytes);
-  if (e == cudaSuccess)
-    e = raise_smem_limit(reinterpret_cast<const void*>(append_update_kernel<W, V, false, true>), bytes);
-  if (e == cudaSuccess)
-    e = raise_smem_limit(reinterpret_cast<const void*>(append_update_kernel<W, V, true, true>), bytes);
+    e = raise_smem_limit(reinterpret_cast<const void*>(append_update_kernel<W, V, G24, true>), bytes);
   return e;
 }
 
+template <int W, int V>
+cudaError_t set_attr_t(const Ws& ws) {
+  const int bytes = static_cast<int>(group_bytes(ws));
+  return ws.A24h ? set_attr_g<W, V, true>(bytes) : set_attr_g<W, V, false>(bytes);
+}
+
+// the kernels that the handle's row length takes with W warps (none if the row needs more)
 template <int W>
 cudaError_t set_attr_w(const Ws& ws) {
-  const int bytes = static_cast<int>(group_bytes(ws));
-  cudaError_t e = set_attr_t<W, 1>(bytes);
-  if (e == cudaSuccess) e = set_attr_t<W, 2>(bytes);
-  if (e == cudaSuccess) e = set_attr_t<W, 4>(bytes);
-  if (e == cudaSuccess) e = set_attr_t<W, 8>(bytes);
-  return e;
+  const int V = update_slots(ws.Mp, W);
+  if (V == 0) return cudaSuccess;
+  return V == 1 ? set_attr_t<W, 1>(ws) : V == 2 ? set_attr_t<W, 2>(ws) : V == 4 ? set_attr_t<W, 4>(ws) : set_attr_t<W, 8>(ws);
 }
 
 }  // namespace

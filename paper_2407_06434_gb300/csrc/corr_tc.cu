@@ -367,11 +367,10 @@ cudaError_t tc_setup(const Ws& ws, int sm_count, TcPlan** plan) {
     return cudaErrorNotSupported;
   }
   cudaError_t e = cudaSuccess;
-  for (int prec : {static_cast<int>(OMP_PREC_BF16), static_cast<int>(OMP_PREC_FP8_E4M3)})
-    for (int nst : {2, 3, 4, 6})
-      for (int cl = 1; cl <= 2; ++cl)
-        if (e == cudaSuccess && kern_of(prec, nst, cl))
-          e = set_smem_attr(kern_of(prec, nst, cl), smem_bytes(nst, cl));
+  for (int nst : {2, 3, 4, 6})
+    for (int cl = 1; cl <= 2; ++cl)
+      if (e == cudaSuccess && kern_of(ws.tcprec, nst, cl))
+        e = set_smem_attr(kern_of(ws.tcprec, nst, cl), smem_bytes(nst, cl));
   if (e != cudaSuccess) {
     delete p;
     return e;

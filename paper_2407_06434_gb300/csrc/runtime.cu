@@ -72,20 +72,43 @@ bool fault_alloc_due() {
   return at > 0 && ++counter == at;
 }
 
-template <class T>
-bool dalloc(omp_handle_s* h, T** p, size_t count) {
+bool device_alloc(omp_handle_s* h, void** p, size_t bytes) {
   *p = nullptr;
-  if (count == 0) return true;
-  if (fault_alloc_due()) return false;
-  void* q = nullptr;
-  if (cudaMalloc(&q, count * sizeof(T)) != cudaSuccess) {
+  if (cudaMalloc(p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  h->allocs.push_back(q);
-  *p = static_cast<T*>(q);
+  h->allocs.push_back(*p);
   return true;
 }
+
+// A handle's workspaces come from one allocation: each is asked for, then all pointers are set. (One
+// cudaMalloc and cudaFree per workspace, about forty, made up most of creating and destroying a
+// handle: 470 and 300 us, which a caller with one batch per dictionary pays every time.)
+struct Arena {
+  struct Want {
+    void** p;
+    size_t at;
+  };
+  std::vector<Want> wants;
+  size_t bytes = 0;
+
+  template <class T>
+  bool ask(T** p, size_t count) {
+    *p = nullptr;
+    if (count == 0) return true;
+    if (fault_alloc_due()) return false;
+    wants.push_back({reinterpret_cast<void**>(p), bytes});
+    bytes += (count * sizeof(T) + 511) / 512 * 512;
+    return true;
+  }
+  bool allocate(omp_handle_s* h) {
+    void* base = nullptr;
+    if (!device_alloc(h, &base, bytes)) return false;
+    for (const Want& w : wants) *w.p = static_cast<char*>(base) + w.at;
+    return true;
+  }
+};
 
 void release(omp_handle_s* h) {
   for (auto& g : h->graphs) cudaGraphExecDestroy(g.exec);
@@ -385,9 +408,12 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
     cudaGetLastError();
     return OMP_ERR_UNSUPPORTED_DEVICE;
   }
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, d.device) != cudaSuccess) return OMP_ERR_CUDA;
-  if (prop.major != 10 || prop.minor != 3) return OMP_ERR_UNSUPPORTED_DEVICE;
+  int major = 0, minor = 0, sms = 0;  // (the attributes alone: the whole property record takes long to fill)
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, d.device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, d.device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d.device) != cudaSuccess)
+    return OMP_ERR_CUDA;
+  if (major != 10 || minor != 3) return OMP_ERR_UNSUPPORTED_DEVICE;
   DeviceGuard guard(d.device);
 
   omp_handle_s* h = new (std::nothrow) omp_handle_s();
@@ -395,7 +421,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   h->d = d;
   if (h->d.rescore_topk == 0) h->d.rescore_topk = kMaxTopk;
   h->dev = d.device;
-  h->sm_count = prop.multiProcessorCount;
+  h->sm_count = sms;
   Ws& ws = h->ws;
   ws.M = static_cast<int>(d.M);
   // one tensor-core K stage is 128 bytes: 64 BF16 or 128 E4M3 elements
@@ -430,24 +456,22 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   if (tc) tc_fill_sched(ws, h->sm_count);
   const size_t N = ws.N, Mp = ws.Mp, Bm = ws.Bmax, Bp = ws.Bpad, Sm = ws.Smax;
   const size_t qbytes = ws.tcprec == OMP_PREC_BF16 ? 2 : 1;
+  Arena ar;
   bool ok = true;
-  ok = ok && dalloc(h, &ws.A32, N * Mp);
-  if (d.gather24) ok = ok && dalloc(h, &ws.A24h, N * Mp) && dalloc(h, &ws.A24l, N * Mp);
-  if (ws.tcprec == OMP_PREC_BF16) ok = ok && dalloc(h, &ws.A16, N * Mp);
-  if (d.precision == OMP_PREC_FP8_E4M3) ok = ok && dalloc(h, &ws.A8, N * Mp) && dalloc(h, &ws.sa, N);
+  ok = ok && ar.ask(&ws.A32, N * Mp);
+  if (d.gather24) ok = ok && ar.ask(&ws.A24h, N * Mp) && ar.ask(&ws.A24l, N * Mp);
+  if (ws.tcprec == OMP_PREC_BF16) ok = ok && ar.ask(&ws.A16, N * Mp);
+  if (d.precision == OMP_PREC_FP8_E4M3) ok = ok && ar.ask(&ws.A8, N * Mp) && ar.ask(&ws.sa, N);
   const size_t Npad = (N + 255) / 256 * 256;
-  if (tc) ok = ok && dalloc(h, &ws.escale, Npad);
-  ok = ok && dalloc(h, &ws.inv_norm, N) && dalloc(h, &ws.norm2, N) && dalloc(h, &ws.gram, N * ws.ldg);
-  ok = ok && dalloc(h, &ws.R32, Bm * Mp);
+  if (tc) ok = ok && ar.ask(&ws.escale, Npad);
+  ok = ok && ar.ask(&ws.inv_norm, N) && ar.ask(&ws.norm2, N) && ar.ask(&ws.gram, N * ws.ldg);
+  ok = ok && ar.ask(&ws.R32, Bm * Mp);
   if (tc) {
-    uint8_t* q0 = nullptr;
-    uint8_t* q1 = nullptr;
-    ok = ok && dalloc(h, &q0, Bp * Mp * qbytes) && dalloc(h, &q1, Bp * Mp * qbytes);
-    ws.Rq[0] = q0;
-    ws.Rq[1] = q1;
-    ok = ok && dalloc(h, &ws.sr[0], Bp) && dalloc(h, &ws.sr[1], Bp);
-    ok = ok && dalloc(h, &ws.cand_s, Bp * ws.pieces * kMaxTopk) &&
-         dalloc(h, &ws.cand_i, Bp * ws.pieces * kMaxTopk);
+    ok = ok && ar.ask(reinterpret_cast<uint8_t**>(&ws.Rq[0]), Bp * Mp * qbytes) &&
+         ar.ask(reinterpret_cast<uint8_t**>(&ws.Rq[1]), Bp * Mp * qbytes);
+    ok = ok && ar.ask(&ws.sr[0], Bp) && ar.ask(&ws.sr[1], Bp);
+    ok = ok && ar.ask(&ws.cand_s, Bp * ws.pieces * kMaxTopk) &&
+         ar.ask(&ws.cand_i, Bp * ws.pieces * kMaxTopk);
   }
   // The pruning thresholds (and the data-driven bound they carry): on BF16 always; on E4M3,
   // whose worst-case bound is too loose to prune, only where the one-warp update quantises the
@@ -455,26 +479,27 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   const bool want_tau = ws.prec == OMP_PREC_BF16 ||
                         (ws.prec == OMP_PREC_FP8_E4M3 && update_default_warps(ws.Mp) == 1);
   if (want_tau && ws.rescore_eps > 0.f && ws.Smax <= kTauSmax)
-    ok = ok && dalloc(h, &ws.tau, Bm) && dalloc(h, &ws.tau_pos, Bp) && dalloc(h, &ws.win_pos, Bp) &&
-         (ws.prec != OMP_PREC_FP8_E4M3 || dalloc(h, &ws.ea, 1));
+    ok = ok && ar.ask(&ws.tau, Bm) && ar.ask(&ws.tau_pos, Bp) && ar.ask(&ws.win_pos, Bp) &&
+         (ws.prec != OMP_PREC_FP8_E4M3 || ar.ask(&ws.ea, 1));
   if (ws.filt)
-    ok = ok && dalloc(h, &ws.win_pos, Bp) && dalloc(h, &ws.ea, 1) && dalloc(h, &ws.ovf, Bm) &&
-         dalloc(h, &ws.ovf_cnt, Sm + 1);
-  ok = ok && dalloc(h, &ws.live[0], Bm) && dalloc(h, &ws.live[1], Bm);
-  ok = ok && dalloc(h, &ws.livek[0], Bm) && dalloc(h, &ws.livek[1], Bm);
-  ok = ok && dalloc(h, &ws.cnt, Sm + 2) && dalloc(h, &ws.kdev, 1) && dalloc(h, &ws.flag, Bm) && dalloc(h, &ws.cand1, Bm);
-  ok = ok && dalloc(h, &ws.upd_ctr, Sm + 1);
-  ok = ok && dalloc(h, &ws.score, small_score_floats(ws.N, ws.Bmax));
-  ok = ok && dalloc(h, &ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
-       dalloc(h, &ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && dalloc(h, &ws.bv, Bm * Sm) &&
-       dalloc(h, &ws.sup, Bm * Sm);
-  ok = ok && dalloc(h, &ws.drop, Bm * Sm) && dalloc(h, &ws.fb, Bm);
-  ok = ok && dalloc(h, &ws.ynorm, Bm) && dalloc(h, &ws.rnorm, Bm) && dalloc(h, &ws.niter, Bm) &&
-       dalloc(h, &ws.stop, Bm) && dalloc(h, &ws.err, 1) && dalloc(h, &h->args_dev, 1);
-  ok = ok && dalloc(h, &h->y_stage, Bm * static_cast<size_t>(ws.M)) &&
-       dalloc(h, &h->x_stage, Bm * Sm) && dalloc(h, &h->s_stage, Bm * Sm) &&
-       dalloc(h, &h->margin_buf, Bm * Sm);
-  if (d.precision == OMP_PREC_FP32) ok = ok && dalloc(h, &h->cand2_buf, Bm);
+    ok = ok && ar.ask(&ws.win_pos, Bp) && ar.ask(&ws.ea, 1) && ar.ask(&ws.ovf, Bm) &&
+         ar.ask(&ws.ovf_cnt, Sm + 1);
+  ok = ok && ar.ask(&ws.live[0], Bm) && ar.ask(&ws.live[1], Bm);
+  ok = ok && ar.ask(&ws.livek[0], Bm) && ar.ask(&ws.livek[1], Bm);
+  ok = ok && ar.ask(&ws.cnt, Sm + 2) && ar.ask(&ws.kdev, 1) && ar.ask(&ws.flag, Bm) && ar.ask(&ws.cand1, Bm);
+  ok = ok && ar.ask(&ws.upd_ctr, Sm + 1);
+  ok = ok && ar.ask(&ws.score, small_score_floats(ws.N, ws.Bmax));
+  ok = ok && ar.ask(&ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
+       ar.ask(&ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && ar.ask(&ws.bv, Bm * Sm) &&
+       ar.ask(&ws.sup, Bm * Sm);
+  ok = ok && ar.ask(&ws.drop, Bm * Sm) && ar.ask(&ws.fb, Bm);
+  ok = ok && ar.ask(&ws.ynorm, Bm) && ar.ask(&ws.rnorm, Bm) && ar.ask(&ws.niter, Bm) &&
+       ar.ask(&ws.stop, Bm) && ar.ask(&ws.err, 1) && ar.ask(&h->args_dev, 1);
+  ok = ok && ar.ask(&h->y_stage, Bm * static_cast<size_t>(ws.M)) &&
+       ar.ask(&h->x_stage, Bm * Sm) && ar.ask(&h->s_stage, Bm * Sm) &&
+       ar.ask(&h->margin_buf, Bm * Sm);
+  if (d.precision == OMP_PREC_FP32) ok = ok && ar.ask(&h->cand2_buf, Bm);
+  ok = ok && ar.allocate(h);
   if (!ok) {
     release(h);
     delete h;
@@ -488,7 +513,8 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
                  (!ws.tau_pos || cudaMemset(ws.tau_pos, 0, Bp * sizeof(float)) == cudaSuccess) &&
                  (!ws.win_pos || cudaMemset(ws.win_pos, 0, Bp * sizeof(float)) == cudaSuccess) &&
                  cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
-                 cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking) == cudaSuccess &&
+                 (d.use_graph != 2 ||
+                  cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking) == cudaSuccess) &&
                  configure_update_kernels(ws) == cudaSuccess && configure_corr_simt(ws) == cudaSuccess &&
                  configure_small(ws) == cudaSuccess;
   if (cuda_ok && tc) cuda_ok = tc_setup(ws, h->sm_count, &h->tc) == cudaSuccess;
@@ -581,7 +607,9 @@ omp_status omp_solve_batch_gram(omp_handle h, const float* A, const float* Y, in
       return OMP_ERR_INVALID_ARGUMENT;
     }
     if (configure_c0_simt() != cudaSuccess) return OMP_ERR_CUDA;
-    if (!dalloc(h, &h->ws.c0, static_cast<size_t>(h->ws.Bmax) * h->ws.ldg)) return OMP_ERR_OUT_OF_MEMORY;
+    if (fault_alloc_due() || !device_alloc(h, reinterpret_cast<void**>(&h->ws.c0),
+                                           static_cast<size_t>(h->ws.Bmax) * h->ws.ldg * sizeof(float)))
+      return OMP_ERR_OUT_OF_MEMORY;
   }
   if (A != h->prepared_A) {
     st = prepare(h, A, s);

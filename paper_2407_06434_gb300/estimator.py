@@ -32,22 +32,22 @@ def _as_cuda_f32(a, device):
 
 def _solve(X, Y_rows, S, eps, eps_relative, precision, device):
     """One batched solve: X (M, N) dictionary, Y_rows (B, M) signals. Returns (coef (B, N) dense
-    float32 tensor, n_iter (B,) int32 tensor, X_t) on the device."""
-    import torch
+    float32, n_iter (B,) int32) as numpy arrays. Only the B x S picks leave the device; they are
+    spread over the dense rows here (on the device that took a boolean index with its waits, and B x N
+    floats to copy back)."""
     M, N = X.shape
     B = Y_rows.shape[0]
     Xd = X.t().contiguous().t()                     # column-major (stride (1, M))
     solver = omp.OmpSolver(M, N, max_batch=B, max_iters=S, precision=precision,
                            eps_relative=eps_relative, device=device.index or 0)
     try:
-        Xc, sup, n_iter, _, _ = solver.solve(Xd, Y_rows.contiguous(), S, eps, diagnostics=True)
-        coef = torch.zeros((B, N), dtype=torch.float32, device=device)
-        valid = sup >= 0
-        rows = torch.arange(B, device=device)[:, None].expand_as(sup)
-        coef[rows[valid], sup[valid].long()] = Xc[valid]
-        torch.cuda.synchronize(device)
+        out = solver.solve(Xd, Y_rows.contiguous(), S, eps, diagnostics=True)
+        Xc, sup, n_iter = (t.cpu().numpy() for t in out[:3])
     finally:
         solver.close()
+    coef = np.zeros((B, N), dtype=np.float32)
+    rows, k = np.nonzero(sup >= 0)
+    coef[rows, sup[rows, k]] = Xc[rows, k]
     return coef, n_iter
 
 
@@ -83,11 +83,10 @@ def orthogonal_mp(X, y, *, n_nonzero_coefs=None, tol=None, precision="bf16",
     S = _iters(N, M, n_nonzero_coefs, tol)
     eps = float(np.sqrt(tol)) if tol is not None else 0.0
     coef, n_iter = _solve(Xt, yt.t(), S, eps, tol is None, precision, dev)
-    out = coef.cpu().numpy().T
+    out = coef.T
     out = out[:, 0] if single else out
     if return_n_iter:
-        n = n_iter.cpu().numpy()
-        return out, (int(n[0]) if single else n)
+        return out, (int(n_iter[0]) if single else n_iter)
     return out
 
 
