@@ -75,6 +75,17 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // 157 us on average and take 67 us now, the loss kernel 856 us and now 192 us, the GELU backward
 // 102 us and now 72 us.
 
+// The warp's EPI_COLS columns of a vector over the columns (bias or scale) of column tile t, staged in
+// its shared scratch at each unit (16 bytes a lane): the chunks read them there.
+__device__ __forceinline__ void stage_columns(float* scratch, const float* x, int t, int part, int cols, int lane) {
+  static_assert(EPI_COLS == 128 && EPI_SCRATCH >= 128, "one float4 per lane");
+  const int c = t * BN + part * EPI_COLS + 4 * lane;
+  const float4 v = c < cols ? __ldg(reinterpret_cast<const float4*>(x + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncwarp();  // every lane has finished with the previous unit's
+  reinterpret_cast<float4*>(scratch)[lane] = v;
+  __syncwarp();
+}
+
 // value = acc * rowscale[r] * colscale[c] + bias[c], optional GELU; BF16 store (row-major and
 // optionally transposed into a matrix with leading dimension ldT) and optional FP32 store of the
 // pre-activation.
@@ -86,14 +97,21 @@ struct EpiAct {
   float* pre;
   __nv_bfloat16* out;
   __nv_bfloat16* outT;
-  int row;
-  __device__ void begin(int, int, int, int row_, int, float*, unsigned long long*) { row = row_; }
-  __device__ void unit(int, int) {}
+  int row, part;
+  float* scr;
+  __device__ void begin(int, int, int, int row_, int part_, float* scratch, unsigned long long*) {
+    row = row_;
+    part = part_;
+    scr = scratch;
+  }
+  // (a scale or a bias is given, not both)
+  __device__ void unit(int, int t) { stage_columns(scr, colscale ? colscale : bias, t, part, cols, row & 31); }
   __device__ void chunk(int s, int t, int c0, const uint32_t (&v)[32]) {
     const int r = s * BM + row;
     const int cb = t * BN + c0;
     if (r >= rows || cb >= cols) return;
     const float rs = rowscale ? __ldg(rowscale + r) : 1.f;
+    const float4* cv = reinterpret_cast<const float4*>(scr + (c0 - part * EPI_COLS));
     uint4* dst = reinterpret_cast<uint4*>(out + static_cast<size_t>(r) * cols + cb);
     float4* pdst = reinterpret_cast<float4*>(pre + static_cast<size_t>(r) * cols + cb);
     __nv_bfloat16* tdst = outT + static_cast<size_t>(cb) * ldT + r;
@@ -107,14 +125,13 @@ struct EpiAct {
 #pragma unroll
         for (int e = 0; e < 4; ++e) x[e] = __uint_as_float(v[j + e]) * rs;
         if (colscale) {
-          const float4 c = __ldg(reinterpret_cast<const float4*>(colscale + cb + j));
+          const float4 c = cv[j >> 2];
           x[0] *= c.x;
           x[1] *= c.y;
           x[2] *= c.z;
           x[3] *= c.w;
-        }
-        if (bias) {
-          const float4 c = __ldg(reinterpret_cast<const float4*>(bias + cb + j));
+        } else {
+          const float4 c = cv[j >> 2];
           x[0] += c.x;
           x[1] += c.y;
           x[2] += c.z;
@@ -203,14 +220,17 @@ struct EpiBCE {
   __nv_bfloat16* dO;
   __nv_bfloat16* dOT;
   float* loss;
-  int row;
+  int row, part;
+  float* scr;
   float lsum, bsum;
-  __device__ void begin(int, int, int, int row_, int, float*, unsigned long long*) {
+  __device__ void begin(int, int, int, int row_, int part_, float* scratch, unsigned long long*) {
     row = row_;
+    part = part_;
+    scr = scratch;
     lsum = 0.f;
     bsum = 0.f;
   }
-  __device__ void unit(int, int) {}
+  __device__ void unit(int, int t) { stage_columns(scr, bias, t, part, cols, row & 31); }
   __device__ void chunk(int s, int t, int c0, const uint32_t (&v)[32]) {
     const int r = s * BM + row;
     const int cb = t * BN + c0;
@@ -220,15 +240,19 @@ struct EpiBCE {
     const uint4* xsrc = reinterpret_cast<const uint4*>(skipX + static_cast<size_t>(r) * cols + cb);
     uint4* dst = reinterpret_cast<uint4*>(dO + static_cast<size_t>(r) * cols + cb);
     __nv_bfloat16* tdst = dOT + static_cast<size_t>(cb) * ldT + r;
+    const float4* cv = reinterpret_cast<const float4*>(scr + (c0 - part * EPI_COLS));
+    uint4 xq[4];  // the row's 32 features, in flight together
+#pragma unroll
+    for (int q = 0; q < 4; ++q) xq[q] = __ldg(xsrc + q);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const uint4 xw = __ldg(xsrc + q);
+      const uint4 xw = xq[q];
       const uint32_t xs[4] = {xw.x, xw.y, xw.z, xw.w};
       uint32_t ow[4];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int j = 8 * q + 4 * h;
-        const float4 c = __ldg(reinterpret_cast<const float4*>(bias + cb + j));
+        const float4 c = cv[j >> 2];
         const float bc[4] = {c.x, c.y, c.z, c.w};
         float g[4];
 #pragma unroll
@@ -283,9 +307,12 @@ struct EpiGeluBwd {
     if (r >= rows || cb >= cols) return;
     const float4* zsrc = reinterpret_cast<const float4*>(Z1 + static_cast<size_t>(r) * cols + cb);
     __nv_bfloat16* tdst = dZT + static_cast<size_t>(cb) * ldT + r;
+    float4 zq[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) zq[q] = __ldg(zsrc + q);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float4 z = __ldg(zsrc + q);
+      const float4 z = zq[q];
       const float zz[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e)

@@ -528,7 +528,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* tm_a, const CUtenso
       // one 32-column load at a time (the wait takes the loaded registers as operands, so no
       // read of them moves above it); once the last load has landed the accumulator goes back
       // to the MMA (PAIR: to the even CTA's barrier) before that chunk is scanned
-#pragma unroll
+#pragma unroll 1  // one copy of the chunk's code: four of them overran the instruction cache
       for (int c = 0; c < CH; ++c) {
         uint32_t cur[32];
         tmem_ld32_issue(taddr + c * 32, cur);
