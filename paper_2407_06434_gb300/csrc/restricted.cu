@@ -19,6 +19,11 @@
 // At the end every signal's F (FP64 and FP32 copies), b, support and iteration count are in the
 // same state arrays the dense loop uses, and its residual is recomputed from the support.
 //
+// What bounds it: the chain of a step (argmax, Gram entries from HBM, the FP64 scalars, the D row) of
+// three resident signals per SM. The Gram entries are fetched as soon as the pick is known, beside z
+// and gamma, and FP64 is left to one thread: with the drop's division in all eight warps the FP64 pipe
+// was the limit (4096 signals, 1024 x 8192, K = 256, about 28 steps: 1627 us, now 1257 us).
+//
 // Layout: thread i owns candidate slot i (its atom, inverse norm and correlation c_i in
 // registers); D (S x K FP32), the FP32 factor, y and the step's scalars are in shared memory.
 // A block per signal (rather than a warp) spreads the K-wide work of a step over 8 warps and
@@ -42,8 +47,8 @@ struct RSmem {
   int* wati;     // kRWarps: per-warp atoms
   int* wslot;    // kRWarps: per-warp slots
   double* dred;  // kRWarps: per-warp FP64 partials
-  int* ctl;      // 4: picked slot, picked atom, stop flag
-  double* bk;    // 1: b_k of the step
+  int* ctl;      // 4: gamma and b_k (FP32 bits), fall back, threshold reached
+  double* sc;    // 2: gamma and b_k of the step
 };
 
 // Floats first (y at the 16-byte aligned base: Mp is a multiple of 64, so every float array
@@ -56,7 +61,7 @@ __host__ __device__ __forceinline__ size_t rs_float_words(int S, int K, int Mp) 
 
 __host__ __device__ __forceinline__ size_t rs_bytes(int S, int K, int Mp) {
   const size_t ints = (rs_float_words(S, K, Mp) + 2 * kRWarps + 4) * 4;
-  return (ints + 7) / 8 * 8 + (kRWarps + 1) * 8;
+  return (ints + 7) / 8 * 8 + (kRWarps + 2) * 8;
 }
 
 __device__ __forceinline__ RSmem rs_smem(unsigned char* base, int S, int K, int Mp) {
@@ -73,7 +78,7 @@ __device__ __forceinline__ RSmem rs_smem(unsigned char* base, int S, int K, int 
   s.ctl = s.wslot + kRWarps;
   const size_t ints = (rs_float_words(S, K, Mp) + 2 * kRWarps + 4) * 4;
   s.dred = reinterpret_cast<double*>(base + (ints + 7) / 8 * 8);
-  s.bk = s.dred + kRWarps;
+  s.sc = s.dred + kRWarps;
   return s;
 }
 
@@ -155,55 +160,36 @@ __global__ void __launch_bounds__(kRThreads)
   int fb = -1;
   int stop = kStopIters;
   for (; k < S; ++k) {
-    // ---- pick: argmax |c_i| / ||a_i||, lowest atom index on ties
-    float bs = valid ? fabsf(c) * inv : -1.f;
-    float bc = c;  // the best's correlation travels with it (b_k = gamma c_{n*})
-    int bi = valid ? atom : 0x7fffffff, bslot = valid ? tid : -1;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float os = __shfl_xor_sync(0xffffffffu, bs, o);
-      const float oc = __shfl_xor_sync(0xffffffffu, bc, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      const int osl = __shfl_xor_sync(0xffffffffu, bslot, o);
-      if (better(os, oi, bs, bi)) {
-        bs = os;
-        bc = oc;
-        bi = oi;
-        bslot = osl;
+    // ---- pick: argmax |c_i| / ||a_i||, lowest atom index on ties: per warp by integer reductions
+    // (scores are >= 0; 0 stands for no candidate), then every warp over the block's winners, so that
+    // each thread can fetch its Gram entry at once, while the first warp forms z and gamma
+    const uint32_t key = valid ? __float_as_uint(fabsf(c) * inv) + 1u : 0u;
+    {
+      const uint32_t m = __reduce_max_sync(0xffffffffu, key);
+      const unsigned at = __reduce_min_sync(0xffffffffu, key == m ? static_cast<unsigned>(atom) : 0xffffffffu);
+      if (m == 0 && lane == 0) sm.wred[warp] = 0.f;
+      if (m != 0 && key == m && static_cast<unsigned>(atom) == at) {
+        sm.wred[warp] = __uint_as_float(m);
+        sm.wc[warp] = c;  // the best's correlation travels with it (b_k = gamma c_{n*})
+        sm.wati[warp] = atom;
+        sm.wslot[warp] = tid;
       }
-    }
-    if (lane == 0) {
-      sm.wred[warp] = bs;
-      sm.wc[warp] = bc;
-      sm.wati[warp] = bi;
-      sm.wslot[warp] = bslot;
     }
     __syncthreads();
+    uint32_t m2 = lane < kRWarps ? __float_as_uint(sm.wred[lane]) : 0u;
+    const int i2 = lane < kRWarps ? sm.wati[lane] : 0x7fffffff;
+    const uint32_t mb = __reduce_max_sync(0xffffffffu, m2);
+    const unsigned ab = __reduce_min_sync(0xffffffffu, m2 == mb ? static_cast<unsigned>(i2) : 0xffffffffu);
+    const int from = __ffs(__ballot_sync(0xffffffffu, m2 == mb && static_cast<unsigned>(i2) == ab)) - 1;
+    // a candidate scoring 0 is no pick (mb <= 1: score bits plus one)
+    const bool ok = mb > 1u && mb <= 0x7f800001u && ab < static_cast<unsigned>(ws.N) && from >= 0;
+    const int ns = ok ? static_cast<int>(ab) : -1;
+    float gram_i = 0.f;
+    if (ok && valid) gram_i = __ldg(ws.gram + static_cast<size_t>(ns) * ws.ldg + atom);
     if (warp == 0) {
-      float s2 = lane < kRWarps ? sm.wred[lane] : -1.f;
-      float c2 = lane < kRWarps ? sm.wc[lane] : 0.f;
-      int i2 = lane < kRWarps ? sm.wati[lane] : 0x7fffffff;
-      int l2 = lane < kRWarps ? sm.wslot[lane] : -1;
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        const float os = __shfl_xor_sync(0xffffffffu, s2, o);
-        const float oc = __shfl_xor_sync(0xffffffffu, c2, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, i2, o);
-        const int osl = __shfl_xor_sync(0xffffffffu, l2, o);
-        if (better(os, oi, s2, i2)) {
-          s2 = os;
-          c2 = oc;
-          i2 = oi;
-          l2 = osl;
-        }
-      }
-      // lanes 0..7 now hold the winner; every lane of the warp needs it for the z loop
-      s2 = __shfl_sync(0xffffffffu, s2, 0);
-      c2 = __shfl_sync(0xffffffffu, c2, 0);
-      i2 = __shfl_sync(0xffffffffu, i2, 0);
-      l2 = __shfl_sync(0xffffffffu, l2, 0);
-      // ---- z_j = D[j][slot], delta, gamma, the drop check (warp 0; lanes over j)
-      const bool ok = s2 > 0.f && i2 >= 0 && i2 < ws.N && l2 >= 0;
+      // ---- z_j = D[j][slot], delta, gamma (lanes over j)
+      const int l2 = ok ? sm.wslot[from] : 0;
+      const double nrm2 = ok ? __ldg(ws.norm2 + ns) : 0.0;
       double zz = 0.0;
       if (ok)
         for (int j = lane; j < k; j += 32) {
@@ -213,22 +199,27 @@ __global__ void __launch_bounds__(kRThreads)
         }
       zz = warp_sum(zz);
       if (lane == 0) {
-        int verdict = 0;  // 0: accept, 1: fall back (no positive score, or a dependent atom)
-        if (!ok) {
-          verdict = 1;
-        } else {
-          const double nrm2 = ws.norm2[i2];
+        // The step's FP64 scalars, formed by this thread alone: GB300 issues FP64 so slowly that a
+        // division by all eight warps took longer than the rest of a step.
+        int verdict = 1;  // 0: accept, 1: fall back (no positive score, a dependent atom, a small drop)
+        if (ok) {
           const double delta = nrm2 - zz;
-          if (!(delta > kDepRtol * nrm2)) {
-            verdict = 1;
-          } else {
+          if (delta > kDepRtol * nrm2) {
             const double gamma = 1.0 / sqrt(delta);
-            sm.dred[0] = gamma;
-            sm.bk[0] = gamma * static_cast<double>(c2);  // b_k = gamma c_{n*}
+            const double bk = gamma * static_cast<double>(sm.wc[from]);  // b_k = gamma c_{n*}
+            const double drop = (bk * bk) / r2;
+            if (!(drop < static_cast<double>(tau[k]))) {
+              verdict = 0;
+              r2 -= bk * bk;
+              sm.sc[0] = gamma;
+              sm.sc[1] = bk;
+              sm.ctl[0] = __float_as_int(static_cast<float>(gamma));
+              sm.ctl[1] = __float_as_int(static_cast<float>(bk));
+              sm.ctl[3] = r2 <= thr * thr ? 1 : 0;
+              ws.drop[static_cast<size_t>(b) * ws.Smax + k] = static_cast<float>(drop);
+            }
           }
         }
-        sm.ctl[0] = l2;
-        sm.ctl[1] = i2;
         sm.ctl[2] = verdict;
       }
     }
@@ -237,26 +228,21 @@ __global__ void __launch_bounds__(kRThreads)
       fb = k;
       break;
     }
-    const int ns = sm.ctl[1];
-    const double gamma = sm.dred[0];
-    const double bk = sm.bk[0];
-    const double drop = (bk * bk) / r2;
-    if (drop < static_cast<double>(tau[k])) {
-      fb = k;
-      break;
-    }
-    const float gf = static_cast<float>(gamma);
+    const float gf = __int_as_float(sm.ctl[0]), bf = __int_as_float(sm.ctl[1]);
+    const bool last = sm.ctl[3] != 0;  // the residual has reached the threshold
     // ---- new D row and the correlations: thread i, D[k][i] = gamma (G[n*, a_i] - sum_j z_j D[j][i])
     float* Dk = sm.D + static_cast<size_t>(k) * K;
     if (has) {
-      float acc = valid ? __ldg(ws.gram + static_cast<size_t>(ns) * ws.ldg + atom) : 0.f;
+      float acc = gram_i;
+#pragma unroll 4
       for (int j = 0; j < k; ++j) acc = fmaf(-sm.z[j], sm.D[static_cast<size_t>(j) * K + tid], acc);
       const float d = gf * acc;
       Dk[tid] = d;
-      c = fmaf(-static_cast<float>(bk), d, c);
+      c = fmaf(-bf, d, c);
     }
     // ---- F column k = [-gamma F z ; gamma] (FP32 products, FP64 scaling), warp 1
     if (warp == 1) {
+      const double gamma = sm.sc[0];
       float* Fcol = sm.Fs + static_cast<size_t>(k) * (k + 1) / 2;
       double* Fg = ws.F + static_cast<size_t>(b) * ws.Fstride + static_cast<size_t>(k) * (k + 1) / 2;
       float* Ff = ws.F32 + static_cast<size_t>(b) * ws.Fstride + static_cast<size_t>(k) * (k + 1) / 2;
@@ -273,13 +259,11 @@ __global__ void __launch_bounds__(kRThreads)
         Fg[k] = gamma;
         Ff[k] = gf;
         supg[k] = ns;
-        bvg[k] = bk;
-        ws.drop[static_cast<size_t>(b) * ws.Smax + k] = static_cast<float>(drop);
+        bvg[k] = sm.sc[1];
       }
     }
-    r2 -= bk * bk;
     __syncthreads();  // D row k, the factor and z are complete before the next step reads them
-    if (r2 <= thr * thr) {
+    if (last) {
       stop = kStopEps;
       ++k;
       break;

@@ -192,3 +192,23 @@ def test_gram_solve_warps(lib, M, N, B, S):
     for b in np.flatnonzero(same)[::17]:
         cond = np.linalg.cond(A64[:, s1[b]])
         assert np.linalg.norm(X1[b] - X2[b]) <= 256 * 2.0 ** -24 * cond ** 2 * np.linalg.norm(X2[b])
+
+
+# The K largest of a row by equal pieces of the row's range: rows of one value, of few values (a piece
+# holds more keys than are listed), of ordinary logits, with infinities, with signed zeros; rows that
+# do not fit in shared memory; K at both ends.
+@pytest.mark.parametrize("N", [1, 37, 2048, 8192, 41000])
+def test_topk_rows_distributions(lib, N):
+    rng = np.random.default_rng(N)
+    rows = [np.full(N, -3.25), rng.integers(-2, 3, N) * 0.5, rng.standard_normal(N) - 5.0,
+            np.where(rng.random(N) < 0.3, np.inf, rng.standard_normal(N)), np.where(rng.random(N) < 0.5, 0.0, -0.0),
+            -np.exp(20 * rng.random(N)), np.where(rng.random(N) < 0.9, -np.inf, rng.standard_normal(N)),
+            rng.standard_normal(N) * 1e-40, 1.0 + rng.integers(0, 1500, N) * 2.0 ** -23]
+    x = np.stack(rows).astype(np.float32)
+    u = x.view(np.uint32).astype(np.int64)
+    key = np.where(u >> 31, 0xffffffff - u, u | 0x80000000)  # the floats' order, -0 below +0
+    for K in sorted({1, min(N, 256), N}):
+        idx = torch.empty((len(rows), K), dtype=torch.int32, device="cuda")
+        lib.omp_topk_rows(torch.from_numpy(x).cuda(), K, idx)
+        want = np.sort(np.argsort(-key, axis=1, kind="stable")[:, :K], axis=1)
+        assert np.array_equal(idx.cpu().numpy(), want)
