@@ -299,9 +299,13 @@ __device__ __forceinline__ float4 widen(const Slot4<G24>& r) {
   }
 }
 
+// A step in one kernel (kWhole), or, for dictionaries that L2 does not hold, in three launches: kHead
+// up to the append, then gather.cu forms q, then kTail from b on with q read back.
+constexpr int kWhole = 0, kHead = 1, kTail = 2;
+
 // One step of the signal at live position p (p < L), by the block's W warps; every return is
 // taken by the whole block.
-template <int W, int V, bool G24>
+template <int W, int V, bool G24, int MODE>
 __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int p, int S, float eps,
                                                 int eps_rel, unsigned char* smem) {
   const bool top1 = ws.prec == OMP_PREC_FP32;
@@ -317,7 +321,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
   // issued first; they are only read at the merge below.
   Lists l;
   int total = 0;
-  if (!top1 && wig == 0) {
+  if (MODE != kTail && !top1 && wig == 0) {
     total = tc_piece_count(ws, L, p) * kMaxTopk;
     load_lists(ws, total, p, lane, l);
   }
@@ -328,7 +332,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
   // and the rescoring run, and the append waits for them (the first group this warp commits).
   float* Ff = ws.F32 + static_cast<size_t>(id) * ws.Fstride;
   const bool staged = ws.Smax <= kTriMax;
-  if (wig == 0) {
+  if (MODE != kTail && wig == 0) {
     if (staged) {
       const int tn4 = (kk * (kk + 1) / 2 + 3) >> 2;  // within the padded stride
       for (int e = lane; e < tn4; e += 32) cp_async16(gs.tri + 4 * e, Ff + 4 * e);
@@ -353,15 +357,45 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
   const int M4 = ws.Mp >> 2;
   const float4* rrow = reinterpret_cast<const float4*>(ws.R32 + static_cast<size_t>(id) * ws.Mp);
   float4 r[V];
+  if (MODE == kWhole) {
 #pragma unroll
-  for (int t = 0; t < V; ++t) {
-    const int s = t * (W * 32) + wig * 32 + lane;
-    r[t] = s < M4 ? rrow[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int t = 0; t < V; ++t) {
+      const int s = t * (W * 32) + wig * 32 + lane;
+      r[t] = s < M4 ? rrow[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
 
   // ---------------------------------------------------------------- selection
   int ns;
-  if (top1) {
+  auto stage_rows = [&](int n0, int n1) {
+    // the two best merged candidates' FP32 rows and inverse norms, for the next step's
+    // threshold: copied to shared memory in the background (each warp its own slots), read at
+    // the end of the kernel
+    for (int c = 0; c < 2 && c < ws.topk; ++c) {
+      const int n = c ? n1 : n0;
+      if (n < 0) continue;
+      const float4* src = reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp);
+      float4* dst = reinterpret_cast<float4*>(gs.rows + static_cast<size_t>(c) * ws.Mp);
+#pragma unroll
+      for (int t = 0; t < V; ++t) {
+        const int s = t * (W * 32) + wig * 32 + lane;
+        if (s < M4) cp_async16(dst + s, src + s);
+      }
+      if (wig == 0 && lane == c) cp_async4(gs.rinv + c, ws.inv_norm + n);
+    }
+    cp_async_commit();
+    rows_group = true;
+  };
+  if (MODE == kTail) {
+    const int4 sel = ws.sel[p];
+    if (sel.x < 0) return;  // the head ended the signal
+    ns = sel.x;
+    if (wig == 0 && lane == 0) {  // for the threshold below (barriers in between)
+      gs.cidx[0] = sel.y;
+      gs.cidx[1] = sel.z;
+    }
+    if (ws.tau) stage_rows(sel.y, sel.z);
+  } else if (top1) {
     ns = key_index(ws.cand1[p]);
   } else {
     if (wig == 0) {
@@ -408,25 +442,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     group_sync(W, grp);
     const bool skip = gs.scal[2] != 0;
     int nres = gs.scal[3];
-    if (ws.tau) {
-      // the two best merged candidates' FP32 rows and inverse norms, for the next step's
-      // threshold: copied to shared memory in the background (each warp its own slots), read at
-      // the end of the kernel
-      for (int c = 0; c < 2 && c < ws.topk; ++c) {
-        const int n = gs.cidx[c];
-        if (n < 0) continue;
-        const float4* src = reinterpret_cast<const float4*>(ws.A32 + static_cast<size_t>(n) * ws.Mp);
-        float4* dst = reinterpret_cast<float4*>(gs.rows + static_cast<size_t>(c) * ws.Mp);
-#pragma unroll
-        for (int t = 0; t < V; ++t) {
-          const int s = t * (W * 32) + wig * 32 + lane;
-          if (s < M4) cp_async16(dst + s, src + s);
-        }
-        if (wig == 0 && lane == c) cp_async4(gs.rinv + c, ws.inv_norm + n);
-      }
-      cp_async_commit();
-      rows_group = true;
-    }
+    if (MODE == kWhole && ws.tau) stage_rows(gs.cidx[0], ws.topk > 1 ? gs.cidx[1] : -1);
     // FP32 rescoring: every warp dots its residual slice with each candidate's FP32 row, two
     // candidates per pass so their row loads are in flight together. With the bound, a pass
     // starts only if its first candidate (they come best first) could still beat the best FP32
@@ -449,8 +465,9 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
         if (s < M4) {
           const float4 x0 = n0 >= 0 ? __ldg(a0 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
           const float4 x1 = n1 >= 0 ? __ldg(a1 + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-          acc0 += slot_dot<V == 1>(x0, r[t]);
-          acc1 += slot_dot<V == 1>(x1, r[t]);
+          const float4 rv = MODE == kWhole ? r[t] : rrow[s];
+          acc0 += slot_dot<V == 1>(x0, rv);
+          acc1 += slot_dot<V == 1>(x1, rv);
         }
       }
       acc0 = warp_sum_f(acc0);
@@ -509,6 +526,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     if (wig == 0 && lane == 0) {
       atomicOr(ws.err, OMP_DEVERR_BAD_STATE);
       ws.flag[p] = 0;
+      if (MODE == kHead) ws.sel[p] = make_int4(-1, -1, -1, 0);
     }
     return;
   }
@@ -518,7 +536,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
   // so FP64 arithmetic there would add no accuracy. The Schur complement delta, gamma and the
   // stored factor (used by the back-substitution) are FP64.
   double* Fg = ws.F + static_cast<size_t>(id) * ws.Fstride;
-  if (wig == 0) {
+  if (MODE != kTail && wig == 0) {
     // the staged factor and the support have landed (the candidate rows of the threshold,
     // committed after them, may still be in flight) and are visible to the whole warp
     if (rows_group)
@@ -544,20 +562,42 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     }
   }
   group_sync(W, grp);
-  if (gs.scal[1]) {
+  if (MODE != kTail && gs.scal[1]) {
     if (ws.tau) cp_async_wait_all();  // no copy outlives the block
     if (wig == 0 && lane == 0) {
       ws.flag[p] = 0;
       ws.stop[id] = kStopDependent;
+      if (MODE == kHead) ws.sel[p] = make_int4(-1, -1, -1, 0);
     }
+    return;
+  }
+  if (MODE != kTail && ws.margin && wig == 0 && lane == 0) {
+    float mg;
+    if (top1) {  // the correlation's best and runner-up keys (FP32 scores)
+      const unsigned long long k2 = ws.cand2[p];
+      const float s1 = key_score(ws.cand1[p]), s2 = k2 ? key_score(k2) : 0.f;
+      mg = s1 > 0.f ? (s1 - s2) / s1 : 0.f;
+    } else {
+      mg = gs.top2[1];
+    }
+    ws.margin[static_cast<size_t>(id) * ws.Smax + kk] = mg;
+  }
+  if (MODE != kTail && wig == 0 && lane == 0) ws.sup[static_cast<size_t>(id) * ws.Smax + kk] = ns;
+  if (MODE == kHead) {
+    if (wig == 0 && lane == 0)
+      ws.sel[p] = top1 ? make_int4(ns, -1, -1, 0) : make_int4(ns, gs.cidx[0], ws.topk > 1 ? gs.cidx[1] : -1, 0);
     return;
   }
 
   // ---------------------------------------------------------------- q, b, residual update
   float4 q[V];
 #pragma unroll
-  for (int t = 0; t < V; ++t) q[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int na = kk + 1;
+  for (int t = 0; t < V; ++t) {
+    const int s = t * (W * 32) + wig * 32 + lane;
+    q[t] = MODE == kTail && s < M4 ? reinterpret_cast<const float4*>(ws.Q + static_cast<size_t>(p) * ws.Mp)[s]
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const int na = MODE == kTail ? 0 : kk + 1;
   int a = 0;
   // r is not needed during the gather (it is read again below), so its registers carry a third
   // row in flight
@@ -735,19 +775,7 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
     rk = sqrtf(tot);
     const float rn = rk;
     ws.bv[static_cast<size_t>(id) * ws.Smax + kk] = static_cast<double>(bf);
-    ws.sup[static_cast<size_t>(id) * ws.Smax + kk] = ns;
     ws.drop[static_cast<size_t>(id) * ws.Smax + kk] = rprev > 0.f ? (bf / rprev) * (bf / rprev) : 0.f;
-    if (ws.margin) {
-      float mg;
-      if (top1) {  // the correlation's best and runner-up keys (FP32 scores)
-        const unsigned long long k2 = ws.cand2[p];
-        const float s1 = key_score(ws.cand1[p]), s2 = k2 ? key_score(k2) : 0.f;
-        mg = s1 > 0.f ? (s1 - s2) / s1 : 0.f;
-      } else {
-        mg = gs.top2[1];
-      }
-      ws.margin[static_cast<size_t>(id) * ws.Smax + kk] = mg;
-    }
     ws.niter[id] = kk + 1;
     ws.rnorm[id] = rn;
     const float thr = eps_rel ? eps * ynorm : eps;
@@ -812,7 +840,7 @@ __global__ void __launch_bounds__(W * 32, update_min_warps(W, V) / W)
   extern __shared__ __align__(16) unsigned char smem[];
   if (!P) {
     if (static_cast<int>(blockIdx.x) < L)
-      update_position<W, V, G24>(ws, k, L, blockIdx.x, S, eps, eps_rel, smem);
+      update_position<W, V, G24, kWhole>(ws, k, L, blockIdx.x, S, eps, eps_rel, smem);
     return;
   }
   __shared__ int next_p;
@@ -822,8 +850,20 @@ __global__ void __launch_bounds__(W * 32, update_min_warps(W, V) / W)
     const int p = next_p;
     __syncthreads();  // every thread has read it before the next position is taken
     if (p >= L) break;
-    update_position<W, V, G24>(ws, k, L, p, S, eps, eps_rel, smem);
+    update_position<W, V, G24, kWhole>(ws, k, L, p, S, eps, eps_rel, smem);
   }
+}
+
+// The head and tail of a step whose q is gathered apart (gather.cu). The head's chain needs few
+// registers, the tail streams.
+template <int W, int V, int MODE>
+__global__ void __launch_bounds__(W * 32, (MODE == kHead ? 28 : 16) / W)
+    step_part_kernel(Ws ws, int k, int S, float eps, int eps_rel) {
+  k = iter_of(ws, k);
+  const int L = ws.cnt[k + 1];
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (static_cast<int>(blockIdx.x) < L)
+    update_position<W, V, false, MODE>(ws, k, L, blockIdx.x, S, eps, eps_rel, smem);
 }
 
 // resident blocks of one persistent append/update kernel variant on the device (0 if the query
@@ -861,6 +901,13 @@ void launch_g(const Ws& ws, int k, int B, int S, float eps, int eps_rel, cudaStr
 
 template <int W, int V>
 void launch_t(const Ws& ws, int k, int B, int S, float eps, int eps_rel, cudaStream_t s) {
+  if (gather_apart(ws, B)) {
+    const size_t smem = group_bytes(ws);
+    step_part_kernel<W, V, kHead><<<B, W * 32, smem, s>>>(ws, k, S, eps, eps_rel);
+    launch_gather(ws, k, B, s);
+    step_part_kernel<W, V, kTail><<<B, W * 32, smem, s>>>(ws, k, S, eps, eps_rel);
+    return;
+  }
   if (ws.A24h)
     launch_g<W, V, true>(ws, k, B, S, eps, eps_rel, s);
   else
@@ -886,6 +933,11 @@ cudaError_t set_attr_g(int bytes) {
 template <int W, int V>
 cudaError_t set_attr_t(const Ws& ws) {
   const int bytes = static_cast<int>(group_bytes(ws));
+  if (ws.Q) {
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(step_part_kernel<W, V, kHead>), bytes);
+    if (e == cudaSuccess) e = raise_smem_limit(reinterpret_cast<const void*>(step_part_kernel<W, V, kTail>), bytes);
+    if (e != cudaSuccess) return e;
+  }
   return ws.A24h ? set_attr_g<W, V, true>(bytes) : set_attr_g<W, V, false>(bytes);
 }
 

@@ -104,6 +104,8 @@ struct Ws {
                    // window below the row's running best outside which columns are pruned)
   int* ovf;        // FP32 path: positions that need every atom scored in FP32, and their
   int* ovf_cnt;    // number per iteration (Smax + 1)
+  int4* sel;       // per position, a step in parts: its pick (-1: none) and its two best merged candidates
+  float* Q;        // Bmax x Mp, a step in parts: q (null: the dictionary stays in L2)
   uint8_t* flag;
   unsigned long long* cand1;
   float* cand_s;
@@ -361,6 +363,10 @@ void launch_finalize(const Ws& ws, const CallArgs* args, int B, int S, cudaStrea
 void launch_topk_out(const Ws& ws, const CallArgs* args, int B, int topk, cudaStream_t s);
 void launch_set_args(CallArgs* dst, const CallArgs& v, cudaStream_t s);
 cudaError_t configure_update_kernels(const Ws& ws);
+// q gathered by a launch of its own (gather.cu): for the handle's shape, and for a batch of it
+bool gather_apart_shape(int64_t N, int64_t Mp, int64_t Bmax);
+bool gather_apart(const Ws& ws, int B);
+void launch_gather(const Ws& ws, int k, int B, cudaStream_t s);
 int update_slots(int Mp, int W);
 int update_default_warps(int Mp);
 // per warp count (append_w1.cu .. append_w8.cu)

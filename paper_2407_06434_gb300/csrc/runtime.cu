@@ -488,6 +488,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   ok = ok && ar.ask(&ws.livek[0], Bm) && ar.ask(&ws.livek[1], Bm);
   ok = ok && ar.ask(&ws.cnt, Sm + 2) && ar.ask(&ws.kdev, 1) && ar.ask(&ws.flag, Bm) && ar.ask(&ws.cand1, Bm);
   ok = ok && ar.ask(&ws.upd_ctr, Sm + 1);
+  if (gather_apart_shape(ws.N, ws.Mp, ws.Bmax)) ok = ok && ar.ask(&ws.sel, Bm) && ar.ask(&ws.Q, Bm * Mp);
   ok = ok && ar.ask(&ws.score, small_score_floats(ws.N, ws.Bmax));
   ok = ok && ar.ask(&ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
        ar.ask(&ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && ar.ask(&ws.bv, Bm * Sm) &&

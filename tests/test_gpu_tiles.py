@@ -212,3 +212,32 @@ def test_topk_rows_distributions(lib, N):
         lib.omp_topk_rows(torch.from_numpy(x).cuda(), K, idx)
         want = np.sort(np.argsort(-key, axis=1, kind="stable")[:, :K], axis=1)
         assert np.array_equal(idx.cpu().numpy(), want)
+
+
+# A dictionary that L2 does not hold has its gather in a launch of its own for 1024 signals and more:
+# the same bits as the one-kernel step that smaller batches take. Ragged row lengths (the last piece
+# short), every precision, the 24-bit gather, an eps stop that retires signals, margins recorded.
+@pytest.mark.parametrize("prec,M,N,kw", [("fp8", 4000, 11000, {}), ("bf16", 3001, 14002, {}), ("fp32", 2050, 20500, {}),
+                                         ("bf16", 2048, 21000, {"gather24": True}), ("bf16", 8192, 5200, {})])
+def test_gather_apart_is_exact(lib, prec, M, N, kw):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N)
+    B, S = 1100, 9
+    At = torch.randn((N, M), generator=g, device="cuda")
+    At /= At.norm(dim=1, keepdim=True)
+    sup = torch.rand((B, N), generator=g, device="cuda").topk(6).indices
+    coef = torch.randn((B, 6), generator=g, device="cuda")
+    Y = 1e-3 * torch.randn((B, M), generator=g, device="cuda")
+    for j in range(6):
+        Y += coef[:, j, None] * At[sup[:, j]]
+    Y[5] = 0.0
+    for eps, margins in ((0.0, False), (0.3, False), (0.0, not kw)):
+        out = []
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=prec, **kw)
+        for n in (B, 550):
+            parts = [s.solve(At.t(), Y[lo:lo + n].clone(), S, eps, diagnostics=True, margins=margins)
+                     for lo in range(0, B, n)]
+            out.append([torch.cat(p).cpu().numpy() for p in zip(*parts)])
+        s.close()
+        for got, want in zip(*out):
+            assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
