@@ -122,18 +122,21 @@ struct EpiTop8 {
     const int piece = g - tc_owner(s / ws.tc_cl * ws.tc_tn, T, Geff);
     const size_t off =
         (static_cast<size_t>(p) * ws.pieces + EPI_PARTS * piece + part) * kMaxTopk;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      ws.cand_s[off + q] = ts[q];
-      ws.cand_i[off + q] = ti[q];
-    }
+    // a list is one 32-byte sector of each array (slots are multiples of 8 entries)
+    float4* cs = reinterpret_cast<float4*>(ws.cand_s + off);
+    int4* ci = reinterpret_cast<int4*>(ws.cand_i + off);
+    cs[0] = make_float4(ts[0], ts[1], ts[2], ts[3]);
+    cs[1] = make_float4(ts[4], ts[5], ts[6], ts[7]);
+    ci[0] = make_int4(ti[0], ti[1], ti[2], ti[3]);
+    ci[1] = make_int4(ti[4], ti[5], ti[6], ti[7]);
   }
   // The update kernel's lower bound on the row's best score, less three score error bounds
   // (written per live position by the compaction, in the units of the scores); a column at or
   // below it can be neither the pick nor a rescoring candidate that changes it.
   __device__ float load_tau(int s) const {
     const int p = s * BM + row;
-    if (!ws.tau_pos || p >= L) return -1.f;
+    if (p >= L) return INFINITY;  // a tile's rows past the last signal: no column is looked at
+    if (!ws.tau_pos) return -1.f;
     const float v = __ldg(ws.tau_pos + p);
     return v > 0.f ? v : -1.f;
   }
@@ -189,19 +192,64 @@ struct EpiTop8 {
     pf_t = t + 1 < ws.tc_tn ? t + 1 : 0;  // the next unit's column tile (units run t-major)
     pf = load_scales(pf_t);
   }
-  // A compare-only pass marks the columns whose score beats the threshold; only those are
-  // inserted (few per chunk once the list is warm), each read back from the registers with a
-  // select tree, so the warp neither diverges per column nor needs a staging buffer. A fresh list
-  // is seeded, without a per-column loop, with the best column of each group of 4 (lowest index
-  // on ties): those 8 are distinct columns of the chunk, so their smallest score is a safe
-  // threshold for the rest (at least 8 scores reach it), and a high one, which keeps the first
-  // chunk's insertions few. A row with a pruning threshold is not seeded: its threshold already
-  // holds back all but the few columns near the best, so its list may stay short of 8.
+  __device__ void insert(float score, int n) {
+    if (PREC == OMP_PREC_BF16 && ti[1] < 0) {
+      // the list's first or second entry, which is what a list with a pruning threshold sees
+      // most: 10 instructions for 38
+      const bool first = score > ts[0];
+      ts[1] = first ? ts[0] : score;
+      ti[1] = first ? ti[0] : n;
+      ts[0] = first ? score : ts[0];
+      ti[0] = first ? n : ti[0];
+    } else if (score > ts[7]) {
+      top8_insert(ts, ti, score, n);
+    }
+  }
+  // What bounds a chunk is the half-rate integer and compare pipe: every instruction per column
+  // costs 64 cycles a scheduler (two warps on each), and the rows of a warp wait for the row with
+  // the most to insert. So the pass over all columns is one packed multiply for two columns, one
+  // logic operation that makes the key and one maximum (the key carries its column, so the best
+  // column needs no search); only columns that beat the threshold are inserted, each read back
+  // from the registers with a select tree, so the warp neither diverges per column nor needs a
+  // staging buffer; the insertion decides each place on its own instead of bubbling; and rows
+  // past the last signal look at nothing. At 2000 signals x 256 x 1024 (BF16) a chunk takes 1200
+  // cycles where a search, a mask of all columns and a bubbling insertion took 1700, and a step's
+  // correlation 8.1 us instead of 11.0 (2.5 of them from the lists' vector stores: 16 scalar
+  // stores to 32 lines each kept the store unit busy for 4000 cycles); 5000 signals: 13.9 -> 10.9.
+  // A fresh list without a threshold is seeded, without a per-column loop, with the best column
+  // of each group of 4 (lowest index on ties): those 8 are distinct columns of the chunk, so
+  // their smallest score is a safe threshold for the rest (at least 8 scores reach it), and a
+  // high one, which keeps the first chunk's insertions few. A row with a pruning threshold is
+  // not seeded: its threshold already holds back all but the few columns near the best, so its
+  // list may stay short of 8.
   __device__ void chunk(int, int t, int c0, const uint32_t (&cur)[32]) {
     const int nb = t * BN + c0;
     const int lim = min(32, ws.N - nb);
-    const float* scl = scr + (c0 - part * EPI_COLS);
-    const float4* sc4 = reinterpret_cast<const float4*>(scl);
+    const float4* sc4 = reinterpret_cast<const float4*>(scr + (c0 - part * EPI_COLS));
+    unsigned long long peer[EPI_PARTS];  // read ahead of the products that hide the latency
+#pragma unroll
+    for (int o = 1; o < EPI_PARTS; ++o)
+      peer[o] = *reinterpret_cast<volatile unsigned long long*>(peers + (part + o) % EPI_PARTS * BM + row);
+    // The chunk's scores (still with their sign, which every reader drops), and of every group of
+    // four the best column as a key: score bits with the low 5 replaced by 31 - the column's
+    // place, so that an integer max gives the best score and, among scores equal above those
+    // bits, the lowest column. Scores are non-negative, so they order as their bits do (a NaN's
+    // bits above every number's).
+    float sv[32];
+    uint32_t gk[8];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      const float4 sc = sc4[g];
+      mul2(cur[4 * g + 0], cur[4 * g + 1], sc.x, sc.y, sv[4 * g + 0], sv[4 * g + 1]);
+      mul2(cur[4 * g + 2], cur[4 * g + 3], sc.z, sc.w, sv[4 * g + 2], sv[4 * g + 3]);
+      uint32_t kq[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        kq[q] = (__float_as_uint(sv[4 * g + q]) & 0x7fffffe0u) | static_cast<uint32_t>(31 - (4 * g + q));
+      gk[g] = max(max(max(kq[0], kq[1]), kq[2]), kq[3]);
+    }
+    const uint32_t kmax =
+        max(max(max(gk[0], gk[1]), gk[2]), max(max(max(gk[3], gk[4]), gk[5]), max(gk[6], gk[7])));
     uint32_t seeded = 0;
     if (ti[0] < 0 && thr0 < 0.f) {
 #pragma unroll
@@ -211,7 +259,7 @@ struct EpiTop8 {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int j = 4 * g + q;
-          const float v = fabsf(__uint_as_float(cur[j])) * scl[j];
+          const float v = fabsf(sv[j]);
           if (j < lim && v > bv) {  // false for NaN
             bv = v;
             bj = j;
@@ -228,38 +276,15 @@ struct EpiTop8 {
     float thr = fmaxf(ts[7], thr0);
 #pragma unroll
     for (int o = 1; o < EPI_PARTS; ++o) {
-      const int q = (part + o) % EPI_PARTS;
-      const unsigned long long v = *reinterpret_cast<volatile unsigned long long*>(peers + q * BM + row);
-      const float othr = __uint_as_float(static_cast<uint32_t>(v));
-      if (static_cast<int>(v >> 32) == cur_s && othr > 0.f)
+      const float othr = __uint_as_float(static_cast<uint32_t>(peer[o]));
+      if (static_cast<int>(peer[o] >> 32) == cur_s && othr > 0.f)
         thr = fmaxf(thr, __uint_as_float(__float_as_uint(othr) - 1u));
     }
-    // The chunk's scores, as bits, and their largest: scores are non-negative, so they order as
-    // their bits do (a NaN's bits above every number's). One multiply and one integer max per
-    // column; the per-column threshold test and the best-column search below run only for a lane
-    // whose largest score beats its threshold or its list's best key (few, once lists are warm).
-    uint32_t sv[32];
-    uint32_t mbits = 0;
-#pragma unroll
-    for (int j4 = 0; j4 < 8; ++j4) {
-      const float4 sc = sc4[j4];
-      sv[4 * j4 + 0] = __float_as_uint(fabsf(__uint_as_float(cur[4 * j4 + 0])) * sc.x);
-      sv[4 * j4 + 1] = __float_as_uint(fabsf(__uint_as_float(cur[4 * j4 + 1])) * sc.y);
-      sv[4 * j4 + 2] = __float_as_uint(fabsf(__uint_as_float(cur[4 * j4 + 2])) * sc.z);
-      sv[4 * j4 + 3] = __float_as_uint(fabsf(__uint_as_float(cur[4 * j4 + 3])) * sc.w);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) mbits = max(mbits, sv[4 * j4 + q]);
-    }
-    // the list's best column as a key: score bits with the low 5 replaced by 31 - the column's
-    // place, so that among scores equal above those bits the lowest column wins; columns past N
-    // score 0 (zero escale), so they never beat a real column's key
-    if (kTrack && (mbits & ~31u) > (lbk & ~31u)) {  // strictly higher: an earlier column keeps a tie
-      int jb = 31;
-#pragma unroll
-      for (int j = 31; j >= 0; --j)
-        if ((sv[j] & ~31u) == (mbits & ~31u)) jb = j;
-      lbk = (mbits & ~31u) | static_cast<uint32_t>(31 - jb);
-      lbi = nb + jb;
+    // the list's best column; columns past N score 0 (zero escale), so they never beat a real
+    // column's key
+    if (kTrack && (kmax & ~31u) > (lbk & ~31u)) {  // strictly higher: an earlier column keeps a tie
+      lbk = kmax;
+      lbi = nb + 31 - static_cast<int>(kmax & 31u);
     }
     // the window below the running best (lower bounds of scores this thread has seen, this
     // chunk's largest included), rounded down
@@ -267,23 +292,60 @@ struct EpiTop8 {
       const float best = fmaxf(ts[0], __uint_as_float(lbk & ~31u));
       thr = fmaxf(thr, best * (1.f - 0x1p-20f) - win0);
     }
-    // x > thr for x, thr >= 0 exactly when bits(x) > bits(thr); a negative thr (an unfilled list
-    // with no pruning threshold) passes every column
-    uint32_t mask = 0;
-    if (thr < 0.f || mbits > __float_as_uint(thr)) {
+    // Only a lane whose largest score can beat its threshold looks at its columns, and only at
+    // the groups that can (few, once lists are warm): x > thr for x, thr >= 0 exactly when
+    // bits(x) > bits(thr), so only if the bits above the low 5, which the keys hold, are no
+    // smaller; a negative thr (an unfilled list with no pruning threshold) passes every column.
+    const uint32_t tb = thr < 0.f ? 0u : __float_as_uint(thr) & ~31u;
+    uint32_t gmask = 0;
+    if (kmax >= tb) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) mask |= (__uint_as_float(sv[j]) > thr ? 1u : 0u) << j;
-      if (lim < 32) mask &= lim > 0 ? (0xffffffffu >> (32 - lim)) : 0u;
-      mask &= ~seeded;
+      for (int g = 0; g < 8; ++g) gmask |= (gk[g] >= tb ? 1u : 0u) << g;
     }
-    while (mask) {
-      const int j = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const float score = __uint_as_float(pick32(sv, j));
-      if (score > ts[7]) top8_insert(ts, ti, score, nb + j);
+    // Where no row of the warp has more than one group to look at (most chunks past a solve's
+    // first step), a round picks the group's four scores, 28 selects; else every row marks its
+    // columns, 64 instructions once, and a round picks one of them, 31. (Groups always: first
+    // steps 8 % slower; columns always: 5000 x 256 x 1024 11.2 us a step for 10.9. The FP8 lists,
+    // whose wider windows pass more columns, mark them always: 512 x 2048 19.9 us, 20.9 by this
+    // rule.)
+    const uint32_t groups = __reduce_max_sync(0xffffffffu, __popc(gmask));
+    if (PREC == OMP_PREC_BF16 && groups <= 1u) {
+      while (gmask) {
+        const int g = __ffs(gmask) - 1;
+        gmask &= gmask - 1;
+        float v[4];
+        pick_group(sv, g, v);
+        uint32_t mask = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          mask |= (fabsf(v[q]) > thr && 4 * g + q < lim ? 1u : 0u) << q;
+        mask &= ~(seeded >> (4 * g));
+        while (mask) {
+          const int q = __ffs(mask) - 1;
+          mask &= mask - 1;
+          const float lo = q & 1 ? v[1] : v[0], hi = q & 1 ? v[3] : v[2];
+          insert(fabsf(q & 2 ? hi : lo), nb + 4 * g + q);
+        }
+      }
+    } else {
+      uint32_t mask = 0;
+      if (gmask) {
+        uint32_t mq[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 32; ++j) mq[j & 3] |= (fabsf(sv[j]) > thr ? 1u : 0u) << j;
+        mask = (mq[0] | mq[1]) | (mq[2] | mq[3]);
+        if (lim < 32) mask &= lim > 0 ? (0xffffffffu >> (32 - lim)) : 0u;
+        mask &= ~seeded;
+      }
+      while (mask) {
+        const int j = __ffs(mask) - 1;
+        mask &= mask - 1;
+        insert(fabsf(pick32(sv, j)), nb + j);
+      }
     }
-    *reinterpret_cast<volatile unsigned long long*>(peers + part * BM + row) =
-        (static_cast<unsigned long long>(static_cast<uint32_t>(cur_s)) << 32) | __float_as_uint(ts[7]);
+    if (ts[7] > 0.f)  // (a list short of 8 entries tells the other parts nothing)
+      *reinterpret_cast<volatile unsigned long long*>(peers + part * BM + row) =
+          (static_cast<unsigned long long>(static_cast<uint32_t>(cur_s)) << 32) | __float_as_uint(ts[7]);
   }
   __device__ void end(bool ok) {
     if (ok && cur_s >= 0) flush(cur_s);

@@ -270,9 +270,18 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
                : "memory");
 }
 
+// (x0 y0, x1 y1) by one packed multiply, x as FP32 bits; each half rounds as a plain multiply does
+__device__ __forceinline__ void mul2(uint32_t x0, uint32_t x1, float y0, float y1, float& z0, float& z1) {
+  uint64_t x, y, z;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(x0), "r"(x1));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(y0), "f"(y1));
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(z0), "=f"(z1) : "l"(z));
+}
+
 // v[j] for a run-time j without local memory: a 5-level select tree
-__device__ __forceinline__ uint32_t pick32(const uint32_t (&v)[32], int j) {
-  uint32_t a[16];
+__device__ __forceinline__ float pick32(const float (&v)[32], int j) {
+  float a[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) a[i] = (j & 16) ? v[i + 16] : v[i];
 #pragma unroll
@@ -284,24 +293,32 @@ __device__ __forceinline__ uint32_t pick32(const uint32_t (&v)[32], int j) {
   return (j & 1) ? a[1] : a[0];
 }
 
-// Insert (v, n) into a descending top-8; the caller has checked v > s[7]. Equal scores keep
-// the earlier (lower-index) entry in front.
-__device__ __forceinline__ void top8_insert(float (&s)[8], int (&ix)[8], float v, int n) {
-  s[7] = v;
-  ix[7] = n;
+// columns [4 g, 4 g + 4) of v for a run-time g without local memory: a 3-level select tree
+__device__ __forceinline__ void pick_group(const float (&v)[32], int g, float (&o)[4]) {
+  float a[16];
 #pragma unroll
-  for (int q = 7; q > 0; --q) {
-    if (s[q] > s[q - 1]) {
-      const float ts = s[q];
-      s[q] = s[q - 1];
-      s[q - 1] = ts;
-      const int ti = ix[q];
-      ix[q] = ix[q - 1];
-      ix[q - 1] = ti;
-    }
-  }
+  for (int i = 0; i < 16; ++i) a[i] = (g & 4) ? v[i + 16] : v[i];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = (g & 2) ? a[i + 8] : a[i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) o[i] = (g & 1) ? a[i + 4] : a[i];
 }
 
+// Insert (v, n) into a descending top-8; the caller has checked v > s[7]. Equal scores keep
+// the earlier (lower-index) entry in front. Each place is decided on its own, from comparisons
+// with the list as it was (a bubble from the last place is a chain of seven).
+__device__ __forceinline__ void top8_insert(float (&s)[8], int (&ix)[8], float v, int n) {
+  bool above[8];  // v goes before entry q
+#pragma unroll
+  for (int q = 0; q < 8; ++q) above[q] = v > s[q];
+#pragma unroll
+  for (int q = 7; q > 0; --q) {
+    s[q] = above[q - 1] ? s[q - 1] : above[q] ? v : s[q];
+    ix[q] = above[q - 1] ? ix[q - 1] : above[q] ? n : ix[q];
+  }
+  s[0] = above[0] ? v : s[0];
+  ix[0] = above[0] ? n : ix[0];
+}
 
 // ------------------------------------------------------------------------------- mainloop
 // CL = 1: one CTA per unit. CL = 2: a CTA pair on two SMs runs one 256 x 256 MMA per K step
@@ -332,8 +349,9 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap* tm_a, const CUtenso
   const int Tn = col_tiles;
   constexpr int SA = A_BYTES;              // this CTA's A_op tile, then its B_op rows
   constexpr int SS = stage_bytes(CL);
-  const int u0 = static_cast<int>(static_cast<long long>(g) * T / Geff);
-  const int u1 = static_cast<int>(static_cast<long long>(g + 1) * T / Geff);
+  // [g T / Geff, (g + 1) T / Geff), without a 64-bit division
+  const int tq = T / Geff, tr = T - tq * Geff;
+  const int u0 = g * tq + g * tr / Geff, u1 = (g + 1) * tq + (g + 1) * tr / Geff;
 
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;

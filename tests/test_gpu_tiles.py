@@ -241,3 +241,27 @@ def test_gather_apart_is_exact(lib, prec, M, N, kw):
         s.close()
         for got, want in zip(*out):
             assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
+
+
+# The tensor-core lists against the FP32 tiles: ragged row and column tiles, lists of one column tile
+# and of several, duplicate atoms at the edges of groups of 4 and 32 columns and of column tiles (the
+# lowest index wins). The planted coefficients are far apart, so the picks are the same integers.
+@pytest.mark.parametrize("prec", ["bf16", "fp8"])
+@pytest.mark.parametrize("M,N,B", [(128, 253, 1), (256, 300, 129), (256, 1021, 2000), (200, 4099, 700), (512, 1030, 5003)])
+def test_tensor_core_lists_pick_as_fp32(lib, prec, M, N, B):
+    S = 6
+    rng = np.random.default_rng(M + N + B)
+    At = rng.standard_normal((N, M)).astype(np.float32)
+    At /= np.linalg.norm(At, axis=1, keepdims=True)
+    for n in (3, 31, 127, 159, 251):
+        At[n + 1] = At[n]
+    sup = np.stack([rng.choice(N, S, replace=False) for _ in range(B)])
+    coef = rng.permuted(np.tile(1.6 ** np.arange(S, dtype=np.float32), (B, 1)), axis=1)
+    Y = np.einsum("bs,bsm->bm", coef * rng.choice([-1, 1], (B, S)), At[sup]).astype(np.float32)
+    out = []
+    for p in ("fp32", prec):
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=p, use_graph=2)
+        out.append(s.solve(torch.from_numpy(At).cuda().t(), torch.from_numpy(Y).cuda(), 3)[1].cpu().numpy())
+        s.close()
+    assert np.array_equal(out[0][:, :3], out[1][:, :3])
+    assert not np.isin(out[1][:, :3], (4, 32, 128, 160, 252)).any()
