@@ -2,10 +2,13 @@
 // dictionary preparation, the per-iteration launch sequence, CUDA-graph capture and replay.
 //
 // One solve is: set_args, init, compaction 0, then for k = 0..S-1 {correlate(k), update(k),
-// compaction(k+1)}, then finalize. Every kernel reads the live count of its iteration from
-// device memory and returns at once past it, so the whole sequence is launch-invariant: it is
-// captured once per (B, S, eps) into a CUDA graph and replayed with one cudaGraphLaunch, the
-// per-call pointers travelling through a small device-side argument block.
+// compaction(k+1)}, then finalize. On the FP32 path correlate is a BF16 correlation, a selection
+// and an overflow pass (filter.cu); where L2 does not hold the dictionary update is three launches
+// (gather.cu); few signals take a form of their own between init and finalize (small.cu). Every
+// kernel reads the live count of its iteration from device memory and returns at once past it, so
+// the whole sequence is launch-invariant: it is captured once per (B, S, eps) into a CUDA graph and
+// replayed with one cudaGraphLaunch, the per-call pointers travelling through a small device-side
+// argument block.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>

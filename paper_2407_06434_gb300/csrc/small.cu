@@ -9,6 +9,8 @@
 //   wide   a large dictionary and up to 8 signals: per step one launch scores every atom with the
 //          whole GPU (bound by reading the FP32 atom rows from L2), one does the rest with a block
 //          per signal
+// One signal over 1024 x 8192 then takes 13 us a step, 16 signals over 64 x 256 7 us: a chain of
+// short dependent phases, of which the append's FP64 part is 1900 cycles.
 // Scores here are FP32 dot products in an order of their own. An atom can only be the pick if its
 // score is within two error bounds of the best, so those atoms -- mostly one -- are scored again
 // as the batched path of the handle does it (FP32: one chain of FMAs over m; BF16: the rescoring's
