@@ -269,7 +269,9 @@ __device__ __forceinline__ int tc_piece_count(const Ws& ws, int L, int p) {
 // The candidate lists of live position p, spread over a warp: 8 entries per lane, scores as ordered
 // integers (their bits plus one; 0: no entry). load_lists issues the loads of the first 256 entries,
 // settle_lists waits for them. Entries beyond 256 (a small batch's tiles are split over many CTAs)
-// replace a lane's worst: no lane can hold more than 8 of the position's best 8.
+// replace a lane's worst: no lane can hold more than 8 of the position's best 8. Their loads go out
+// four a lane at a time: one after the other they took 3000 cycles of an update at 304 entries (45 us a
+// step for 43 at 4096 signals, 18.1 for 17.5 at 1024).
 struct Lists {
   float s[8];
   int i[8];
@@ -295,21 +297,32 @@ __device__ __forceinline__ void settle_lists(const Ws& ws, int total, int p, int
   const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
   const int* ci = ws.cand_i + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
 #pragma unroll 1
-  for (int e = 256 + lane; e < total; e += 32) {
-    int n = ci[e];
-    if (n < 0) continue;
-    uint32_t v = __float_as_uint(cs[e]) + 1u;
-    // sink the new entry through the lane's eight: each slot keeps the better of the two
+  for (int e0 = 256; e0 < total; e0 += 128) {  // four entries' loads at a time
+    int ni[4];
+    float si[4];
 #pragma unroll
-    for (int t = 0; t < 8; ++t)
-      if (v > l.k[t] || (v == l.k[t] && n < l.i[t])) {
-        const uint32_t ov = l.k[t];
-        const int on = l.i[t];
-        l.k[t] = v;
-        l.i[t] = n;
-        v = ov;
-        n = on;
-      }
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + 32 * u + lane;
+      ni[u] = e < total ? ci[e] : -1;
+      si[u] = e < total ? cs[e] : 0.f;
+    }
+#pragma unroll 1
+    for (int u = 0; u < 4 && e0 + 32 * u < total; ++u) {
+      int n = u == 0 ? ni[0] : u == 1 ? ni[1] : u == 2 ? ni[2] : ni[3];
+      if (n < 0) continue;
+      uint32_t v = __float_as_uint(u == 0 ? si[0] : u == 1 ? si[1] : u == 2 ? si[2] : si[3]) + 1u;
+      // sink the new entry through the lane's eight: each slot keeps the better of the two
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (v > l.k[t] || (v == l.k[t] && n < l.i[t])) {
+          const uint32_t ov = l.k[t];
+          const int on = l.i[t];
+          l.k[t] = v;
+          l.i[t] = n;
+          v = ov;
+          n = on;
+        }
+    }
   }
 }
 // The best remaining entry (highest score, lowest index among equal ones), taken off the lists: its

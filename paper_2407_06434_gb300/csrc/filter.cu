@@ -8,8 +8,9 @@
 // range, goes on a list for which every atom is scored in FP32 (launch_corr_overflow).
 //
 // The full FP32 correlation of 1000 signals with 8192 atoms of length 1024 takes 309 us a step, the
-// BF16 one 32, this kernel 10 and the (mostly empty) overflow launch 3.5. This kernel is bound by the
-// latency of a position's round trips and of its chain (four cycles an element).
+// BF16 one 20, this kernel 9.7 and the (mostly empty) overflow launch 3.5. This kernel is bound by the
+// latency of a position's round trips and of its chain (four cycles an element at best); with chunks of
+// 256 elements it takes 9.4 there, but 122 registers a thread instead of 80 cost a large batch residency.
 #include "common.cuh"
 
 namespace ompk {
@@ -18,6 +19,7 @@ namespace {
 constexpr int kWarpsF = 4;   // warps (positions) per block
 constexpr int kMaxC = 7;     // candidates scored here
 constexpr int kCh = 128;     // elements of a row staged at a time
+constexpr int kBatch = 4;   // 16-byte reads ahead of a chain
 constexpr int kLd = kCh + 4; // padded: the lanes' 16-byte reads of different rows meet no bank twice
 
 __global__ void __launch_bounds__(32 * kWarpsF) filter_select_kernel(Ws ws, int k) {
@@ -86,13 +88,30 @@ __global__ void __launch_bounds__(32 * kWarpsF) filter_select_kernel(Ws ws, int 
     if (lane < n) {
       const float4* a = reinterpret_cast<const float4*>(st + lane * kLd);
       const float4* r = reinterpret_cast<const float4*>(st + kMaxC * kLd);
-#pragma unroll 8
-      for (int s = 0; s < kCh / 4; ++s) {  // past Mp both are zero, which adds nothing
-        const float4 x = a[s], y = r[s];
-        acc = fmaf(y.x, x.x, acc);
-        acc = fmaf(y.y, x.y, acc);
-        acc = fmaf(y.z, x.z, acc);
-        acc = fmaf(y.w, x.w, acc);
+      // past Mp both are zero, which adds nothing; the reads go a batch ahead of the chain, which
+      // waited for each before (13.7 cycles an element, 9 now: the next chunk's loads are the rest)
+      float4 x[2][kBatch], y[2][kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        x[0][q] = a[q];
+        y[0][q] = r[q];
+      }
+#pragma unroll
+      for (int s = 0; s < kCh / 4; s += kBatch) {
+        const int cur = s / kBatch & 1;
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q)
+          if (s + kBatch < kCh / 4) {
+            x[cur ^ 1][q] = a[s + kBatch + q];
+            y[cur ^ 1][q] = r[s + kBatch + q];
+          }
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+          acc = fmaf(y[cur][q].x, x[cur][q].x, acc);
+          acc = fmaf(y[cur][q].y, x[cur][q].y, acc);
+          acc = fmaf(y[cur][q].z, x[cur][q].z, acc);
+          acc = fmaf(y[cur][q].w, x[cur][q].w, acc);
+        }
       }
     }
   }

@@ -145,7 +145,7 @@ def _solve_both(lib, monkeypatch, A, Y, S, eps, graph=1, **kw):
 @pytest.mark.parametrize("M,N,B,S,planted,eps,graph", [
     (64, 300, 700, 12, 12, 0.0, 1), (256, 1000, 300, 40, 20, 0.0, 1), (203, 1500, 129, 24, 24, 1e-2, 1),
     (1024, 4100, 257, 24, 16, 0.0, 1), (1024, 4100, 200, 20, 20, 1e-2, 2), (2100, 2500, 70, 16, 16, 0.0, 0),
-    (640, 8000, 1100, 8, 4, 0.0, 1)])
+    (640, 8000, 1100, 8, 4, 0.0, 1), (256, 9001, 200, 12, 12, 0.0, 1)])
 def test_fp32_filter_is_exact(lib, monkeypatch, M, N, B, S, planted, eps, graph):
     A, Y = _planted(M, N, B, planted, M + N + B)
     Y[3] = 0.0
@@ -247,7 +247,8 @@ def test_gather_apart_is_exact(lib, prec, M, N, kw):
 # and of several, duplicate atoms at the edges of groups of 4 and 32 columns and of column tiles (the
 # lowest index wins). The planted coefficients are far apart, so the picks are the same integers.
 @pytest.mark.parametrize("prec", ["bf16", "fp8"])
-@pytest.mark.parametrize("M,N,B", [(128, 253, 1), (256, 300, 129), (256, 1021, 2000), (200, 4099, 700), (512, 1030, 5003)])
+@pytest.mark.parametrize("M,N,B", [(128, 253, 1), (256, 300, 129), (256, 1021, 2000), (200, 4099, 700), (512, 1030, 5003),
+                                   (256, 9001, 200)])
 def test_tensor_core_lists_pick_as_fp32(lib, prec, M, N, B):
     S = 6
     rng = np.random.default_rng(M + N + B)
