@@ -14,7 +14,7 @@
 // EPI_PARTS (g - owner(s * Tn)) + part, so a tile's lists occupy consecutive slots; the
 // mainloop's minimum units per CTA (`cmin`) bounds the pieces per tile by kPieces / EPI_PARTS. (With
 // 32 lists a position 8192 atoms took three units a CTA at least: 1000 signals ran on 85 CTAs, 32 us a
-// step at K = 1024; with 68 it is one unit, and 22 us.)
+// step at K = 1024; with 68 it is one unit, and 22 us, 20 since the scan below was shortened.)
 //
 // Each row may carry a pruning threshold from the previous step's update (a lower bound on its
 // best score less three score error bounds, see append.cuh): columns at or below it are not

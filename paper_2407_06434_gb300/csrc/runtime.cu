@@ -161,8 +161,9 @@ Ws solve_ws(const omp_handle_s* h, int B, bool stats) {
   Ws w = h->ws;
   // The FP32 path's filter pays from about 3e8 products a step on, and for rows of 256 elements and
   // more always: the tile kernel then takes a chain of that many products at least. Measured, us a
-  // step with and without: 64 x 256, 2000 signals 29 / 22; 128 x 512, 2000 29 / 25; 100 x 8000, 500
-  // 35 / 42; 256 x 1024, 1000 29 / 30; 512 x 2048, 16 28 / 41; 256 x 1024, 5000 43 / 79.
+  // step with and without: 64 x 256, 2000 signals 29 / 23; 128 x 512, 2000 29 / 27; 128 x 1024, 4000
+  // 33 / 48; 100 x 8000, 500 31 / 43; 256 x 512, 100 22 / 22; 256 x 1024, 1000 28 / 32; 512 x 2048,
+  // 16 27 / 42; 256 x 1024, 5000 44 / 81.
   if (w.filt && (stats || (w.Mp < 256 && static_cast<double>(w.N) * w.Mp * B < 3e8))) no_filter(w);
   if (stats) {
     w.margin = h->margin_buf;
