@@ -267,6 +267,12 @@ bool capture_while_solve(omp_handle_s* h, const Ws& ws, int B, int S, float eps,
 void enqueue_topk(omp_handle_s* h, const float* R, int B, int topk, cudaStream_t s) {
   Ws ws = h->ws;
   if (ws.filt) no_filter(ws);  // the score is an output
+  // the lists are the output: no threshold, and no window, which is sized by the residual norms and
+  // quantisation errors of a solve's signals
+  ws.tau = nullptr;
+  ws.tau_pos = nullptr;
+  ws.win_pos = nullptr;
+  ws.ea = nullptr;
   launch_load_rows(ws, R, B, s);
   launch_compact(ws, 0, B, 1, false, s);
   enqueue_correlate(h, ws, 0, B, s);

@@ -1,0 +1,67 @@
+"""Values and sizes at the edges of what the kernels' shortcuts assume."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2407_06434_gb300 import build
+    build.build()
+    from paper_2407_06434_gb300 import omp
+    omp.load()
+    return omp
+
+
+def _planted(M, N, B, S, seed, sigma=1e-3):
+    rng = np.random.default_rng(seed)
+    At = rng.standard_normal((N, M))
+    At = (At / np.linalg.norm(At, axis=1, keepdims=True)).astype(np.float32)
+    sup = np.stack([rng.choice(N, S, replace=False) for _ in range(B)])
+    Y = np.einsum("bs,bsm->bm", rng.standard_normal((B, S)), At[sup].astype(np.float64))
+    Y += sigma * rng.standard_normal((B, M))
+    return torch.from_numpy(At).cuda(), torch.from_numpy(Y.astype(np.float32)).cuda(), sup
+
+
+def _words(out):
+    return [t.cpu().numpy().view(np.uint32) for t in out]
+
+
+def _quantised(x, prec):
+    """Rows as the correlation multiplies them, in FP64, and each row's scale."""
+    if prec == "bf16":
+        return x.bfloat16().double(), torch.ones(x.shape[0], dtype=torch.float64, device=x.device)
+    amax = x.abs().amax(dim=1, keepdim=True)
+    return (x * (448.0 / amax)).to(torch.float8_e4m3fn).double(), (amax[:, 0] / 448.0).double()
+
+
+# omp_correlate_topk is one correlation of its own: what a solve left on the handle (its signals'
+# residual norms, thresholds) does not enter its lists. A score is within the accumulation's
+# Mp 2^-22 and four roundings of the product of the quantised rows, so the list's j-th score is within
+# that of the j-th largest.
+@pytest.mark.parametrize("prec", ["bf16", "fp8"])
+def test_topk_after_a_solve(lib, prec):
+    M, N, B, S = 256, 2000, 200, 24
+    At, Y, _ = _planted(M, N, B, 6, 3, sigma=0.0)
+    s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=prec)
+    s.solve(At.t(), Y, S)               # residuals far below the rows' norms that follow
+    R = 30.0 * torch.from_numpy(np.random.default_rng(4).standard_normal((B, M)).astype(np.float32)).cuda()
+    idx = torch.empty((B, 8), dtype=torch.int32, device="cuda")
+    sc = torch.empty((B, 8), device="cuda")
+    lib.omp_correlate_topk(s.h, At.t(), R, 8, idx, sc)
+    s.close()
+    qa, sa = _quantised(At, prec)
+    qr, _ = _quantised(R, prec)
+    scale = sa / torch.linalg.vector_norm(At.double(), dim=1)
+    score = (qr @ qa.t()).abs() * scale
+    tol = (M * 2.0 ** -22 + 4 * 2.0 ** -24) * torch.linalg.vector_norm(qr, dim=1, keepdim=True) * (
+        torch.linalg.vector_norm(qa, dim=1) * scale).max()
+    assert all(len(set(row)) == 8 and min(row) >= 0 for row in idx.tolist())
+    own = score.gather(1, idx.long())
+    assert bool(((sc.double() - own).abs() <= tol).all())
+    assert bool(((sc.double() - score.topk(8, dim=1).values).abs() <= tol).all())
