@@ -267,11 +267,13 @@ __device__ __forceinline__ int tc_piece_count(const Ws& ws, int L, int p) {
 }
 
 // The candidate lists of live position p, spread over a warp: 8 entries per lane, scores as ordered
-// integers (their bits plus one; 0: no entry). load_lists issues the loads of the first 256 entries,
+// integers (their bits plus one; 0: no entry, or a NaN, which as an integer would stand above every score:
+// an atom that is not finite, or products that overflowed). load_lists issues the loads of the first 256 entries,
 // settle_lists waits for them. Entries beyond 256 (a small batch's tiles are split over many CTAs)
 // replace a lane's worst: no lane can hold more than 8 of the position's best 8. Their loads go out
 // four a lane at a time: one after the other they took 3000 cycles of an update at 304 entries (45 us a
 // step for 43 at 4096 signals, 18.1 for 17.5 at 1024).
+constexpr uint32_t kInfBits = 0x7f800000u;
 struct Lists {
   float s[8];
   int i[8];
@@ -290,8 +292,9 @@ __device__ __forceinline__ void load_lists(const Ws& ws, int total, int p, int l
 __device__ __forceinline__ void settle_lists(const Ws& ws, int total, int p, int lane, Lists& l) {
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
-    const bool ok = l.i[t] >= 0;  // an unfilled list entry is -1
-    l.k[t] = ok ? __float_as_uint(l.s[t]) + 1u : 0u;  // scores are >= 0
+    const uint32_t v = __float_as_uint(l.s[t]);  // scores are >= 0
+    const bool ok = l.i[t] >= 0 && v <= kInfBits;  // an unfilled list entry is -1
+    l.k[t] = ok ? v + 1u : 0u;
     if (!ok) l.i[t] = 0x7fffffff;
   }
   const float* cs = ws.cand_s + static_cast<size_t>(p) * ws.pieces * kMaxTopk;
@@ -309,8 +312,9 @@ __device__ __forceinline__ void settle_lists(const Ws& ws, int total, int p, int
 #pragma unroll 1
     for (int u = 0; u < 4 && e0 + 32 * u < total; ++u) {
       int n = u == 0 ? ni[0] : u == 1 ? ni[1] : u == 2 ? ni[2] : ni[3];
-      if (n < 0) continue;
-      uint32_t v = __float_as_uint(u == 0 ? si[0] : u == 1 ? si[1] : u == 2 ? si[2] : si[3]) + 1u;
+      uint32_t v = __float_as_uint(u == 0 ? si[0] : u == 1 ? si[1] : u == 2 ? si[2] : si[3]);
+      if (n < 0 || v > kInfBits) continue;
+      ++v;
       // sink the new entry through the lane's eight: each slot keeps the better of the two
 #pragma unroll
       for (int t = 0; t < 8; ++t)

@@ -65,3 +65,24 @@ def test_topk_after_a_solve(lib, prec):
     own = score.gather(1, idx.long())
     assert bool(((sc.double() - own).abs() <= tol).all())
     assert bool(((sc.double() - score.topk(8, dim=1).values).abs() <= tol).all())
+
+
+# An atom with a NaN or an infinity has no score: the solve goes as if it were zero, also at the steps
+# whose thresholds leave a list nothing but that atom.
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8"])
+@pytest.mark.parametrize("B", [1, 300])
+def test_atoms_that_are_not_finite(lib, prec, B):
+    M, N, S = 256, 2000, 12
+    At, Y, sup = _planted(M, N, B, 6, 5)
+    bad = [n for n in (0, 130, 700, 1300, 1999) if n not in set(sup.ravel())] or [2]
+    out = []
+    for v in (0.0, float("nan"), float("inf")):
+        D = At.clone()
+        D[bad] = 0.0
+        D[bad, 7] = v
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=prec)
+        out.append(_words(s.solve(D.t(), Y, S, diagnostics=True)))
+        s.close()
+    for got in out[1:]:
+        for g, want in zip(got, out[0]):
+            assert np.array_equal(g, want)
