@@ -159,6 +159,9 @@ __device__ __forceinline__ float approx_score(float dot, float inv) {
   return inv == 0.f || (inv > 1e-15f && inv < 1e15f) ? fabsf(dot) * inv : __int_as_float(0x7fffffff);
 }
 
+// the larger of two scores, a NaN if either is one
+__device__ __forceinline__ float max_keep_nan(float a, float b) { return a != a || a > b ? a : b; }
+
 __device__ __forceinline__ void load_head(float (&head)[8], const float* gm, int NG) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -451,7 +454,7 @@ __device__ __forceinline__ void score_atoms(const Ws& ws, const float4* rows, co
       for (int o = LPA / 2; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
       const int n = n0 + u * GP + grp;
       const float v = approx_score(acc[u], inv[u]);
-      if (n < N) best = v >= best ? v : best > v ? best : v;  // a NaN stays
+      if (n < N) best = max_keep_nan(best, v);
       if (sub == 0 && n < N) sc[n] = v;
     }
     if (gm && lane == 0) gm[n0 / U] = best;
@@ -554,7 +557,7 @@ __global__ void __launch_bounds__(kT) wide_score_kernel(Ws ws, int B) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const float v = approx_score(warp_sum_f(acc[u][i]), inv[u]);
-          if (n0 + u < N) best = v >= best ? v : best > v ? best : v;  // a NaN stays
+          if (n0 + u < N) best = max_keep_nan(best, v);
           if (lane == 0 && n0 + u < N) sc[n0 + u] = v;
         }
         if (lane == 0) sc[N + n0 / U] = best;

@@ -86,3 +86,25 @@ def test_atoms_that_are_not_finite(lib, prec, B):
     for got in out[1:]:
         for g, want in zip(got, out[0]):
             assert np.array_equal(g, want)
+
+
+# Few signals over a large dictionary: an atom far from unit norm is scored again wherever it stands
+# among the four atoms that share a recorded maximum.
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("B", [1, 4])
+@pytest.mark.parametrize("scale", [1e18, 1e-18])
+def test_few_signals_far_norms_at_any_place(lib, prec, B, scale):
+    M, N, S = 512, 1027, 4
+    At, _, _ = _planted(M, N, 1, 1, 6)
+    atoms = [400, 405, 410, 415]                 # places 0, 1, 2, 3 of their fours
+    Y = 3.0 * At[atoms] + At[[100, 200, 300, 500]]
+    At[atoms] *= scale
+    for lo in range(0, 4, B):
+        out = []
+        for graph in (1, 2):                     # the device-side loop runs the batched kernels
+            s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=prec, use_graph=graph)
+            out.append(_words(s.solve(At.t(), Y[lo:lo + B].clone(), S, diagnostics=True)))
+            s.close()
+        assert out[0][1][:, 0].tolist() == atoms[lo:lo + B]
+        for g, want in zip(*out):
+            assert np.array_equal(g, want)
