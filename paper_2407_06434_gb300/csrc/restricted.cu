@@ -161,9 +161,10 @@ __global__ void __launch_bounds__(kRThreads)
   int stop = kStopIters;
   for (; k < S; ++k) {
     // ---- pick: argmax |c_i| / ||a_i||, lowest atom index on ties: per warp by integer reductions
-    // (scores are >= 0; 0 stands for no candidate), then every warp over the block's winners, so that
+    // (scores are >= 0; 0 stands for no candidate or a NaN), then every warp over the block's winners, so that
     // each thread can fetch its Gram entry at once, while the first warp forms z and gamma
-    const uint32_t key = valid ? __float_as_uint(fabsf(c) * inv) + 1u : 0u;
+    const float score = fabsf(c) * inv;
+    const uint32_t key = valid && score == score ? __float_as_uint(score) + 1u : 0u;
     {
       const uint32_t m = __reduce_max_sync(0xffffffffu, key);
       const unsigned at = __reduce_min_sync(0xffffffffu, key == m ? static_cast<unsigned>(atom) : 0xffffffffu);
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kRThreads)
     const unsigned ab = __reduce_min_sync(0xffffffffu, m2 == mb ? static_cast<unsigned>(i2) : 0xffffffffu);
     const int from = __ffs(__ballot_sync(0xffffffffu, m2 == mb && static_cast<unsigned>(i2) == ab)) - 1;
     // a candidate scoring 0 is no pick (mb <= 1: score bits plus one)
-    const bool ok = mb > 1u && mb <= 0x7f800001u && ab < static_cast<unsigned>(ws.N) && from >= 0;
+    const bool ok = mb > 1u && ab < static_cast<unsigned>(ws.N) && from >= 0;
     const int ns = ok ? static_cast<int>(ab) : -1;
     float gram_i = 0.f;
     if (ok && valid) gram_i = __ldg(ws.gram + static_cast<size_t>(ns) * ws.ldg + atom);

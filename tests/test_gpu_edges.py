@@ -108,3 +108,29 @@ def test_few_signals_far_norms_at_any_place(lib, prec, B, scale):
         assert out[0][1][:, 0].tolist() == atoms[lo:lo + B]
         for g, want in zip(*out):
             assert np.array_equal(g, want)
+
+
+def test_candidate_that_is_not_finite(lib):
+    """A candidate atom with a NaN is passed over by the restricted steps."""
+    M, N, B, S, K = 256, 1000, 50, 6, 40
+    At, Y, sup = _planted(M, N, B, S, 7)
+    rng = np.random.default_rng(8)
+    bad = next(n for n in range(N) if n not in set(sup.ravel()))
+    At[bad, 3] = float("nan")
+    cand = np.stack([np.concatenate([r, rng.choice([n for n in range(N) if n != bad and n not in set(r)], K - S,
+                                                   replace=False)]) for r in sup]).astype(np.int32)
+    out = []
+    for place in (bad, -1):                      # -1: no candidate
+        c = cand.copy()
+        c[:, -1] = place
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision="bf16")
+        X = torch.empty((B, S), device="cuda")
+        so = torch.empty((B, S), dtype=torch.int32, device="cuda")
+        fb = torch.empty(B, dtype=torch.int32, device="cuda")
+        lib.omp_solve_batch_candidates(s.h, At.t(), Y, S, 0.0, torch.from_numpy(c).cuda(),
+                                       torch.zeros(S, device="cuda"), X, so, fallback_out=fb)
+        out.append(_words((X, so, fb)))
+        s.close()
+    assert (out[1][2].view(np.int32) == -1).all()
+    for g, want in zip(*out):
+        assert np.array_equal(g, want)
