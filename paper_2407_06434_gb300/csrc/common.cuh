@@ -58,6 +58,7 @@ struct alignas(16) TauRec {
 
 struct Ws {
   int M, Mp, N, Smax, Bmax, Bpad;
+  int sms;         // SMs of the handle's device
   int prec;        // omp_precision
   int filt;        // FP32 path: BF16 tensor-core scores and a bound leave the few atoms that FP32
                    // scores decide between (filter.cu); 0: every atom scored in FP32

@@ -329,7 +329,6 @@ void launch_one(const Ws& ws, int rows, int k, cudaStream_t s) {
 // 99 / 70 / 50, of 8192 of length 1024 1148 / 1180 / 1192.
 template <int MODE>
 void launch_tiles(const Ws& ws, int rows, int k, cudaStream_t s) {
-  constexpr int kSms = 152;
   int best = 16;
   double least = 0.0;
   for (int tn = 16; tn >= 8; tn -= 4) {
@@ -339,7 +338,7 @@ void launch_tiles(const Ws& ws, int rows, int k, cudaStream_t s) {
       tiles = 0;
       for (int by = 0; by < rts; ++by) tiles += cols - (by * BM) / (TX * tn);
     }
-    const double rounds = tiles <= kSms ? 1.25 : static_cast<double>((tiles + kSms - 1) / kSms);
+    const double rounds = tiles <= ws.sms ? 1.25 : static_cast<double>((tiles + ws.sms - 1) / ws.sms);
     if (least == 0.0 || rounds * tn < least) {
       least = rounds * tn;
       best = tn;

@@ -398,7 +398,7 @@ cudaError_t configure_gram_solve(const Ws& ws) {
 void launch_gram_solve(const Ws& ws, const CallArgs*, int B, int S, float eps, int eps_rel,
                        cudaStream_t s) {
   const size_t smem = gs_bytes(ws.N, S);
-  const int W = gram_warps(ws.N, B, ws.tc_grid > 0 ? ws.tc_grid : 152);
+  const int W = gram_warps(ws.N, B, ws.sms);
   if (W == 1)
     gram_solve_kernel<1><<<B, 32, smem, s>>>(ws, B, S, eps, eps_rel);
   else if (W == 4)

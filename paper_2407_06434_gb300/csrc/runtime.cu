@@ -433,6 +433,7 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   h->dev = d.device;
   h->sm_count = sms;
   Ws& ws = h->ws;
+  ws.sms = sms;
   ws.M = static_cast<int>(d.M);
   // one tensor-core K stage is 128 bytes: 64 BF16 or 128 E4M3 elements
   const int64_t malign = d.precision == OMP_PREC_FP8_E4M3 ? 2 * kMpAlign : kMpAlign;
