@@ -234,6 +234,13 @@ __device__ __forceinline__ bool squares_ok(double s) { return s > 1e-20 && s < 1
 __device__ __forceinline__ int iter_of(const Ws& ws, int k) { return k >= 0 ? k : *ws.kdev; }
 
 
+// FP32 path: whether step k goes without the filter, as after a step that left more than three quarters
+// of its positions undecided (near copies, long rows at the noise floor); every fourth step tries again.
+__device__ __forceinline__ bool filter_rests(const Ws& ws, int k) {
+  if ((k & 3) == 0) return false;
+  return 4ll * __ldg(ws.ovf_cnt + k - 1) > 3ll * __ldg(ws.cnt + k);
+}
+
 // Persistent schedule of the tensor-core correlation (shared by the correlation kernel, which
 // writes candidate slots, and the kernels that merge them). The G CTAs form clusters of CL, and
 // cluster rank r works on signal tile s = CL sg + r of each group sg of CL consecutive tiles.
@@ -362,7 +369,7 @@ cudaError_t raise_smem_limit(const void* kernel, size_t bytes);
 void launch_prep(const Ws& ws, const float* A, cudaStream_t s);
 void launch_gram_simt(const Ws& ws, cudaStream_t s);
 void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s);
-void launch_corr_overflow(const Ws& ws, int k, cudaStream_t s);
+void launch_corr_overflow(const Ws& ws, int k, int B, cudaStream_t s);
 void launch_filter_select(const Ws& ws, int k, int B, cudaStream_t s);
 void launch_c0_simt(const Ws& ws, int B, cudaStream_t s);
 cudaError_t configure_corr_simt(const Ws& ws);

@@ -45,6 +45,17 @@ __device__ __forceinline__ unsigned long long dup2(float x) {
 constexpr int BM = 128, BK = 32;
 constexpr int TX = 8, THREADS = 128;  // threads along the atoms; 16 along the rows, 8 rows each
 
+// kOverflow: a block holds two groups of threads, each with tiles, shared memory and barrier of its own
+template <int MODE>
+constexpr int kGroups = MODE == kOverflow ? 2 : 1;
+template <int MODE>
+__device__ __forceinline__ void tile_sync() {
+  if (MODE == kOverflow)
+    asm volatile("bar.sync %0, %1;" ::"r"(static_cast<int>(threadIdx.x) / THREADS + 1), "r"(THREADS) : "memory");
+  else
+    __syncthreads();
+}
+
 // One tile: rows by * 128 .., atoms bx * 8 TN ..; L rows in all
 template <int MODE, int TN>
 __device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, const int* live, const int* ovf) {
@@ -53,9 +64,9 @@ __device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, c
   constexpr int RS = THREADS / (BK / 4);             // rows apart of a thread's loads (16)
   constexpr int LX = BM / RS / 2, LA = BN / RS / 2;  // loads per thread and half chunk
   extern __shared__ __align__(16) float smem_f[];
-  float* Xs = smem_f;                // 2 x BK x BM
-  float* As = smem_f + 2 * BK * BM;  // 2 x BK x BN
-  const int tid = threadIdx.x;
+  float* Xs = smem_f + (kGroups<MODE> > 1 ? threadIdx.x / THREADS * (2 * BK * (BM + BN)) : 0);  // 2 x BK x BM
+  float* As = Xs + 2 * BK * BM;                                                                // 2 x BK x BN
+  const int tid = kGroups<MODE> > 1 ? threadIdx.x % THREADS : threadIdx.x;
   const int n0 = bx * BN;
   const int p0 = by * BM;
   // a warp loads 4 rows x 128 bytes (whole lines); element (k, r) of a chunk is stored at column
@@ -130,7 +141,7 @@ __device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, c
   sstore(0, 0);
   gload(0, 1);
   sstore(0, 1);
-  __syncthreads();
+  tile_sync<MODE>();
   for (int kt = 0; kt < nk; ++kt) {
     const int buf = kt & 1;
     const bool more = kt + 1 < nk;
@@ -157,7 +168,7 @@ __device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, c
       }
     }
     if (more) sstore(buf ^ 1, 1);
-    __syncthreads();
+    tile_sync<MODE>();
   }
   auto acc = [&](int i, int j) { return (j & 1) ? hi2(acc2[i][j >> 1]) : lo2(acc2[i][j >> 1]); };
 
@@ -275,14 +286,14 @@ __device__ __forceinline__ void simt_tile(const Ws& ws, int bx, int by, int L, c
 }
 
 // MODE kCorrelate: k is the iteration; kGram: k unused; kStoreC: k is the number of signals;
-// kOverflow: as kCorrelate for the positions that the filter could not decide (a launch of one row of
-// tiles, walked down).
+// kOverflow: as kCorrelate for the positions that the filter could not decide (their number is not
+// known at the launch: a grid that fills the SMs strides over the tiles).
 // TN atoms per thread: a tile of 128 rows x 8 TN atoms.
 template <int MODE, int TN>
-__global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
+__global__ void __launch_bounds__(THREADS * kGroups<MODE>, 2 / kGroups<MODE>) simt_tile_kernel(Ws ws, int k) {
   constexpr bool GRAM = MODE == kGram;
   constexpr int BN = TX * TN;
-  const int bx = blockIdx.x, by = blockIdx.y;
+  const int bx = blockIdx.x, by = blockIdx.y;  // (kOverflow: the grid is one row)
   // G is symmetric and every entry's products and sums are the same in both orders, so only tiles
   // that reach the diagonal or lie above it are computed, and each stores its mirror image too
   if (GRAM && bx * BN + BN <= by * BM) return;
@@ -300,9 +311,11 @@ __global__ void __launch_bounds__(THREADS, 2) simt_tile_kernel(Ws ws, int k) {
     ovf = ws.ovf;
   }
   if (MODE == kOverflow) {
-    for (int r = 0; r * BM < L; ++r) {
-      simt_tile<MODE, TN>(ws, bx, r, L, live, ovf);
-      __syncthreads();  // the next tile overwrites the chunks
+    const int cols = (ws.N + BN - 1) / BN, tiles = (L + BM - 1) / BM * cols;
+    const int grp = threadIdx.x / THREADS;  // (no tile for the second group before every block has one)
+    for (int t = blockIdx.x + grp * gridDim.x; t < tiles; t += 2 * gridDim.x) {
+      simt_tile<MODE, TN>(ws, t % cols, t / cols, L, live, ovf);
+      tile_sync<MODE>();  // the next tile overwrites the chunks
     }
     return;
   }
@@ -367,16 +380,23 @@ cudaError_t configure_corr_simt(const Ws& ws) {
   cudaError_t e = set_tile_limits<kGram>();
   if (e == cudaSuccess && ws.prec == OMP_PREC_FP32) e = set_tile_limits<kCorrelate>();
   if (e == cudaSuccess && ws.filt)
-    e = raise_smem_limit(reinterpret_cast<const void*>(simt_tile_kernel<kOverflow, 8>), tile_bytes<8>());
+    e = raise_smem_limit(reinterpret_cast<const void*>(simt_tile_kernel<kOverflow, 8>), 2 * tile_bytes<8>());
   return e;
 }
 cudaError_t configure_c0_simt() { return set_tile_limits<kStoreC>(); }
 
 void launch_corr_simt(const Ws& ws, int k, int B, cudaStream_t s) { launch_tiles<kCorrelate>(ws, B, k, s); }
 
-// Mostly no position is left over: one narrow row of tiles that returns at once
-void launch_corr_overflow(const Ws& ws, int k, cudaStream_t s) {
-  simt_tile_kernel<kOverflow, 8><<<(ws.N + 8 * TX - 1) / (8 * TX), THREADS, tile_bytes<8>(), s>>>(ws, k);
+// Mostly no position is left over, and the blocks return at once (1.7 us). Where a few are, each block
+// has one tile of its own SM; where many are (near copies, long rows at the noise floor), two, side by
+// side, which hide each other's latency as two blocks do. (A grid of two blocks an SM puts some first
+// tiles on one SM: 1000 signals x 8192 atoms x 1024, a step 52.2 us for 50.2.) Every position, us a step
+// here / one row of blocks / without the filter: 40 near copies of each atom, 256 x 1024, 5000 signals
+// 113 / 804 / 80; 1024 x 8192, 1000 signals 368 / 552 / 322; noise floor, 8064 x 1207, 1200 signals
+// 723 / 4352 / 723.
+void launch_corr_overflow(const Ws& ws, int k, int B, cudaStream_t s) {
+  const long long tiles = static_cast<long long>((ws.N + 8 * TX - 1) / (8 * TX)) * ((B + BM - 1) / BM);
+  simt_tile_kernel<kOverflow, 8><<<tiles < ws.sms ? static_cast<int>(tiles) : ws.sms, 2 * THREADS, 2 * tile_bytes<8>(), s>>>(ws, k);
 }
 
 void launch_c0_simt(const Ws& ws, int B, cudaStream_t s) { launch_tiles<kStoreC>(ws, B, B, s); }

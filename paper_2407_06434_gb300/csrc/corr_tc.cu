@@ -359,8 +359,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     corr_tc_kernel(const __grid_constant__ CUtensorMap tm_r0, const __grid_constant__ CUtensorMap tm_r1,
                    const __grid_constant__ CUtensorMap tm_a, Ws ws, int k) {
   k = iter_of(ws, k);
+  const bool rests = ws.filt && filter_rests(ws, k);  // (its loads beside the next one)
   const int L = ws.cnt[k + 1];
-  if (L <= 0) return;
+  if (L <= 0 || rests) return;
   EpiTop8<PREC> epi;
   epi.ws = ws;
   epi.L = L;

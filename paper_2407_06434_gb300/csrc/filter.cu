@@ -5,7 +5,9 @@
 // warp per position takes those: one alone is the pick; up to seven are scored in FP32 exactly as
 // corr_simt.cu scores them (one chain of FMAs over m), so the pick is the one a full FP32 correlation
 // makes. A position with more (the lists may then lack some), or whose norm leaves FP32's normal
-// range, goes on a list for which every atom is scored in FP32 (launch_corr_overflow).
+// range, goes on a list for which every atom is scored in FP32 (launch_corr_overflow). After a step that
+// left most positions on that list the next ones up to a multiple of four do without the filter: the BF16
+// correlation returns at once and the list holds every position (filter_rests).
 //
 // The full FP32 correlation of 1000 signals with 8192 atoms of length 1024 takes 309 us a step, the
 // BF16 one 20, this kernel 9.7 and the (mostly empty) overflow launch 3.5. This kernel is bound by the
@@ -25,10 +27,16 @@ constexpr int kLd = kCh + 4; // padded: the lanes' 16-byte reads of different ro
 __global__ void __launch_bounds__(32 * kWarpsF) filter_select_kernel(Ws ws, int k) {
   __shared__ __align__(16) float stage[kWarpsF][(kMaxC + 1) * kLd];
   k = iter_of(ws, k);
+  const bool rests = filter_rests(ws, k);
   const int L = ws.cnt[k + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int p = blockIdx.x * kWarpsF + warp;
   if (p >= L) return;  // the whole warp
+  if (rests) {
+    if (lane == 0) ws.ovf[p] = p;
+    if (p == 0 && lane == 0) ws.ovf_cnt[k] = L;
+    return;
+  }
   Lists l;
   const int total = tc_piece_count(ws, L, p) * kMaxTopk;
   load_lists(ws, total, p, lane, l);

@@ -143,7 +143,7 @@ void enqueue_correlate(omp_handle_s* h, const Ws& ws, int k, int B, cudaStream_t
   launch_corr_tc(ws, h->tc, k, B, s);
   if (ws.filt) {
     launch_filter_select(ws, k, B, s);
-    launch_corr_overflow(ws, k, s);
+    launch_corr_overflow(ws, k, B, s);
   }
 }
 

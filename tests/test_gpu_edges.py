@@ -134,3 +134,65 @@ def test_candidate_that_is_not_finite(lib):
     assert (out[1][2].view(np.int32) == -1).all()
     for g, want in zip(*out):
         assert np.array_equal(g, want)
+
+
+def _near_copies(M, N, B, seed):
+    """40 near copies of each of N / 40 atoms: FP32's filter decides almost no pick between them."""
+    base, _, _ = _planted(M, (N + 39) // 40, 1, 1, seed)
+    noise, _, _ = _planted(M, N, 1, 1, seed + 1)
+    At = base.repeat_interleave(40, 0)[:N] + 1e-3 * noise
+    At /= At.norm(dim=1, keepdim=True)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    sup = torch.rand((B, N), generator=g, device="cuda").topk(5).indices
+    coef = torch.randn((B, 5), generator=g, device="cuda")
+    Y = 1e-3 * torch.randn((B, M), generator=g, device="cuda")
+    for j in range(5):
+        Y += coef[:, j, None] * At[sup[:, j]]
+    return At, Y
+
+
+# Positions that the filter leaves to FP32 in numbers: more row tiles than one pass of the blocks, few
+# and many column tiles, half of the positions only, steps that go without the filter and steps that try
+# it again; the same words as with every atom scored in FP32.
+@pytest.mark.parametrize("M,N,B,plain,graph", [(256, 2000, 2600, 0, 1), (300, 200, 4000, 0, 2), (256, 2000, 1500, 750, 0),
+                                               (1030, 4100, 300, 0, 1)])
+def test_fp32_overflow_is_exact(lib, monkeypatch, M, N, B, plain, graph):
+    At, Y = _near_copies(M, N, B, M + N)
+    if plain:  # signals that the filter decides: atoms of their own
+        D, Yp, _ = _planted(M, N, plain, 5, 9)
+        At = torch.cat([At[:N // 2], D[:N // 2]])
+        Y[:plain] = D[:N // 2][torch.arange(plain, device="cuda") % (N // 2)] + 0.3 * Yp
+    out = []
+    for hook in ("0", "1"):
+        monkeypatch.setenv("OMP_RESCORE_ALWAYS", hook)
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=10, precision="fp32", use_graph=graph)
+        out.append(_words(s.solve(At.t(), Y, 10, diagnostics=True)))
+        s.close()
+    for g, want in zip(*out):
+        assert np.array_equal(g, want)
+
+
+def _solve_ms(s, At, Y, S):
+    ts = []
+    for _ in range(8):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        s.solve(At.t(), Y, S)
+        b.record()
+        torch.cuda.synchronize()
+        ts.append(a.elapsed_time(b))
+    return min(ts)
+
+
+def test_fp32_overflow_fills_the_gpu(lib, monkeypatch):
+    """Where the filter decides nothing, a solve takes less than twice the time without it (one row of
+    16 blocks took ten times)."""
+    At, Y = _near_copies(256, 1024, 5000, 1)
+    ms = []
+    for hook in ("0", "1"):
+        monkeypatch.setenv("OMP_RESCORE_ALWAYS", hook)
+        s = lib.OmpSolver(256, 1024, max_batch=5000, max_iters=16, precision="fp32")
+        ms.append(_solve_ms(s, At, Y, 16))
+        s.close()
+    assert ms[0] < 2.0 * ms[1], ms
