@@ -196,3 +196,20 @@ def test_fp32_overflow_fills_the_gpu(lib, monkeypatch):
         ms.append(_solve_ms(s, At, Y, 16))
         s.close()
     assert ms[0] < 2.0 * ms[1], ms
+
+
+# Each few-signal form gives way where the batched kernels are faster: more signals than its resident
+# blocks take in a round or two, more atoms than a block scores quickly, more products than the tensor
+# cores need long for. The device-side loop always runs the batched kernels (and takes a few us a step
+# more), so a solve that chooses takes no longer.
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("M,N,B", [(64, 128, 3000), (64, 256, 1500), (64, 4096, 16), (128, 512, 360), (256, 1024, 60),
+                                   (128, 2048, 16), (4096, 6000, 8)])
+def test_few_signal_forms_give_way(lib, prec, M, N, B):
+    At, Y, _ = _planted(M, N, B, 6, M + N)
+    ms = []
+    for graph in (1, 2):
+        s = lib.OmpSolver(M, N, max_batch=B, max_iters=12, precision=prec, use_graph=graph)
+        ms.append(_solve_ms(s, At, Y, 12))
+        s.close()
+    assert ms[0] < 1.1 * ms[1], ms
