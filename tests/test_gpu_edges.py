@@ -213,3 +213,53 @@ def test_few_signal_forms_give_way(lib, prec, M, N, B):
         ms.append(_solve_ms(s, At, Y, 12))
         s.close()
     assert ms[0] < 1.1 * ms[1], ms
+
+
+def _handle_bytes(lib, *args, **kw):
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    s = lib.OmpSolver(*args, **kw)
+    used = free - torch.cuda.mem_get_info()[0]
+    s.close()
+    return used
+
+
+# Bytes a signal of a handle's workspaces: the residual and its two quantised copies, 32 candidate lists
+# at most, the factor in FP64 and FP32, the traces, the staged signals and results.
+@pytest.mark.parametrize("prec,M,N", [("bf16", 256, 1024), ("bf16", 64, 3000), ("fp8", 128, 256), ("fp32", 64, 100)])
+def test_workspace_per_signal(lib, prec, M, N):
+    S = 8
+    B = 46000 if prec == "fp32" else 100000      # (46,000 signals of the FP32 size never use the filter)
+    per = (_handle_bytes(lib, M, N, max_batch=B, max_iters=S, precision=prec) -
+           _handle_bytes(lib, M, N, max_batch=B // 2, max_iters=S, precision=prec)) / (B - B // 2)
+    tri = (S * (S + 1) // 2 + 3) // 4 * 4
+    rows = 4 * M + {"fp32": 0, "bf16": 4 * M, "fp8": 2 * M}[prec] + 4 * M
+    lists = 0 if prec == "fp32" else 32 * 64
+    assert per <= rows + lists + 12 * tri + (8 + 4 * 5) * S + 120, per
+
+
+# A handle whose workspaces do not fit does without those that only make solves faster, and gives the
+# same words; one that does not fit without them either is refused.
+@pytest.mark.parametrize("prec,M,N,B", [("fp32", 300, 700, 3000), ("bf16", 200, 9000, 16000), ("fp8", 3000, 15000, 1100)])
+def test_workspaces_that_do_not_fit(lib, monkeypatch, prec, M, N, B):
+    S = 6
+    At, Y, _ = _planted(M, N, 200, S, M)
+    Y = Y.repeat((B + 199) // 200, 1)[:B].contiguous()
+    kw = dict(max_batch=B, max_iters=S, precision=prec)
+    full = _handle_bytes(lib, M, N, **kw)
+    out, used = [], []
+    for limit in (None, full - (4 << 20)):       # (allocations come in pages of 2 MB)
+        if limit:
+            monkeypatch.setenv("OMP_FAULT_ALLOC_BYTES", str(limit))
+        used.append(_handle_bytes(lib, M, N, **kw))
+        s = lib.OmpSolver(M, N, **kw)
+        out.append(_words(s.solve(At.t(), Y, S, diagnostics=True)))
+        few = s.solve(At.t(), Y[:20].clone(), S)[1]
+        assert torch.equal(few, torch.from_numpy(out[0][1][:20].astype(np.int32)).cuda())
+        s.close()
+    assert used[1] < used[0]
+    for g, want in zip(*out):
+        assert np.array_equal(g, want)
+    monkeypatch.setenv("OMP_FAULT_ALLOC_BYTES", str(1 << 20))
+    with pytest.raises(lib.OmpError):
+        lib.OmpSolver(M, N, **kw)
