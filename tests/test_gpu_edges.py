@@ -263,3 +263,21 @@ def test_workspaces_that_do_not_fit(lib, monkeypatch, prec, M, N, B):
     monkeypatch.setenv("OMP_FAULT_ALLOC_BYTES", str(1 << 20))
     with pytest.raises(lib.OmpError):
         lib.OmpSolver(M, N, **kw)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_autotune_of_few_signals(lib, monkeypatch, tmp_path, prec):
+    """Solves of few signals launch none of the kernels that the tuner times: it keeps the handle's
+    shapes and records nothing, except where the device-side loop runs the batched kernels."""
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("OMP_AUTOTUNE_CACHE", str(cache))
+    At, Y, _ = _planted(64, 256, 16, 6, 2)
+    for graph in (1, 0, 2):
+        s = lib.OmpSolver(64, 256, max_batch=16, max_iters=8, precision=prec, use_graph=graph)
+        before = lib.omp_tuning(s.h)
+        choice = lib.omp_autotune(s.h, At.t(), Y, 8, 0.0, repeats=1)
+        assert choice == lib.omp_tuning(s.h)[0]
+        if graph != 2:
+            assert lib.omp_tuning(s.h) == before and not cache.exists()
+        s.close()
+    assert len(cache.read_text().splitlines()) == 1
