@@ -32,6 +32,8 @@ constexpr int kGS = 4;                             // wide: scores per recorded 
 constexpr int kSmallMaxB = 8;                      // wide: signals that share one pass over A
 constexpr int64_t kWideMaxElems = 24ll << 20;      // wide: FP32 rows of at most 96 MB stay in L2
 constexpr int64_t kWideMaxRows = 48 * 1024;         // wide: residuals in shared memory (192 KB)
+constexpr int64_t kWideMaxWork = 144ll << 20;       // wide: products of a step; past it the tile kernel, for
+constexpr int64_t kWideMaxWork16 = 96ll << 20;      //   BF16 handles the tensor cores, score faster
 constexpr int64_t kSoloMaxElems = 1ll << 18;       // solo: at most 1 MB of atom rows a step and block
 constexpr int64_t kSoloMaxTotal = 24ll << 20;      // solo: at most 96 MB a step over all signals
 constexpr size_t kSmallMaxSmem = 100 * 1024;       // solo: two blocks an SM at least
@@ -637,10 +639,33 @@ void by_slots(int V, F f) {
 int small_form(const Ws& ws, int B) {
   if (ws.prec == OMP_PREC_FP8_E4M3 || ws.A24h || ws.margin) return 0;
   if (ws.prec == OMP_PREC_BF16 && (ws.topk != kMaxTopk || !(ws.rescore_eps > 0.f))) return 0;
+  const bool fp32 = ws.prec == OMP_PREC_FP32;
   const int64_t elems = static_cast<int64_t>(ws.N) * ws.Mp;
-  if (elems <= kSoloMaxElems && elems * B <= kSoloMaxTotal && small_bytes(ws.Mp, ws.Smax, ws.N, 0) <= kSmallMaxSmem)
-    return 1;
-  if (B <= kSmallMaxB && elems <= kWideMaxElems && static_cast<int64_t>(ws.Mp) * B <= kWideMaxRows) return 2;
+  if (elems <= kSoloMaxElems && elems * B <= kSoloMaxTotal && small_bytes(ws.Mp, ws.Smax, ws.N, 0) <= kSmallMaxSmem) {
+    // Two blocks fit on an SM, so a step takes rounds of 4 us and a time an atom: 20 ns and 20 for four
+    // passes of a warp over its row (15 where a block has an SM to itself), 8 for each pass left over,
+    // 9.5 in all for rows of 64. Against it stands the batched step. Measured, us a step solo / batched
+    // FP32 / batched BF16: 64 x 128 300 signals 9.7 / 21 / 23, 900 19.4 / 22.0 / 24.0, 1200 24.4 / 22.6 / 23.6;
+    // 64 x 256 600 signals 15.1 / 20.0 / 21.8, 900 21.2 / 20.5 / 22.4, 1500 34 / 21 / 23; 64 x 1024 300 17.1 /
+    // 20.7 / 22.3, 310 29.8 / 20.8 / 22.6; 64 x 4096 16 41 / 19 / 21; 128 x 512 300 19.4 / 23.3 / 21.0, 310
+    // 35 / 24 / 21; 128 x 2048 16 52 / 21 / 20; 256 x 512 100 21.9 / 26 / 21; 256 x 1024 16 36 / 24 / 19;
+    // 400 x 512 10 30.6 / 26 / 21; 512 x 512 10 20.8 / 26 / 21; 1024 x 256 64 17.5 / 34 / 28.
+    const int rounds = (B + 2 * ws.sms - 1) / (2 * ws.sms), M4 = ws.Mp / 4;
+    const int left = (M4 % 128 + 31) / 32;
+    const double atom = ws.Mp == 64 ? 9.5e-3 : 1e-3 * (20 + M4 / 128 * (B <= ws.sms ? 15 : 20) + 8 * left);
+    const double batched = !fp32 ? 19.0 + ws.Mp / 170.0 : ws.Mp == 64 ? 19.5 : 22.0 + ws.Mp / 100.0;
+    if (rounds * (4.0 + ws.N * atom) <= batched) return 1;
+  }
+  // Wide scores every atom for each signal on the CUDA cores and keeps the residuals in shared memory.
+  // Measured, us a step wide / batched FP32 / batched BF16: 1024 x 8192 1 signal 13.6 / 32 / 28, 8 24.4 /
+  // 36 / 28.5; 2048 x 8192 6 28.8 / 41 / 33, 8 33.6 / 44 / 32.8; 4096 x 3000 6 37 / 53 / 38, 8 44 / 58 / 39;
+  // 4096 x 6000 3 34 to 43 / 53 / 40, 4 43 / 54 / 40, 6 51 / 57 / 41, 8 87 / 72 / 42; 700 x 30000 4 38 / 45 / 41,
+  // 6 47 / 45 / 41, 8 55 / 45 / 41; 8192 x 600 3 43 / 81 / 57, 6 57 / 75 / 57; 8192 x 3000 1 50 to 59 / 70 / 56,
+  // 2 67 / 73 / 57, 6 92 / 87 / 58.
+  const int64_t work = fp32 ? kWideMaxWork : ws.Mp <= 4096 ? kWideMaxWork16 : kWideMaxWork16 / 4;
+  if (B <= kSmallMaxB && elems <= kWideMaxElems && elems * B <= work &&
+      static_cast<int64_t>(ws.Mp) * B <= (fp32 ? kWideMaxRows : kWideMaxRows / 2))
+    return 2;
   return 0;
 }
 
