@@ -89,7 +89,8 @@ typedef struct omp_desc {
 void omp_desc_default(omp_desc* desc, int64_t M, int64_t N);
 
 /* Create a handle: checks the device (sm_103 only), allocates every workspace for max_batch and
- * max_iters (including the N x N FP32 Gram matrix), and returns it in *out. No dictionary is
+ * max_iters (including the N x N FP32 Gram matrix), and returns it in *out. Where they do not fit
+ * it does without those that only make solves faster. No dictionary is
  * prepared yet. Returns OMP_ERR_UNSUPPORTED_DEVICE on any other device, OMP_ERR_OUT_OF_MEMORY if
  * an allocation fails (nothing is leaked). */
 omp_status omp_create(const omp_desc* desc, omp_handle* out);

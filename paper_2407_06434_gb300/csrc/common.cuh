@@ -43,6 +43,7 @@ constexpr int kSigTile = 128;         // signals per correlation tile (TMEM lane
 constexpr int kMaxTopk = 8;
 constexpr int kTauSmax = 64;          // the BF16 pruning threshold is kept for max_iters <= 64
 constexpr int kPieces = 68;           // candidate lists per position at most (tensor-core paths)
+constexpr int kLeanPieces = 32;       // the same for a handle whose full layout does not fit in memory
 constexpr int kTcParts = 2;           // candidate lists per signal and correlation CTA
 constexpr double kDepRtol = 1e-10;    // dependent-atom test: delta <= 1e-10 ||a||^2
 constexpr int kStopIters = 0, kStopEps = 1, kStopDependent = 2, kStopZero = 3;
@@ -424,8 +425,7 @@ bool proposal_run_inference(omp_proposal p, const float* A, const float* Y, int 
 
 // tensor-core correlation (corr_tc.cu)
 struct TcPlan;
-int tc_pieces();
-void tc_fill_sched(Ws& ws, int sm_count);
+void tc_fill_sched(Ws& ws, int sm_count, int max_pieces);
 cudaError_t tc_setup(const Ws& ws, int sm_count, TcPlan** plan);
 void tc_destroy(TcPlan* plan);
 void launch_corr_tc(const Ws& ws, const TcPlan* plan, int k, int B, cudaStream_t s);

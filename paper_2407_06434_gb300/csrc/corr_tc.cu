@@ -12,7 +12,7 @@
 // The EPI_PARTS epilogue warps of a lane quarter see different column parts of each unit, so each
 // keeps its own list; a CTA flushes them for signal tile s into candidate slots
 // EPI_PARTS (g - owner(s * Tn)) + part, so a tile's lists occupy consecutive slots; the
-// mainloop's minimum units per CTA (`cmin`) bounds the pieces per tile by kPieces / EPI_PARTS. (With
+// mainloop's minimum units per CTA (`cmin`) bounds the pieces per tile by ws.pieces / EPI_PARTS. (With
 // 32 lists a position 8192 atoms took three units a CTA at least: 1000 signals ran on 85 CTAs, 32 us a
 // step at K = 1024; with 68 it is one unit, and 22 us, 20 since the scan below was shortened.)
 //
@@ -379,16 +379,16 @@ struct TcPlan {
   int grid;
 };
 
-int tc_pieces() { return kPieces; }
-
-void tc_fill_sched(Ws& ws, int sm_count) {
+// The schedule and the lists a position needs: at most max_pieces, fewer where the atoms have few tiles
+void tc_fill_sched(Ws& ws, int sm_count, int max_pieces) {
   ws.tc_grid = sm_count;
   ws.tc_stages = STAGES;
   ws.tc_cl = 1;
   ws.tc_tn = (ws.N + BN - 1) / BN;
   // a tile of Tn units meets at most ceil(Tn / cmin) + 1 CTA ranges of >= cmin units
-  constexpr int kMaxPieces = kPieces / EPI_PARTS;
-  ws.tc_cmin = (ws.tc_tn + (kMaxPieces - 2) - 1) / (kMaxPieces - 2);
+  const int ranges = max_pieces / EPI_PARTS - 2;
+  ws.tc_cmin = (ws.tc_tn + ranges - 1) / ranges;
+  ws.pieces = EPI_PARTS * ((ws.tc_tn + ws.tc_cmin - 1) / ws.tc_cmin + 1);
 }
 
 namespace {

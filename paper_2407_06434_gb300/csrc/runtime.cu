@@ -77,6 +77,9 @@ bool fault_alloc_due() {
 
 bool device_alloc(omp_handle_s* h, void** p, size_t bytes) {
   *p = nullptr;
+  // test hook: OMP_FAULT_ALLOC_BYTES=n makes allocations of more than n bytes fail
+  const char* v = std::getenv("OMP_FAULT_ALLOC_BYTES");
+  if (v && bytes > std::strtoull(v, nullptr, 10)) return false;
   if (cudaMalloc(p, bytes) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -147,6 +150,13 @@ void enqueue_correlate(omp_handle_s* h, const Ws& ws, int k, int B, cudaStream_t
   }
 }
 
+// The FP32 path's filter pays from about 3e8 products a step on, and for rows of 256 elements and
+// more always: the tile kernel then takes a chain of that many products at least. Measured, us a
+// step with and without: 64 x 256, 2000 signals 29 / 23; 128 x 512, 2000 29 / 27; 128 x 1024, 4000
+// 33 / 48; 100 x 8000, 500 31 / 43; 256 x 512, 100 22 / 22; 256 x 1024, 1000 28 / 32; 512 x 2048,
+// 16 27 / 42; 256 x 1024, 5000 44 / 81.
+bool filter_pays(const Ws& w, int B) { return w.Mp >= 256 || static_cast<double>(w.N) * w.Mp * B >= 3e8; }
+
 // FP32 path: every atom scored in FP32
 void no_filter(Ws& w) {
   w.filt = 0;
@@ -159,12 +169,7 @@ void no_filter(Ws& w) {
 // rescored in FP32, no pruning), which picks the same atoms (the exactness tests compare the two).
 Ws solve_ws(const omp_handle_s* h, int B, bool stats) {
   Ws w = h->ws;
-  // The FP32 path's filter pays from about 3e8 products a step on, and for rows of 256 elements and
-  // more always: the tile kernel then takes a chain of that many products at least. Measured, us a
-  // step with and without: 64 x 256, 2000 signals 29 / 23; 128 x 512, 2000 29 / 27; 128 x 1024, 4000
-  // 33 / 48; 100 x 8000, 500 31 / 43; 256 x 512, 100 22 / 22; 256 x 1024, 1000 28 / 32; 512 x 2048,
-  // 16 27 / 42; 256 x 1024, 5000 44 / 81.
-  if (w.filt && (stats || (w.Mp < 256 && static_cast<double>(w.N) * w.Mp * B < 3e8))) no_filter(w);
+  if (w.filt && (stats || !filter_pays(w, B))) no_filter(w);
   if (stats) {
     w.margin = h->margin_buf;
     w.cand2 = w.prec == OMP_PREC_FP32 ? h->cand2_buf : nullptr;
@@ -456,67 +461,72 @@ omp_status omp_create(const omp_desc* desc, omp_handle* out) {
   // padded to 4 entries so each signal's FP32 factor starts on a 16-byte boundary
   ws.Fstride = (static_cast<int64_t>(ws.Smax) * (ws.Smax + 1) / 2 + 3) / 4 * 4;
   ws.upd_w = update_default_warps(ws.Mp);
-  // The FP32 path filters its atoms with a BF16 correlation. (The test hook that turns the score
-  // bound off turns this off too.)
   const bool hook = always && std::atoi(always) == 1;
-  ws.filt = d.precision == OMP_PREC_FP32 && !hook ? 1 : 0;
-  ws.tcprec = ws.filt ? OMP_PREC_BF16 : ws.prec;
-  const bool tc = ws.tcprec != OMP_PREC_FP32;
-  ws.pieces = tc ? tc_pieces() : 0;
   ws.tc_cl = 1;
-  if (tc) tc_fill_sched(ws, h->sm_count);
   const size_t N = ws.N, Mp = ws.Mp, Bm = ws.Bmax, Bp = ws.Bpad, Sm = ws.Smax;
-  const size_t qbytes = ws.tcprec == OMP_PREC_BF16 ? 2 : 1;
-  Arena ar;
-  bool ok = true;
-  ok = ok && ar.ask(&ws.A32, N * Mp);
-  if (d.gather24) ok = ok && ar.ask(&ws.A24h, N * Mp) && ar.ask(&ws.A24l, N * Mp);
-  if (ws.tcprec == OMP_PREC_BF16) ok = ok && ar.ask(&ws.A16, N * Mp);
-  if (d.precision == OMP_PREC_FP8_E4M3) ok = ok && ar.ask(&ws.A8, N * Mp) && ar.ask(&ws.sa, N);
   const size_t Npad = (N + 255) / 256 * 256;
-  if (tc) ok = ok && ar.ask(&ws.escale, Npad);
-  ok = ok && ar.ask(&ws.inv_norm, N) && ar.ask(&ws.norm2, N) && ar.ask(&ws.gram, N * ws.ldg);
-  ok = ok && ar.ask(&ws.R32, Bm * Mp);
-  if (tc) {
-    ok = ok && ar.ask(reinterpret_cast<uint8_t**>(&ws.Rq[0]), Bp * Mp * qbytes) &&
-         ar.ask(reinterpret_cast<uint8_t**>(&ws.Rq[1]), Bp * Mp * qbytes);
-    ok = ok && ar.ask(&ws.sr[0], Bp) && ar.ask(&ws.sr[1], Bp);
-    ok = ok && ar.ask(&ws.cand_s, Bp * ws.pieces * kMaxTopk) &&
-         ar.ask(&ws.cand_i, Bp * ws.pieces * kMaxTopk);
-  }
-  // The pruning thresholds (and the data-driven bound they carry): on BF16 always; on E4M3,
-  // whose worst-case bound is too loose to prune, only where the one-warp update quantises the
-  // next row itself and so can measure its rounding error (padded lengths up to 1024).
-  const bool want_tau = ws.prec == OMP_PREC_BF16 ||
-                        (ws.prec == OMP_PREC_FP8_E4M3 && update_default_warps(ws.Mp) == 1);
-  if (want_tau && ws.rescore_eps > 0.f && ws.Smax <= kTauSmax)
-    ok = ok && ar.ask(&ws.tau, Bm) && ar.ask(&ws.tau_pos, Bp) && ar.ask(&ws.win_pos, Bp) &&
-         (ws.prec != OMP_PREC_FP8_E4M3 || ar.ask(&ws.ea, 1));
-  if (ws.filt)
-    ok = ok && ar.ask(&ws.win_pos, Bp) && ar.ask(&ws.ea, 1) && ar.ask(&ws.ovf, Bm) &&
-         ar.ask(&ws.ovf_cnt, Sm + 1);
-  ok = ok && ar.ask(&ws.live[0], Bm) && ar.ask(&ws.live[1], Bm);
-  ok = ok && ar.ask(&ws.livek[0], Bm) && ar.ask(&ws.livek[1], Bm);
-  ok = ok && ar.ask(&ws.cnt, Sm + 2) && ar.ask(&ws.kdev, 1) && ar.ask(&ws.flag, Bm) && ar.ask(&ws.cand1, Bm);
-  ok = ok && ar.ask(&ws.upd_ctr, Sm + 1);
-  if (gather_apart_shape(ws.N, ws.Mp, ws.Bmax)) ok = ok && ar.ask(&ws.sel, Bm) && ar.ask(&ws.Q, Bm * Mp);
-  ok = ok && ar.ask(&ws.score, small_score_floats(ws.N, ws.Bmax));
-  ok = ok && ar.ask(&ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
-       ar.ask(&ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && ar.ask(&ws.bv, Bm * Sm) &&
-       ar.ask(&ws.sup, Bm * Sm);
-  ok = ok && ar.ask(&ws.drop, Bm * Sm) && ar.ask(&ws.fb, Bm);
-  ok = ok && ar.ask(&ws.ynorm, Bm) && ar.ask(&ws.rnorm, Bm) && ar.ask(&ws.niter, Bm) &&
-       ar.ask(&ws.stop, Bm) && ar.ask(&ws.err, 1) && ar.ask(&h->args_dev, 1);
-  ok = ok && ar.ask(&h->y_stage, Bm * static_cast<size_t>(ws.M)) &&
-       ar.ask(&h->x_stage, Bm * Sm) && ar.ask(&h->s_stage, Bm * Sm) &&
-       ar.ask(&h->margin_buf, Bm * Sm);
-  if (d.precision == OMP_PREC_FP32) ok = ok && ar.ask(&h->cand2_buf, Bm);
-  ok = ok && ar.allocate(h);
+  // Every workspace, or (lean) all but those that only make solves faster: the FP32 path's filter, the
+  // longer candidate lists and the rows of a gather in a launch of its own.
+  auto ask_all = [&](Arena& ar, bool lean) {
+    // The FP32 path filters its atoms with a BF16 correlation, if a batch of this handle can gain by it.
+    // (The test hook that turns the score bound off turns this off too.)
+    ws.filt = d.precision == OMP_PREC_FP32 && !hook && !lean && filter_pays(ws, ws.Bmax) ? 1 : 0;
+    ws.tcprec = ws.filt ? OMP_PREC_BF16 : ws.prec;
+    const bool tc = ws.tcprec != OMP_PREC_FP32;
+    if (tc) tc_fill_sched(ws, h->sm_count, lean ? kLeanPieces : kPieces);
+    const size_t qbytes = ws.tcprec == OMP_PREC_BF16 ? 2 : 1;
+    bool ok = true;
+    ok = ok && ar.ask(&ws.A32, N * Mp);
+    if (d.gather24) ok = ok && ar.ask(&ws.A24h, N * Mp) && ar.ask(&ws.A24l, N * Mp);
+    if (ws.tcprec == OMP_PREC_BF16) ok = ok && ar.ask(&ws.A16, N * Mp);
+    if (d.precision == OMP_PREC_FP8_E4M3) ok = ok && ar.ask(&ws.A8, N * Mp) && ar.ask(&ws.sa, N);
+    if (tc) ok = ok && ar.ask(&ws.escale, Npad);
+    ok = ok && ar.ask(&ws.inv_norm, N) && ar.ask(&ws.norm2, N) && ar.ask(&ws.gram, N * ws.ldg);
+    ok = ok && ar.ask(&ws.R32, Bm * Mp);
+    if (tc) {
+      ok = ok && ar.ask(reinterpret_cast<uint8_t**>(&ws.Rq[0]), Bp * Mp * qbytes) &&
+           ar.ask(reinterpret_cast<uint8_t**>(&ws.Rq[1]), Bp * Mp * qbytes);
+      ok = ok && ar.ask(&ws.sr[0], Bp) && ar.ask(&ws.sr[1], Bp);
+      ok = ok && ar.ask(&ws.cand_s, Bp * ws.pieces * kMaxTopk) &&
+           ar.ask(&ws.cand_i, Bp * ws.pieces * kMaxTopk);
+    }
+    // The pruning thresholds (and the data-driven bound they carry): on BF16 always; on E4M3,
+    // whose worst-case bound is too loose to prune, only where the one-warp update quantises the
+    // next row itself and so can measure its rounding error (padded lengths up to 1024).
+    const bool want_tau = ws.prec == OMP_PREC_BF16 ||
+                          (ws.prec == OMP_PREC_FP8_E4M3 && update_default_warps(ws.Mp) == 1);
+    if (want_tau && ws.rescore_eps > 0.f && ws.Smax <= kTauSmax)
+      ok = ok && ar.ask(&ws.tau, Bm) && ar.ask(&ws.tau_pos, Bp) && ar.ask(&ws.win_pos, Bp) &&
+           (ws.prec != OMP_PREC_FP8_E4M3 || ar.ask(&ws.ea, 1));
+    if (ws.filt)
+      ok = ok && ar.ask(&ws.win_pos, Bp) && ar.ask(&ws.ea, 1) && ar.ask(&ws.ovf, Bm) &&
+           ar.ask(&ws.ovf_cnt, Sm + 1);
+    ok = ok && ar.ask(&ws.live[0], Bm) && ar.ask(&ws.live[1], Bm);
+    ok = ok && ar.ask(&ws.livek[0], Bm) && ar.ask(&ws.livek[1], Bm);
+    ok = ok && ar.ask(&ws.cnt, Sm + 2) && ar.ask(&ws.kdev, 1) && ar.ask(&ws.flag, Bm) && ar.ask(&ws.cand1, Bm);
+    ok = ok && ar.ask(&ws.upd_ctr, Sm + 1);
+    if (!lean && gather_apart_shape(ws.N, ws.Mp, ws.Bmax)) ok = ok && ar.ask(&ws.sel, Bm) && ar.ask(&ws.Q, Bm * Mp);
+    ok = ok && ar.ask(&ws.score, small_score_floats(ws.N, ws.Bmax));
+    ok = ok && ar.ask(&ws.F, Bm * static_cast<size_t>(ws.Fstride)) &&
+         ar.ask(&ws.F32, Bm * static_cast<size_t>(ws.Fstride)) && ar.ask(&ws.bv, Bm * Sm) &&
+         ar.ask(&ws.sup, Bm * Sm);
+    ok = ok && ar.ask(&ws.drop, Bm * Sm) && ar.ask(&ws.fb, Bm);
+    ok = ok && ar.ask(&ws.ynorm, Bm) && ar.ask(&ws.rnorm, Bm) && ar.ask(&ws.niter, Bm) &&
+         ar.ask(&ws.stop, Bm) && ar.ask(&ws.err, 1) && ar.ask(&h->args_dev, 1);
+    ok = ok && ar.ask(&h->y_stage, Bm * static_cast<size_t>(ws.M)) &&
+         ar.ask(&h->x_stage, Bm * Sm) && ar.ask(&h->s_stage, Bm * Sm) &&
+         ar.ask(&h->margin_buf, Bm * Sm);
+    if (d.precision == OMP_PREC_FP32) ok = ok && ar.ask(&h->cand2_buf, Bm);
+    return ok;
+  };
+  Arena full, lean;
+  const bool ok = ask_all(full, false) && (full.allocate(h) || (ask_all(lean, true) && lean.allocate(h)));
   if (!ok) {
     release(h);
     delete h;
     return OMP_ERR_OUT_OF_MEMORY;
   }
+  const bool tc = ws.tcprec != OMP_PREC_FP32;
   bool cuda_ok = cudaMemset(ws.err, 0, sizeof(unsigned)) == cudaSuccess &&
                  (!ws.escale || cudaMemset(ws.escale, 0, Npad * sizeof(float)) == cudaSuccess) &&
                  cudaMemset(ws.cand1, 0, Bm * sizeof(unsigned long long)) == cudaSuccess &&
