@@ -214,13 +214,16 @@ omp_status omp_solve_batch_trace(omp_handle h, const float* A, const float* Y, i
  * names a file, a choice recorded there for the same GPU, M, N, precision, B and S is used
  * without timing ("key|warps,stages,ctas,persistent,cluster" lines; shorter lines keep the other
  * shapes), and new choices are appended to it. Synchronises `stream`. Captured graphs are
- * dropped when the choice changes. */
+ * dropped when the choice changes. A (B, S) whose solves take a form for few signals launches none
+ * of these kernels: the handle keeps its shapes, nothing is timed or recorded. The BF16
+ * correlation that filters the FP32 path's atoms keeps its default shapes. */
 omp_status omp_autotune(omp_handle h, const float* A, const float* Y, int64_t B, int32_t S, float eps,
                         int32_t repeats, int32_t* choice_out, void* stream);
 
 /* The handle's current launch shapes (each pointer may be NULL): update warps per signal, update
  * persistent form (0 or 1), correlation operand stages, persistent CTAs and CTAs per cluster (1,
- * or 2 for the 2-SM MMA pair; the last three 0 on the FP32 path). Host only. */
+ * or 2 for the 2-SM MMA pair; the last three 0 on the FP32 path, whose filter is not tuned). Host
+ * only. */
 omp_status omp_tuning(omp_handle h, int32_t* update_warps, int32_t* update_persistent,
                       int32_t* corr_stages, int32_t* corr_ctas, int32_t* corr_cluster);
 
