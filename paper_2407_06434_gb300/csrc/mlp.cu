@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;
   const float* y = Y + static_cast<size_t>(b) * M;
-  float hi = 0.f, lo = 0.f;
+  SquareSum sq;
   bool finite = true;
   for (int m0 = 0; m0 < Mp; m0 += 32 * R) {
     float v[R];
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       finite = finite && isfinite(v[i]);
-      square_in(hi, lo, v[i]);
+      square_in(sq, v[i]);
     }
     // written as if finite; a signal with a NaN or Inf is cleared below
     __nv_bfloat16* q = Yq + static_cast<size_t>(b) * Mp;
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
       if (m < Mp) q[m] = __float2bfloat16_rn(v[i]);
     }
   }
-  double s = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
+  double s = warp_sum(total(sq));
   if (!squares_ok(s)) {  // zero, tiny or huge signals (or a NaN)
     s = 0.0;
     for (int m = lane; m < M; m += 32) s += static_cast<double>(y[m]) * y[m];

@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(256) init_kernel(Ws ws, const CallArgs* args, 
   const float* y = args->Y + static_cast<size_t>(b) * ws.M;
   float* r = ws.R32 + static_cast<size_t>(b) * ws.Mp;
   constexpr int R = 16;  // loads in flight per lane
-  float hi = 0.f, lo = 0.f;
+  SquareSum sq;
   bool finite = true;
   for (int m0 = lane; m0 < ws.Mp; m0 += 32 * R) {
     float v[R];
@@ -50,10 +50,10 @@ __global__ void __launch_bounds__(256) init_kernel(Ws ws, const CallArgs* args, 
     for (int i = 0; i < R; ++i) {
       finite = finite && isfinite(v[i]);
       if (m0 + 32 * i < ws.Mp) r[m0 + 32 * i] = v[i];
-      square_in(hi, lo, v[i]);
+      square_in(sq, v[i]);
     }
   }
-  double s = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
+  double s = warp_sum(total(sq));
   if (!squares_ok(s)) {  // zero, tiny or huge signals (or a NaN)
     s = 0.0;
     for (int m = lane; m < ws.M; m += 32) s += static_cast<double>(y[m]) * static_cast<double>(y[m]);

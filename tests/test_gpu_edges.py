@@ -1,4 +1,6 @@
 """Values and sizes at the edges of what the kernels' shortcuts assume."""
+import math
+
 import numpy as np
 import pytest
 
@@ -281,3 +283,34 @@ def test_autotune_of_few_signals(lib, monkeypatch, tmp_path, prec):
             assert lib.omp_tuning(s.h) == before and not cache.exists()
         s.close()
     assert len(cache.read_text().splitlines()) == 1
+
+
+def _near_midpoint(M, d, seed):
+    """A signal whose norm lies d (relative, squared) from the midpoint of two neighbouring floats, and
+    its norm rounded to the nearest."""
+    rng = np.random.default_rng(seed)
+    y = (rng.standard_normal(M) * np.exp(4 * rng.standard_normal(M))).astype(np.float32)
+    y[-3:] = 0.0
+    s = math.fsum(float(v) ** 2 for v in y)      # (the square of a float is a double)
+    lo = np.float32(math.sqrt(s * 1.0001))
+    hi = np.nextafter(lo, np.float32(np.inf))
+    mid2 = ((float(lo) + float(hi)) / 2) ** 2
+    for i, part in ((-3, 0.999), (-2, 0.999), (-1, 1.0)):
+        rest = math.fsum([mid2, mid2 * d] + [-float(v) ** 2 for v in y])
+        y[i] = np.float32(math.sqrt(max(rest, 0.0) * part))
+    off = math.fsum([-mid2] + [float(v) ** 2 for v in y]) / mid2
+    assert 0.5 * abs(d) < off * np.sign(d) < 2 * abs(d)
+    return y, hi if d > 0 else lo
+
+
+def test_signal_norms_keep_the_bits_of_fp64(lib):
+    """||y|| is the float nearest to the norm as FP64 sums form it: to 2^-47 of the sum of squares, four
+    times the rounding that 256 FP64 additions a lane and five across the warp showed (2^-48.8)."""
+    M = 8192
+    rows = [_near_midpoint(M, sign * 2.0 ** -46, seed) for seed in range(40) for sign in (1, -1)]
+    Y = torch.from_numpy(np.stack([y for y, _ in rows])).cuda()
+    s = lib.OmpSolver(M, 2, max_batch=len(rows), max_iters=1, precision="fp32")
+    out = s.solve(torch.zeros(2, M, device="cuda").t(), Y, 1, diagnostics=True)
+    s.close()
+    assert not out[2].any()                      # no atom to pick: the residual is the signal
+    assert np.array_equal(out[3].cpu().numpy(), np.array([n for _, n in rows]))
