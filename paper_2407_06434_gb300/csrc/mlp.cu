@@ -41,12 +41,21 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
   return cdf + x * pdf;
 }
 
-// log(1 + e^-|o|) from E = e^-o (any o; E = inf gives 0): with e = e^-|o| it is 2 atanh(s),
-// s = e / (2 + e) <= 1/3, by the odd series of atanh (seven terms leave 1.5e-8 relative), so the
-// sigmoid's exponential serves the loss too and no logarithm is taken
+// log(1 + e^-|o|) from E = e^-o, so that the sigmoid's exponential serves the loss too and no logarithm is
+// taken: 2 atanh(s), s = e / (2 + e) <= 1/3 with e = e^-|o|, by the odd series of atanh (seven terms leave
+// 1.5e-8 relative). What the denominator, its reciprocal and the quotient round off comes back in by ds:
+// against 64 bits the largest error and the root mean square are then no more than those of
+// log1pf(expf(-|o|)) (o from -16 to 0: 1.82e-7 for 1.94e-7, 4.64e-8 for 4.66e-8; from -6 to 30: 1.93e-7 both,
+// 4.42e-8 for 4.43e-8), without it 2.6e-7. A step at batch 4096, 8192 -> 1024 -> 8192: 633 us; without the
+// correction 618, with expf and log1pf 677.
 __device__ __forceinline__ float log1p_exp_neg_abs(float E) {
   const bool big = E >= 1.f;  // o <= 0: e = 1 / E
-  const float s = __fdividef(big ? 1.f : E, big ? fmaf(2.f, E, 1.f) : 2.f + E);
+  const float w = fminf(E, 0x1p124f);
+  const float a = big ? 1.f : w, two = big ? 2.f * w : 2.f, x = big ? 1.f : w;
+  const float b = two + x, be = x - (b - two);
+  const float rb = __fdividef(1.f, b);
+  const float s = a * rb;
+  const float ds = fmaf(-s, be, fmaf(-s, b, a)) * rb;
   const float q = s * s;
   float p = 1.f / 13.f;
   p = fmaf(p, q, 1.f / 11.f);
@@ -54,7 +63,7 @@ __device__ __forceinline__ float log1p_exp_neg_abs(float E) {
   p = fmaf(p, q, 1.f / 7.f);
   p = fmaf(p, q, 1.f / 5.f);
   p = fmaf(p, q, 1.f / 3.f);
-  return 2.f * fmaf(p * q, s, s);
+  return 2.f * (s + fmaf(s, p * q, fmaf(ds, q, ds)));
 }
 
 // two BF16 values of a word (the lower index in the low half) as FP32

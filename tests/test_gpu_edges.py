@@ -314,3 +314,35 @@ def test_signal_norms_keep_the_bits_of_fp64(lib):
     s.close()
     assert not out[2].any()                      # no atom to pick: the residual is the signal
     assert np.array_equal(out[3].cpu().numpy(), np.array([n for _, n in rows]))
+
+
+def test_training_loss_has_the_bits_of_log1p(lib):
+    """One logit at a time, all others at -40 with label 0: the loss is log(1 + e^-|o|) of that logit to
+    the error of FP32's own log1p and exp (those of torch on the same values)."""
+    n = 64
+    At = torch.eye(n, device="cuda")
+    Y = torch.zeros(n, n, device="cuda")
+    Y[0, 0] = 1.0
+    Y[1:, 1] = 1.0
+    s = lib.OmpSolver(n, n, max_batch=n, max_iters=1, precision="bf16")
+    p = lib.Proposal(s.h, hidden=n, topk=8, train_batch=n)
+    zero = [torch.zeros(k, device="cuda") for k in ((n, n), n, (n, n))]
+    got, o = [], []
+    loss = torch.zeros(1, device="cuda")
+    for i, beta in enumerate(40.0 + np.random.default_rng(3).uniform(-12, 12, 1500).astype(np.float32)):
+        b2 = torch.full((n,), -40.0, device="cuda")
+        b2[1] = -200.0                           # the other rows' one feature
+        logit = np.float32(beta) - np.float32(40.0)
+        labels = torch.full((n, 1), -1, dtype=torch.int32, device="cuda")
+        labels[0, 0] = 0 if logit > 0 else -1    # the label that leaves the logarithm alone
+        p.set_weights(zero[0], zero[1], zero[2], b2, torch.full((1,), float(beta), device="cuda"))
+        p.gradients(At.t(), Y, labels, loss_out=loss)
+        got.append(float(loss) * n * n)          # (a power of two)
+        o.append(float(logit))
+    p.close()
+    s.close()
+    o = torch.tensor(o, device="cuda")
+    exact = torch.log1p(torch.exp(-o.double().abs()))
+    err = ((torch.tensor(got, device="cuda", dtype=torch.float64) - exact).abs() / exact).max()
+    own = ((torch.log1p(torch.exp(-o.abs())).double() - exact).abs() / exact).max()
+    assert err <= own * (1 + 1e-9), (float(err), float(own))
