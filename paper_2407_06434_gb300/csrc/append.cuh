@@ -901,7 +901,7 @@ void launch_g(const Ws& ws, int k, int B, int S, float eps, int eps_rel, cudaStr
 
 template <int W, int V>
 void launch_t(const Ws& ws, int k, int B, int S, float eps, int eps_rel, cudaStream_t s) {
-  if (gather_apart(ws, B)) {
+  if (gather_apart(ws, B, k, S)) {
     const size_t smem = group_bytes(ws);
     step_part_kernel<W, V, kHead><<<B, W * 32, smem, s>>>(ws, k, S, eps, eps_rel);
     launch_gather(ws, k, B, s);

@@ -398,9 +398,10 @@ void launch_finalize(const Ws& ws, const CallArgs* args, int B, int S, cudaStrea
 void launch_topk_out(const Ws& ws, const CallArgs* args, int B, int topk, cudaStream_t s);
 void launch_set_args(CallArgs* dst, const CallArgs& v, cudaStream_t s);
 cudaError_t configure_update_kernels(const Ws& ws);
-// q gathered by a launch of its own (gather.cu): for the handle's shape, and for a batch of it
+// q gathered by a launch of its own (gather.cu): for the handle's shape, and for step k of a solve of
+// S steps (k -1: one form for all steps)
 bool gather_apart_shape(int64_t N, int64_t Mp, int64_t Bmax);
-bool gather_apart(const Ws& ws, int B);
+bool gather_apart(const Ws& ws, int B, int k, int S);
 void launch_gather(const Ws& ws, int k, int B, cudaStream_t s);
 int update_slots(int Mp, int W);
 int update_default_warps(int Mp);

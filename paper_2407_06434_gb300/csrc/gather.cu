@@ -113,7 +113,28 @@ int pieces_of(const Ws& ws) {
 bool gather_apart_shape(int64_t N, int64_t Mp, int64_t Bmax) {
   return static_cast<size_t>(N) * Mp * 4 > kWholeBytes && Bmax >= kApartMinB;
 }
-bool gather_apart(const Ws& ws, int B) { return ws.Q != nullptr && B >= kApartMinB; }
+// Two launches more and q's way through memory cost about as much at every step, while the rows that
+// are read from L2 and not from HBM grow with the step. So the first steps are one kernel; from which
+// step on three are faster depends on the row length (warps a signal), the batch and on what the head
+// carries besides (BF16: two candidate rows in shared memory for the threshold). Measured, us a step on
+// average over solves of 12, 48 and 100 steps, one kernel / three: 1024 x 60000, FP8, 4096 signals 235 /
+// 243, 290 / 284, 390 / 353, 1024 signals 84 / 93, 100 / 108, 146 / 149; 2048 x 24576, 4096 signals, FP8
+// 239 / 242, 329 / 296, 448 / 366, BF16 329 / 348, 394 / 391, 510 / 455, FP32 (48) 417 / 401; 2048 x 24576,
+// 1024 signals, FP8 90 / 98, 106 / 115, 137 / 139; 4096 x 16384, 4096 signals, FP8 334 / 341, 517 / 438, 751 /
+// 557, BF16 464 / 492, 592 / 569, 821 / 667, FP32 (48) 645 / 593; 1024 signals, FP8 114 / 115, 160 / 144,
+// 222 / 178, BF16 147 / 157, 180 / 184, 245 / 215.
+bool gather_apart(const Ws& ws, int B, int k, int S) {
+  if (!ws.Q || B < kApartMinB) return false;
+  const bool many = B >= 2048, bf16 = ws.prec == OMP_PREC_BF16, fp8 = ws.prec == OMP_PREC_FP8_E4M3;
+  int from;
+  if (ws.Mp <= 1024)
+    from = many ? 24 : 64;
+  else if (ws.Mp <= 2048)
+    from = bf16 ? (many ? 24 : 40) : fp8 ? (many ? 7 : 48) : (many ? 18 : 28);
+  else
+    from = bf16 ? (many ? 19 : 28) : fp8 ? 4 : 12;
+  return (k >= 0 ? k : S / 2) >= from;
+}
 
 void launch_gather(const Ws& ws, int k, int B, cudaStream_t s) {
   const int M4 = ws.Mp / 4;

@@ -346,3 +346,44 @@ def test_training_loss_has_the_bits_of_log1p(lib):
     err = ((torch.tensor(got, device="cuda", dtype=torch.float64) - exact).abs() / exact).max()
     own = ((torch.log1p(torch.exp(-o.abs())).double() - exact).abs() / exact).max()
     assert err <= own * (1 + 1e-9), (float(err), float(own))
+
+
+# The gather in a launch of its own from some step of a solve on (later for short rows, few signals and
+# BF16), or for all steps of the device-side loop: the same words as the one-kernel steps that smaller
+# batches take throughout.
+@pytest.mark.parametrize("prec,M,N,B,S,kw", [
+    ("fp8", 4000, 11000, 1100, 14, {}), ("fp8", 4000, 11000, 1100, 18, {"use_graph": 2}), ("bf16", 8192, 5200, 1100, 32, {}),
+    ("fp32", 2050, 20500, 1100, 16, {}), ("bf16", 2048, 21000, 2100, 28, {"gather24": True}),
+    ("fp8", 1000, 41000, 2100, 27, {}), ("fp32", 2048, 21000, 2100, 40, {"use_graph": 2})])
+def test_gather_apart_from_a_step_on(lib, prec, M, N, B, S, kw):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N)
+    At = torch.randn((N, M), generator=g, device="cuda")
+    At /= At.norm(dim=1, keepdim=True)
+    sup = torch.randint(0, N, (B, S), generator=g, device="cuda")
+    coef = torch.randn((B, S), generator=g, device="cuda")
+    coef[::3, S // 2:] = 0.0                     # these reach the threshold half way
+    Y = 1e-4 * torch.randn((B, M), generator=g, device="cuda")
+    for j in range(S):
+        Y += coef[:, j, None] * At[sup[:, j]]
+    Y[5] = 0.0
+    out = []
+    s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision=prec, **kw)
+    for n in (B, 550):
+        parts = [s.solve(At.t(), Y[lo:lo + n].clone(), S, 0.01, diagnostics=True) for lo in range(0, B, n)]
+        out.append([torch.cat(p).cpu().numpy().view(np.uint32) for p in zip(*parts)])
+    s.close()
+    for got, want in zip(*out):
+        assert np.array_equal(got, want)
+
+
+def test_gather_apart_not_in_short_solves(lib):
+    """1024 signals take a gather of its own where it pays; a short solve of them takes no longer than
+    one of 1000, which never do (both fill eight row tiles): 2.4 % more signals, and as much again."""
+    At, Y, _ = _planted(2048, 24576, 1024, 6, 1)
+    ms = []
+    for B in (1024, 1000):
+        s = lib.OmpSolver(2048, 24576, max_batch=1024, max_iters=12, precision="bf16")
+        ms.append(_solve_ms(s, At, Y[:B].contiguous(), 12))
+        s.close()
+    assert ms[0] < 1.05 * ms[1], ms
