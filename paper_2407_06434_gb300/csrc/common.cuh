@@ -246,9 +246,12 @@ __device__ __forceinline__ int iter_of(const Ws& ws, int k) { return k >= 0 ? k 
 
 // FP32 path: whether step k goes without the filter, as after a step that left more than three quarters
 // of its positions undecided (near copies, long rows at the noise floor); every fourth step tries again.
+// Of less than a row tile of positions, whose FP32 scores cost as much whatever their number, a few
+// undecided ones say little about the next step (one signal, 1024 x 8192: 40 us a step, 47 with rests).
 __device__ __forceinline__ bool filter_rests(const Ws& ws, int k) {
   if ((k & 3) == 0) return false;
-  return 4ll * __ldg(ws.ovf_cnt + k - 1) > 3ll * __ldg(ws.cnt + k);
+  const int live = __ldg(ws.cnt + k);
+  return 4ll * __ldg(ws.ovf_cnt + k - 1) > 3ll * live && live >= kSigTile;
 }
 
 // Persistent schedule of the tensor-core correlation (shared by the correlation kernel, which
