@@ -387,3 +387,24 @@ def test_gather_apart_not_in_short_solves(lib):
         ms.append(_solve_ms(s, At, Y[:B].contiguous(), 12))
         s.close()
     assert ms[0] < 1.05 * ms[1], ms
+
+
+def test_candidates_without_the_filter(lib):
+    """A small FP32 solve restricted to candidates runs its dense loop in three launches a step."""
+    from torch.profiler import ProfilerActivity, profile
+    M, N, B, S = 256, 1024, 20, 8
+    At, Y, sup = _planted(M, N, B, S, 11)
+    s = lib.OmpSolver(M, N, max_batch=B, max_iters=S, precision="fp32")
+    X = torch.empty((B, S), device="cuda")
+    so = torch.empty((B, S), dtype=torch.int32, device="cuda")
+    cand = torch.from_numpy(np.ascontiguousarray(sup[:, :S // 2]).astype(np.int32)).cuda()
+    tau = torch.full((S,), 1e-6, device="cuda")
+    n = 0
+    for _ in range(2):                           # (the profiler may miss the first)
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            lib.omp_solve_batch_candidates(s.h, At.t(), Y, S, 0.0, cand, tau, X, so)
+            torch.cuda.synchronize()
+        n = max(n, sum(1 for e in p.events() if e.device_type == torch.autograd.DeviceType.CUDA
+                       and "kernel" in e.name))
+    s.close()
+    assert n <= 3 * S + 5, n
