@@ -419,7 +419,7 @@ void launch_update_w4(const Ws& ws, int V, int k, int B, int S, float eps, int e
 void launch_update_w8(const Ws& ws, int V, int k, int B, int S, float eps, int eps_rel, cudaStream_t s);
 
 // solves of few signals (small.cu): the form a solve takes (0: batched), and its launches
-int small_form(const Ws& ws, int B);
+int small_form(const Ws& ws, int B, float eps);
 size_t small_score_floats(int N, int Bmax);
 cudaError_t configure_small(const Ws& ws);
 void launch_solo(const Ws& ws, int B, int S, float eps, int eps_rel, cudaStream_t s);

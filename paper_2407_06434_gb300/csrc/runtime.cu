@@ -191,7 +191,7 @@ void prof_mark(omp_handle_s* h, bool prof, int kind, int k, int end, cudaStream_
 
 // A solve of few signals (small.cu), where the sizes and options take one of those forms.
 bool enqueue_small(omp_handle_s* h, const Ws& ws, int B, int S, float eps, cudaStream_t s) {
-  const int form = small_form(ws, B);
+  const int form = small_form(ws, B, eps);
   if (form == 0) return false;
   launch_init(ws, h->args_dev, B, s);
   if (form == 1)
@@ -778,7 +778,7 @@ omp_status omp_autotune(omp_handle h, const float* A, const float* Y, int64_t B,
     }
   }
   // a solve that takes a few-signals form launches none of the kernels tuned here
-  if (!best.w && h->d.use_graph != 2 && small_form(solve_ws(h, static_cast<int>(B), false), static_cast<int>(B)) != 0)
+  if (!best.w && h->d.use_graph != 2 && small_form(solve_ws(h, static_cast<int>(B), false), static_cast<int>(B), eps) != 0)
     best.w = saved.w;
   if (!best.w) {
     omp_status st = OMP_OK;

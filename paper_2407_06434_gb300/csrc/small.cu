@@ -636,7 +636,7 @@ void by_slots(int V, F f) {
 // Which arrangement a solve takes: 0 batched, 1 solo, 2 wide. The quantised 8-bit path, fewer than
 // 8 rescored candidates, recorded margins, the 24-bit gather and the hook that turns the score
 // bound off stay batched: their picks depend on what the batched path keeps of its lists.
-int small_form(const Ws& ws, int B) {
+int small_form(const Ws& ws, int B, float eps) {
   if (ws.prec == OMP_PREC_FP8_E4M3 || ws.A24h || ws.margin) return 0;
   if (ws.prec == OMP_PREC_BF16 && (ws.topk != kMaxTopk || !(ws.rescore_eps > 0.f))) return 0;
   const bool fp32 = ws.prec == OMP_PREC_FP32;
@@ -654,7 +654,10 @@ int small_form(const Ws& ws, int B) {
     const int left = (M4 % 128 + 31) / 32;
     const double atom = ws.Mp == 64 ? 9.5e-3 : 1e-3 * (20 + M4 / 128 * (B <= ws.sms ? 15 : 20) + 8 * left);
     const double batched = !fp32 ? 19.0 + ws.Mp / 170.0 : ws.Mp == 64 ? 19.5 : 22.0 + ws.Mp / 100.0;
-    if (rounds * (4.0 + ws.N * atom) <= batched) return 1;
+    // (With a threshold a block ends with its signal, where every other form launches what is left of
+    // the S steps: one signal over 256 x 512, BF16, 128 steps of which it takes some 16, 318 us a solve
+    // for 412 by the wide form and 721 batched.)
+    if (rounds * (4.0 + ws.N * atom) <= (eps > 0.f ? 1.3 : 1.0) * batched) return 1;
   }
   // Wide scores every atom for each signal on the CUDA cores and keeps the residuals in shared memory.
   // Measured, us a step wide / batched FP32 / batched BF16: 1024 x 8192 1 signal 13.6 / 32 / 28, 8 24.4 /

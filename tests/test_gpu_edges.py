@@ -408,3 +408,26 @@ def test_candidates_without_the_filter(lib):
                        and "kernel" in e.name))
     s.close()
     assert n <= 3 * S + 5, n
+
+
+def test_one_block_a_signal_ends_with_it(lib):
+    """A signal that reaches its threshold after a few of many steps takes a fraction of the time of all
+    the steps: its block ends, where the other forms still launch every step."""
+    At, Y, _ = _planted(256, 512, 1, 4, 5)
+    s = lib.OmpSolver(256, 512, max_batch=1, max_iters=128, precision="bf16")
+    ms = []
+    for eps in (0.05, 1e-30):
+        for _ in range(3):
+            s.solve(At.t(), Y, 128, eps)
+        ts = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            n = s.solve(At.t(), Y, 128, eps, diagnostics=True)[2]
+            b.record()
+            torch.cuda.synchronize()
+            ts.append(a.elapsed_time(b))
+        ms.append((min(ts), int(n)))
+    s.close()
+    (t0, n0), (t1, n1) = ms
+    assert n0 <= 8 and n1 > 64 and t0 < 0.2 * t1, ms
