@@ -41,7 +41,7 @@ METRIC = "OMP signals/s, chosen form vs plain FP32 on same GB300 at matched supp
 L2_RESIDENT_BYTES = 64 << 20   # an FP32 dictionary up to half the 129 MB L2 stays resident
 MEASURED_TRAFFIC = {
     ("gaussian_1024x8192_s32_b4096", "bf16", "correlate"): 25272832.0,
-    ("gaussian_1024x8192_s32_b4096", "bf16", "update"): 72470272.0,
+    ("gaussian_1024x8192_s32_b4096", "bf16", "update"): 72896256.0,
 }
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 # FP32 non-tensor peak: 152 SMs x 128 FP32 lanes x 2 FLOP x 2.07 GHz (nominal unit counts)
@@ -262,6 +262,7 @@ def run_gpu(args):
             upd += u
             live = lv
             n_prof = i + 1
+        prof_launches = count_launches(h, X, sup)
         omp.omp_profile_enable(h, False)
         corr /= n_prof
         upd /= n_prof
@@ -282,7 +283,7 @@ def run_gpu(args):
         torch.cuda.synchronize()
         res = dict(total_ms=total, ms=ms, corr=corr, upd=upd, live=live, update_warps=tuned, shapes=shapes,
                    e2e_s=float(np.sum(e2e_t)), e2e_steps=len(e2e_t), launches=count_launches(h, X, sup),
-                   sup=Sd.cpu().numpy(), X=Xd.cpu().numpy(), n_iter=nd.cpu().numpy(),
+                   prof_launches=prof_launches, sup=Sd.cpu().numpy(), X=Xd.cpu().numpy(), n_iter=nd.cpu().numpy(),
                    resid=rd.cpu().numpy())
         solver.close()
         return res
@@ -316,10 +317,10 @@ def run_gpu(args):
     if corr_ms.sum() >= upd_ms.sum():
         dur = corr_ms.mean() / 1e3
         achieved = float(flops_corr.mean() / dur / 1e12)
-        mp64 = (w.M + 63) // 64 * 64
-        # the FP32 form scores every atom in FP32 on short rows of small problems only; elsewhere a
-        # BF16 tensor-core pass bounds every score and FP32 scores the atoms that the bound leaves
-        if args.precision == "fp32" and mp64 < 256 and float(w.N) * mp64 * w.B < 3e8:
+        # the FP32 form scores every atom in FP32 in a step of three launches; where it filters them, a
+        # BF16 tensor-core pass bounds every score, FP32 scores the atoms that the bound leaves, and a
+        # step has five
+        if args.precision == "fp32" and chosen["prof_launches"] < 5 * w.S:
             peak, unit, bound, src = FP32_SIMT_PEAK_TFLOPS, "TFLOP/s", "alu", "nominal"
         else:
             # each correlation launch is timed on its own (tens of microseconds inside a solve of

@@ -155,7 +155,10 @@ omp_status omp_correlate_topk(omp_handle h, const float* A, const float* R, int6
 
 /* Per-launch timing. When enabled, the next solves record CUDA events around every correlation
  * and update launch (a separate captured graph with event-record nodes; results are the same
- * as without it). omp_profile_read synchronises `stream` and returns, for the most recent
+ * as without it). It always runs the batched kernels: a solve of few signals, which otherwise
+ * takes a form without such launches, is measured as the batch it would be (BF16: its picks may
+ * then differ where more than eight atoms lie within the score error bound of the best).
+ * omp_profile_read synchronises `stream` and returns, for the most recent
  * solve, each iteration's correlation and update launch duration in milliseconds
  * (corr_ms, update_ms: S floats each, device-independent host arrays) and the live signal count
  * at the start of each iteration (live_out: S int32, may be NULL). S must equal that solve's S.

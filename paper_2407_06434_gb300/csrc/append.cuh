@@ -827,7 +827,8 @@ __device__ __forceinline__ void update_position(const Ws& ws, int k, int L, int 
 // takes another. The two are separate kernels, so each holds one copy of the step's code.
 // Resident warps asked of the compiler per SM, by the float4 slots V a lane holds: 16 warps
 // (128 registers) for 8 slots, 24 (80 registers) for 4, 32 (64 registers) for 2 or 1; the
-// one-warp form keeps 16 for 4 slots and 24 for fewer, where those limits spill nothing.
+// one-warp form keeps 16 for 4 slots and 24 for fewer. (Spills: none in the one-warp form at 1 and 4 slots,
+// 12 to 60 bytes in its persistent and 24-bit ones, up to 32 bytes at more warps, 88 in persistent ones.)
 constexpr int update_min_warps(int W, int V) {
   return V >= 8 ? 16 : W == 1 ? (V == 4 ? 16 : 24) : V == 4 ? 24 : 32;
 }

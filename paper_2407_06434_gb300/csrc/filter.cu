@@ -10,7 +10,7 @@
 // correlation returns at once and the list holds every position (filter_rests).
 //
 // The full FP32 correlation of 1000 signals with 8192 atoms of length 1024 takes 309 us a step, the
-// BF16 one 20, this kernel 9.7 and the (mostly empty) overflow launch 3.5. This kernel is bound by the
+// BF16 one 20, this kernel 9.7 and the overflow launch 3.4 on average (1.7 where empty). This kernel is bound by the
 // latency of a position's round trips and of its chain (four cycles an element at best); with chunks of
 // 256 elements it takes 9.4 there, but 122 registers a thread instead of 80 cost a large batch residency.
 #include "common.cuh"

@@ -6,8 +6,8 @@
 // the row length is cut into pieces and the blocks of all signals' first pieces come before any second,
 // so that a piece of the dictionary stays in L2 while the whole batch reads it: HBM then reads the
 // dictionary about once a step. 4096 signals, 4096 x 32768, FP8, 64 steps (us a step on average): one
-// kernel 463; head 128, gather 149, tail 35. (A head of one warp per signal took 190: its rescoring reads up
-// to eight rows of 16 KB one warp at a time.)
+// kernel 463; head 127, gather 157, tail 35 (60 steps; the first four, in one kernel, 234). (A head of one
+// warp per signal took 190: its rescoring reads up to eight rows of 16 KB one warp at a time.)
 //
 // q's rows are summed in the same order as in the one kernel: the same bits.
 #include "append.cuh"

@@ -81,8 +81,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // pieces, a transposed store puts a warp's 32 consecutive rows side by side. Scalar row-major
 // accesses (32 sectors per instruction) bounded these kernels by their epilogue: at batch 4096,
 // 8192 -> 1024 -> 8192 (MMAs of about 40 us each) the features and the hidden layer in training took
-// 157 us on average and take 67 us now, the loss kernel 856 us and now 192 us, the GELU backward
-// 102 us and now 72 us.
+// 157 us on average and take 64 us now, the loss kernel 856 us and now 149 us, the GELU backward
+// 102 us and now 60 us.
 
 // The warp's EPI_COLS columns of a vector over the columns (bias or scale) of column tile t, staged in
 // its shared scratch at each unit (16 bytes a lane): the chunks read them there.
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 // ------------------------------------------------------------------------ small kernels
 // Feature input: y in BF16 (zero padded to Mp) and 1/||y|| (0 for y == 0 or non-finite y). One warp
-// per signal, the row read once: up to 16 values a lane stay in registers for the second step 
+// per signal, the row read once, 16 loads in flight a lane.
 __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict__ Y, int M, int Mp, int B,
                                                         __nv_bfloat16* Yq, float* inv_ynorm) {
   constexpr int R = 16;

@@ -14,7 +14,9 @@
 // Scores here are FP32 dot products in an order of their own. An atom can only be the pick if its
 // score is within two error bounds of the best, so those atoms -- mostly one -- are scored again
 // as the batched path of the handle does it (FP32: one chain of FMAs over m; BF16: the rescoring's
-// order), and b and ||r|| are summed in the batched update's order: the same picks and bits.
+// order), and b and ||r|| are summed in the batched update's order: the same picks and bits as the
+// batched kernels, but for BF16 signals with more than eight atoms in the window (near copies). The
+// batched path rescores the eight best by BF16 score; here all of them are, so the pick is FP32's.
 #include <type_traits>
 
 #include "append.cuh"
