@@ -358,10 +358,17 @@ __global__ void __launch_bounds__(256) feat_prep_kernel(const float* __restrict_
       const int m = m0 + 32 * i + lane;
       v[i] = m < M ? __ldg(y + m) : 0.f;
     }
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
+    auto take = [&](int i) {
       finite = finite && isfinite(v[i]);
       square_in(sq, v[i]);
+    };
+    if (m0 + 32 * R <= Mp) {
+#pragma unroll
+      for (int i = 0; i < R; ++i) take(i);
+    } else {  // no chain over zeros past the end of the row
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (m0 + 32 * i < Mp) take(i);
     }
     // written as if finite; a signal with a NaN or Inf is cleared below
     __nv_bfloat16* q = Yq + static_cast<size_t>(b) * Mp;

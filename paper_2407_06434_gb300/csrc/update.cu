@@ -42,15 +42,22 @@ __global__ void __launch_bounds__(256) init_kernel(Ws ws, const CallArgs* args, 
   constexpr int R = 16;  // loads in flight per lane
   SquareSum sq;
   bool finite = true;
-  for (int m0 = lane; m0 < ws.Mp; m0 += 32 * R) {
+  for (int m0 = 0; m0 < ws.Mp; m0 += 32 * R) {
     float v[R];
 #pragma unroll
-    for (int i = 0; i < R; ++i) v[i] = m0 + 32 * i < ws.M ? __ldg(y + m0 + 32 * i) : 0.f;
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
+    for (int i = 0; i < R; ++i) v[i] = m0 + 32 * i + lane < ws.M ? __ldg(y + m0 + 32 * i + lane) : 0.f;
+    auto take = [&](int i) {
       finite = finite && isfinite(v[i]);
-      if (m0 + 32 * i < ws.Mp) r[m0 + 32 * i] = v[i];
+      r[m0 + 32 * i + lane] = v[i];
       square_in(sq, v[i]);
+    };
+    if (m0 + 32 * R <= ws.Mp) {
+#pragma unroll
+      for (int i = 0; i < R; ++i) take(i);
+    } else {  // no chain over zeros past the end of the row
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+        if (m0 + 32 * i < ws.Mp) take(i);
     }
   }
   double s = warp_sum(total(sq));
